@@ -63,11 +63,17 @@ struct Store {
   uint64_t* k1 = nullptr;
   void* amp = nullptr;
   uint64_t cap = 0;
-  unsigned int* segs = nullptr;  // per-segment counts (cap >> kBucketLog2 + 1 entries)
+  unsigned int* segs = nullptr;  // per-segment counts (seg_entries(cap) of them)
+  // The bucket store: its counters lie 2^sqs::kBucketCntLog2 entries apart
+  // (the cluster merge's bins and the sort leave them packed or untouched).
+  bool buckets = false;
   bool segmented = false;
   uint32_t seg_log2 = 0;
   uint32_t n_seg = 0;
 
+  size_t seg_entries() const {
+    return ((size_t)(cap >> kBucketLog2) + 1) << (buckets ? sqs::kBucketCntLog2 : 0u);
+  }
   Arr view() const {
     Arr a;
     a.k0 = k0;
@@ -340,17 +346,18 @@ bool ensure_store(sqs_state* st, Store& s, uint64_t need) {
   }
   free_store(st, s);
   const uint64_t cap = round_cap(need);
-  const uint64_t nseg = (cap >> kBucketLog2) + 1;
+  s.buckets = &s == &st->bk;
+  s.cap = cap;
+  const size_t seg_bytes = s.seg_entries() * sizeof(unsigned int);
   s.k0 = (uint64_t*)dalloc(st, cap * 8);
   s.k1 = st->kw == 2 ? (uint64_t*)dalloc(st, cap * 8) : nullptr;
   s.amp = dalloc(st, cap * amp_bytes(st));
-  s.segs = (unsigned int*)dalloc(st, nseg * 4);
-  s.cap = cap;
+  s.segs = (unsigned int*)dalloc(st, seg_bytes);
   if (!s.k0 || (st->kw == 2 && !s.k1) || !s.amp || !s.segs) {
     free_store(st, s);
     return false;
   }
-  cudaMemsetAsync(s.segs, 0, nseg * 4, st->stream);
+  cudaMemsetAsync(s.segs, 0, seg_bytes, st->stream);
   return true;
 }
 
@@ -1818,7 +1825,7 @@ sqs_status run_lazy(sqs_state* st) {
     cudaMemsetAsync(&c->err, 0, sizeof(c->err) + sizeof(c->err_where), st->stream);
     cudaMemsetAsync(&c->need, 0, sizeof(c->need), st->stream);
     if (st->bk.segs)
-      cudaMemsetAsync(st->bk.segs, 0, ((st->bk.cap >> kBucketLog2) + 1) * 4, st->stream);
+      cudaMemsetAsync(st->bk.segs, 0, st->bk.seg_entries() * sizeof(unsigned int), st->stream);
     s = sync_ctl(st);  // exact input count of the failed step
     for (size_t i = f; i < n && s == SQS_OK; ++i) {
       st->pending = st->lazy[i].ops;
@@ -2276,7 +2283,7 @@ sqs_status sqs_state_reset(sqs_state* st) {
   st->ub = 1;
   history_reset(st, true);
   if (st->bk.segs)
-    cudaMemsetAsync(st->bk.segs, 0, ((st->bk.cap >> kBucketLog2) + 1) * 4, st->stream);
+    cudaMemsetAsync(st->bk.segs, 0, st->bk.seg_entries() * sizeof(unsigned int), st->stream);
   st->cur.set_dense();
   st->call = 1;  // API calls are numbered from the reset
   Traced tr(st, SQS_K_INIT);

@@ -189,7 +189,18 @@ cudaError_t launch_apply_compact(const Launch& L, int kw, bool amp32, Ctl* ctl, 
 // bk.n_seg buckets of 2^bk.seg_log2 slots, counters zero on entry.
 // Buckets follow the device count: ceil(count / fill_target) of them, at
 // most bk.n_seg (the host's bound; fill_target 0 keeps bk.n_seg); the pair
-// kernel leaves the others empty.
+// kernel leaves the others empty.  Bucket b's counter is
+// bk.seg_cnt[b << kBucketCntLog2].
+//
+// Bucket counters lie one 128-byte L2 line apart.  Packed, the counters of a
+// state of up to a million branches fill a few lines of one or two L2
+// slices, and every branch's atomic queues there: on a 64-system walk batch
+// (0.5M branches, 500 buckets) ncu showed the busiest slice at 81 % of its
+// tag rate with the average at 10 %, and the partition took 75 us; spread
+// it takes 30 us (stride 8 counters: 40 us; 128 or more: as 32).  At 2^23
+// branches 178 -> 118 us; from about 2^24 the counters fill all slices
+// either way.
+constexpr uint32_t kBucketCntLog2 = 5;
 cudaError_t launch_partition(const Launch& L, int kw, bool amp32, Ctl* ctl, Arr in, int in_slot,
                              const OpList& ops, const Gate1& g, Arr bk, uint32_t fill_target);
 

@@ -258,7 +258,7 @@ __global__ void __launch_bounds__(kStreamThreads)
       if (live[q]) {
         const uint64_t h = khash(k[q] & ~bmask);
         bkt[q] = (uint32_t)(((h >> 32) * (uint64_t)n_buckets) >> 32);
-        pos[q] = atomicAdd(&bk.seg_cnt[bkt[q]], 1u);
+        pos[q] = atomicAdd(&bk.seg_cnt[(uint64_t)bkt[q] << kBucketCntLog2], 1u);
       }
     }
 #pragma unroll
@@ -312,7 +312,8 @@ __global__ void __launch_bounds__(kPairThreads, 3)
   for (uint32_t b = next_b; b < nb; b = next_b) {
     uint32_t drawn = 0u;
     if (threadIdx.x == 0) drawn = atomicAdd(&ctl->pair_next, 1u);
-    const uint32_t n = bk.seg_cnt[b];
+    unsigned int* const bcnt = &bk.seg_cnt[(uint64_t)b << kBucketCntLog2];
+    const uint32_t n = *bcnt;
     if (n > C) {  // overflow already flagged by the partition
       __syncthreads();  // every thread has read next_b
       if (threadIdx.x == 0) next_b = drawn;
@@ -329,7 +330,7 @@ __global__ void __launch_bounds__(kPairThreads, 3)
     for (uint32_t i = threadIdx.x; i < S; i += blockDim.x) slot[i] = 0u;
     if (threadIdx.x == 0) fill = 0;
     __syncthreads();
-    if (threadIdx.x == 0) bk.seg_cnt[b] = 0u;  // bucket is clean for the next use
+    if (threadIdx.x == 0) *bcnt = 0u;  // bucket is clean for the next use
 
     const K bmask = bit_mask<KW>(g.t);
     const K cmask = mk<KW>(g.cmask[0], g.cmask[1]);

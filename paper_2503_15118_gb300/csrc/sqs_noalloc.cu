@@ -36,7 +36,7 @@ constexpr size_t kBkK1Off = align256(kBkK0Off + kBkSlots * 8);
 constexpr size_t kBkAmpOff = align256(kBkK1Off + kBkSlots * 8);
 constexpr size_t kBkCntOff = align256(kBkAmpOff + kBkSlots * 16);
 constexpr size_t kOutSlots = kMaxB << kSegLog2;
-constexpr size_t kOutK0Off = align256(kBkCntOff + kMaxB * 4);
+constexpr size_t kOutK0Off = align256(kBkCntOff + (kMaxB << sqs::kBucketCntLog2) * 4);
 constexpr size_t kOutK1Off = align256(kOutK0Off + kOutSlots * 8);
 constexpr size_t kOutAmpOff = align256(kOutK1Off + kOutSlots * 8);
 constexpr size_t kOutCntOff = align256(kOutAmpOff + kOutSlots * 16);
@@ -65,7 +65,7 @@ sqs_status say(sqs_status s, const char* msg) {
 __global__ void k_noalloc_begin(Ctl* ctl, unsigned int* bucket_cnt, unsigned int* seg_cnt,
                                 uint32_t B, uint64_t n_in) {
   for (uint32_t i = threadIdx.x; i < B; i += blockDim.x) {
-    bucket_cnt[i] = 0u;
+    bucket_cnt[i << sqs::kBucketCntLog2] = 0u;
     seg_cnt[i] = 0u;
   }
   if (threadIdx.x == 0) {
