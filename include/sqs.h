@@ -502,7 +502,9 @@ void sqs_graph_destroy(sqs_graph* g);
 typedef struct {
   uint64_t host_waits;       /* times the host read the device counts         */
   uint64_t overflow_reruns;  /* learned-mode steps re-run at the exact size    */
-  uint64_t learned_steps;    /* steps sized from a prediction                  */
+  uint64_t learned_steps;    /* steps queued for learned sizing (sized from a
+                                prediction, or from the hard bound while that is
+                                small)                                          */
   uint64_t bytes_live;       /* device bytes currently held by the state       */
   uint64_t bytes_peak;       /* largest bytes_live since creation              */
   uint64_t steps_expand;     /* interference steps by path: constant target   */

@@ -37,6 +37,8 @@ struct sqs_table {
   void* dev;
   uint64_t n;
   uint32_t bytes;
+  // Address bits some entry depends on (entries past the end read 0).
+  uint64_t varies = 0;
 };
 
 namespace {
@@ -111,7 +113,7 @@ struct HostSnap {
   std::vector<int64_t> last_branch;
   std::vector<uint32_t> writes_since, reads_since;
   std::vector<uint8_t> arith_since;
-  std::vector<int8_t> const_val, pair_sign;
+  std::vector<int8_t> const_val, known_val, pair_sign;
   int64_t n_branch = 0, last_target = -1;
 };
 
@@ -120,6 +122,9 @@ struct HostSnap {
 struct HostOp {
   DevOp d;
   std::complex<double> c0, c1;
+  // OP_QRAM: the table's address bits that matter, and which bits of the data
+  // field were known constant before the operation (mask, values).
+  uint64_t varies = 0, was_const = 0, was_value = 0;
 };
 
 }  // namespace
@@ -148,6 +153,7 @@ struct sqs_state {
 
   std::vector<HostOp> pending;
   OpList ops_buf;   // staging for one launch's fused operations
+  sqs::RunProg run_prog;  // staging for one addressed run
   uint64_t ub = 1;  // upper bound of the current branch count
   uint32_t seq = 0;
   uint64_t launches = 0;
@@ -165,7 +171,10 @@ struct sqs_state {
   std::vector<int64_t> last_branch;  // index of the last interference step on the bit, -1: none
   std::vector<uint32_t> writes_since, reads_since;  // operations since that step
   std::vector<uint8_t> arith_since;  // the bit's register was an arithmetic destination since
-  std::vector<int8_t> const_val;     // value when the bit is known constant, else -1
+  // Value of the bit when known constant, else -1: const_val by the rules the
+  // predictor's features were defined with, known_val (everything else) also
+  // through arithmetic on known fields and loads that are undone.
+  std::vector<int8_t> const_val, known_val;
   // +1 / -1 when every branch's partner across the bit is known to exist with
   // exactly +1 / -1 times its amplitude (set by an uncontrolled expansion with
   // U[1][b] = +-U[0][b], kept while nothing reads or writes the bit), else 0.
@@ -240,10 +249,22 @@ struct sqs_state {
 
   // Fused run (exact sizing): interference steps on distinct targets issued
   // back to back with nothing queued between them, held until the run ends.
-  std::vector<Gate1> run_gates;
+  struct Held {
+    Gate1 g;
+    bool after_phase;  // `phase` (one queued phase) comes between the last step and this one
+    HostOp phase;
+  };
+  std::vector<Held> run;
   std::vector<HostOp> run_pre;       // operations queued before the run's first step
   uint64_t run_tmask[2] = {0, 0};    // the run's target bits
-  uint64_t run_reads[2] = {0, 0};    // control and angle bits its steps read
+  uint64_t run_reads[2] = {0, 0};    // control, angle and table address bits its steps read
+  uint32_t run_items = 0;            // steps and phases held
+  bool run_sorted_form = true;       // distinct targets that no step reads, no phase, no fold
+  // Slots of addressed runs (sqs_run.cu): amplitudes, and presence bytes that
+  // are zero between runs.
+  void* slot_amp = nullptr;
+  uint8_t* slot_pres = nullptr;
+  uint64_t slot_cap = 0;
 
   // CUDA-graph capture (sqs_capture_begin / _end): while capturing, nothing
   // may wait for the device or allocate, and the branch-count bound is held
@@ -253,6 +274,9 @@ struct sqs_state {
   sqs_status capture_err = SQS_OK;
   HostSnap entry_snap;
   uint64_t launches_at_capture = 0;
+  // A graph was captured: it holds the buffers, which eager issue then leaves
+  // where they are as long as the count allows.
+  bool captured = false;
 
   sqs_stats stats{};
   std::unordered_map<void*, size_t> sizes;
@@ -363,6 +387,25 @@ bool ensure_store(sqs_state* st, Store& s, uint64_t need) {
 
 uint64_t max_branches(const sqs_state* st) {
   return st->total_bits >= 62 ? (1ull << 62) : (1ull << st->total_bits);
+}
+
+// Bounds up to this many branches are allocated for without reading the exact
+// count first: a few MB against a host wait per step.  None after a graph
+// capture, whose buffers eager issue leaves in place while the count allows,
+// nor under the measured merge choice, whose timings complete as it waits.
+uint64_t small_bound(const sqs_state* st) {
+  return st->captured || (st->flags & SQS_MERGE_TUNED) ? 1ull : 1ull << 16;
+}
+
+// Branches a state can hold once step g has run: one per setting of the key
+// bits not known constant (of all bits under SQS_MERGE_PLAIN, which uses
+// nothing the host proves).
+uint64_t vary_cap(const sqs_state* st, const Gate1& g) {
+  if (st->flags & SQS_MERGE_PLAIN) return max_branches(st);
+  uint64_t v[2] = {g.vary[0], g.vary[1]};
+  v[g.t >> 6] |= 1ull << (g.t & 63);
+  const int bits = __builtin_popcountll(v[0]) + __builtin_popcountll(v[1]);
+  return std::min<uint64_t>(max_branches(st), 1ull << std::min(bits, 62));
 }
 
 // The count bound after an operation: v, held at the static bound while a
@@ -583,8 +626,17 @@ sqs_status run_list(sqs_state* st, const OpList& L) {
 // follows to fuse; otherwise everything runs.
 sqs_status flush_run(sqs_state* st);
 
+// Forgets the held run (its bookkeeping; not the operations queued after it).
+void drop_run(sqs_state* st) {
+  st->run.clear();
+  st->run_pre.clear();
+  st->run_tmask[0] = st->run_tmask[1] = st->run_reads[0] = st->run_reads[1] = 0;
+  st->run_items = 0;
+  st->run_sorted_form = true;
+}
+
 sqs_status run_pending(sqs_state* st, bool keep_tail) {
-  if (!st->run_gates.empty()) {
+  if (!st->run.empty()) {
     sqs_status s = flush_run(st);  // the held run precedes everything queued
     if (s != SQS_OK) return s;
   }
@@ -619,10 +671,10 @@ sqs_status run_expand(sqs_state* st, const Gate1& g, int64_t rec_idx) {
   // Output bound: an expansion at most doubles the branches, a fold keeps
   // their number (each pair's two members become its two children).
   auto out_bound = [&] {
-    return g.fold_sign ? st->ub : std::min(max_branches(st), 2 * st->ub);
+    return g.fold_sign ? st->ub : std::min(vary_cap(st, g), 2 * st->ub);
   };
   uint64_t need = std::max<uint64_t>(bound_after(st, out_bound()), 1);
-  if (need > st->alt.cap && st->ub > 1) {
+  if (need > st->alt.cap && st->ub > small_bound(st)) {
     sqs_status s = sync_bound(st);  // the bound outgrew the allocation: exact count
     if (s != SQS_OK) return s;
     need = std::max<uint64_t>(bound_after(st, out_bound()), 1);
@@ -700,7 +752,7 @@ sqs_status run_binned(sqs_state* st, const Gate1& g, uint64_t B1, int64_t rec_id
   }
   std::swap(st->cur, st->alt);
   st->cur_slot = out_slot;
-  st->ub = bound_after(st, std::min(max_branches(st), 2 * st->ub));
+  st->ub = bound_after(st, std::min(vary_cap(st, g), 2 * st->ub));
   return SQS_OK;
 }
 
@@ -731,7 +783,7 @@ sqs_status run_hashed(sqs_state* st, const Gate1& g, double est_in, int64_t rec_
   };
   uint64_t B, B1;
   uint64_t need = plan(want, B, B1);
-  if (need > st->alt.cap && st->ub > 1) {
+  if (need > st->alt.cap && st->ub > small_bound(st)) {
     // The bound (exact mode) or the estimate (learned mode) outgrew the
     // allocation: learn the exact count first.
     s = est_in < 0 ? sync_ctl(st) : sync_bound(st);
@@ -780,7 +832,7 @@ sqs_status run_hashed(sqs_state* st, const Gate1& g, double est_in, int64_t rec_
   }
   std::swap(st->cur, st->alt);
   st->cur_slot = out_slot;
-  st->ub = bound_after(st, std::min(max_branches(st), 2 * st->ub));
+  st->ub = bound_after(st, std::min(vary_cap(st, g), 2 * st->ub));
   return SQS_OK;
 }
 
@@ -832,7 +884,7 @@ sqs_status sort_scratch(sqs_state* st, uint64_t tiles, unsigned int*& hist, unsi
 uint32_t bits_to_sort(const sqs_state* st, const uint64_t keep[2]) {
   uint32_t n = 0;
   for (uint32_t q = 0; q < st->total_bits; ++q)
-    if (((keep[q >> 6] >> (q & 63)) & 1ull) && st->const_val[q] < 0) ++n;
+    if (((keep[q >> 6] >> (q & 63)) & 1ull) && st->known_val[q] < 0) ++n;
   return n;
 }
 
@@ -1094,7 +1146,7 @@ sqs_status run_sorted(sqs_state* st, const Gate1& g, int64_t rec_idx) {
   }
   std::swap(st->cur, st->alt);
   st->cur_slot = out_slot;
-  st->ub = bound_after(st, std::min(max_branches(st), 2 * st->ub));
+  st->ub = bound_after(st, std::min(vary_cap(st, g), 2 * st->ub));
   return SQS_OK;
 }
 
@@ -1145,7 +1197,7 @@ sqs_status run_branching(sqs_state* st, const Gate1& g, double est_in = -1.0,
                          int64_t rec_idx = -1) {
   TraceCall attribution(st, g.issue_call);
   sqs_status s = SQS_OK;
-  if (g.defer_ops && st->run_gates.empty()) {
+  if (g.defer_ops && st->run.empty()) {
     // The queued operations stay queued past this step (defer_ops_ok).
     st->ops_buf.n = 0;
     st->ops_buf.n_tab = 0;
@@ -1351,22 +1403,233 @@ bool fuse_pays(const sqs_state* st, const std::vector<Gate1>& gates) {
   return fused < alone;
 }
 
-// Executes the held run: alone (the per-step dispatch with its shortcuts) or
-// fused.  Operations queued after the run stay queued after it.
+// ---- addressed runs (sqs_run.cu) --------------------------------------------
+// Key bits that vary over the state while the run executes: those not known
+// constant at its last step, and its targets.
+void run_vary(const Gate1& last, const uint64_t tmask[2], uint64_t v[2]) {
+  for (int w = 0; w < 2; ++w) v[w] = last.vary[w] | tmask[w];
+  v[last.t >> 6] |= 1ull << (last.t & 63);
+}
+int bits_set(const uint64_t m[2]) {
+  return __builtin_popcountll(m[0]) + __builtin_popcountll(m[1]);
+}
+
+// Whether the held run pays as an addressed run against its steps one by one.
+// Below a few million branches either way is a matter of launches: a step
+// alone costs one (expansion, fold) or two (partition and pair) of about 5 us
+// each, an addressed run two and a few block-wide barriers per step; above,
+// of the slots visited against the branches streamed.
+bool slots_pay(const sqs_state* st, const std::vector<sqs_state::Held>& run, int slot_bits) {
+  if (st->flags & SQS_FUSE_ALWAYS) return true;
+  const double slots = std::ldexp(1.0, slot_bits);
+  // The bound is often the number of slots, far above the count.
+  const double n = std::min((double)st->ub, slots / 8);
+  double alone = 0.0, fused = 12.0 + slots * 3e-6;
+  for (const auto& h : run) {
+    const double launches = h.g.no_partners || h.g.fold_sign ? 1.0 : 2.0;
+    alone += launches * (4.0 + n * 3e-5);
+    fused += 1.2 + slots * 5e-7;
+  }
+  return fused < alone;
+}
+
+// The held run (k targets) by direct addressing: the queued operations and
+// the scatter of every branch to its slot, then every group transformed in
+// shared memory.  No host wait: the output holds at most one branch per slot,
+// or 2^k per input branch.
+sqs_status run_slots(sqs_state* st, const std::vector<sqs_state::Held>& run,
+                     const uint64_t tmask[2]) {
+  TraceCall attribution(st, run[0].g.issue_call);
+  sqs_status s = run_pending(st, true);  // leaves the fused operations in ops_buf
+  if (s != SQS_OK) return st->sticky = s;
+  const Gate1& last = run.back().g;
+  uint64_t vary[2];
+  run_vary(last, tmask, vary);
+  const uint32_t bits = (uint32_t)bits_set(vary), k = (uint32_t)bits_set(tmask);
+  const uint64_t slots = 1ull << bits;
+
+  // Slot layout: the targets in key order in the low k bits, then the others.
+  sqs::SlotMap map;
+  std::memset(&map, 0, sizeof(map));
+  uint8_t at[128];  // slot bit of each varying key bit
+  uint32_t pos = 0;
+  for (int pass = 0; pass < 2; ++pass)
+    for (uint32_t q = 0; q < st->total_bits; ++q) {
+      const bool v = (vary[q >> 6] >> (q & 63)) & 1ull, t = (tmask[q >> 6] >> (q & 63)) & 1ull;
+      if (!v || t != (pass == 0)) continue;
+      at[q] = (uint8_t)pos;
+      sqs::BitMove* m = map.n ? &map.mv[map.n - 1] : nullptr;
+      if (m && m->src + m->len == q && m->dst + m->len == pos && (q & 63))
+        m->len++;
+      else
+        map.mv[map.n++] = sqs::BitMove{(uint8_t)q, (uint8_t)pos, 1, 0};
+      ++pos;
+    }
+  for (int w = 0; w < 2; ++w) map.base[w] = last.fixed[w] & ~vary[w];
+  // A predicate over the key as one over the slot; false when a constant bit
+  // fails it.
+  auto slot_pred = [&](const uint64_t pm[2], const uint64_t pv[2], sqs::RunItem& it) {
+    it.smask = it.sval = 0;
+    for (uint32_t q = 0; q < st->total_bits; ++q) {
+      if (!((pm[q >> 6] >> (q & 63)) & 1ull)) continue;
+      const uint32_t want = (uint32_t)((pv[q >> 6] >> (q & 63)) & 1ull);
+      if ((vary[q >> 6] >> (q & 63)) & 1ull) {
+        it.smask |= 1u << at[q];
+        it.sval |= want << at[q];
+      } else if (((map.base[q >> 6] >> (q & 63)) & 1ull) != want) {
+        return false;
+      }
+    }
+    return true;
+  };
+  sqs::RunProg& prog = st->run_prog;
+  prog.n = 0;
+  for (const auto& h : run) {
+    if (h.after_phase) {
+      sqs::RunItem& it = prog.it[prog.n];
+      std::memset(&it, 0, sizeof(it));
+      if (slot_pred(h.phase.d.pmask, h.phase.d.pval, it)) {
+        it.phase = 1;
+        it.g.u[0] = h.phase.c0.real();
+        it.g.u[1] = h.phase.c0.imag();
+        ++prog.n;
+      }
+    }
+    sqs::RunItem& it = prog.it[prog.n];
+    it.phase = 0;
+    it.j = at[h.g.t];
+    it.g = h.g;
+    if (slot_pred(h.g.cmask, h.g.cval, it)) ++prog.n;  // else it acts on no branch
+  }
+  prog.area_log2 = sqs::run_area_log2(k);
+  prog.n_areas = bits > prog.area_log2 ? 1u << (bits - prog.area_log2) : 1u;
+  const uint64_t want = (uint64_t)prog.n_areas << prog.area_log2;
+  if (st->slot_cap < want) {
+    dfree(st, st->slot_amp);
+    dfree(st, st->slot_pres);
+    st->slot_amp = dalloc(st, want * amp_bytes(st));
+    st->slot_pres = (uint8_t*)dalloc(st, want);
+    st->slot_cap = st->slot_amp && st->slot_pres ? want : 0;
+    if (!st->slot_cap) {
+      dfree(st, st->slot_amp);
+      dfree(st, st->slot_pres);
+      st->slot_amp = st->slot_pres = nullptr;
+      return st->sticky = fail(st, SQS_ERR_OOM, "cannot allocate %llu slots",
+                               (unsigned long long)want);
+    }
+    cudaMemsetAsync(st->slot_pres, 0, want, st->stream);
+  }
+  const uint64_t grown = st->ub > (slots >> k) ? slots : st->ub << k;
+  if (st->alt.cap < grown && !ensure_store(st, st->alt, grown))
+    return st->sticky = fail(st, SQS_ERR_OOM, "cannot allocate %llu branches",
+                             (unsigned long long)grown);
+  st->alt.set_dense();
+  const uint64_t in_slots = st->cur.slots(st->ub);
+  const int out_slot = (st->cur_slot + 1) & 3;
+  cudaError_t e;
+  {
+    Traced tr(st, SQS_K_PARTITION);
+    e = sqs::launch_slot_scatter(launch_of(st, in_slots), st->kw, st->amp32, st->ctl,
+                                 st->cur.view(), st->cur_slot, st->ops_buf, map, st->slot_amp,
+                                 st->slot_pres);
+  }
+  if (e != cudaSuccess) return cuda_fail(st, e, "slot scatter launch");
+  {
+    Traced tr(st, SQS_K_GROUP);
+    e = sqs::launch_slot_run(launch_of(st, slots), st->kw, st->amp32, st->ctl, st->slot_amp,
+                             st->slot_pres, map, prog, st->alt.view(), out_slot);
+  }
+  if (e != cudaSuccess) return cuda_fail(st, e, "slot run launch");
+  std::swap(st->cur, st->alt);
+  st->cur_slot = out_slot;
+  st->ub = grown;
+  st->stats.runs_fused++;
+  st->stats.steps_fused += run.size();
+  return SQS_OK;
+}
+
+// Reads of a step besides its target: controls, angle bits, and the table
+// address bits that some entry depends on.
+void step_reads(const Gate1& g, uint64_t reads[2]) {
+  reads[0] = g.cmask[0];
+  reads[1] = g.cmask[1];
+  auto add = [&](uint32_t q) {
+    if (q < 128) reads[q >> 6] |= 1ull << (q & 63);
+  };
+  if (g.mode == 1)
+    for (uint32_t b = 0; b < g.ang_w; ++b) add(g.ang_off + b);
+  if (g.atab)
+    for (uint32_t b = 0; b < g.atab_w; ++b)
+      if ((g.atab_varies >> b) & 1ull) add(g.atab_off + b);
+}
+
+// A run of steps with nothing between them, in the sorted form's terms:
+// fused when that pays, else one by one.
+sqs_status run_steps(sqs_state* st, const std::vector<Gate1>& gates) {
+  if (gates.size() >= 2 && fuse_pays(st, gates)) return run_group(st, gates);
+  sqs_status s = SQS_OK;
+  for (size_t j = 0; j < gates.size() && s == SQS_OK; ++j)
+    s = run_branching(st, gates[j]);  // the queued operations go with the first
+  return s;
+}
+
+// Executes the held run: by direct addressing where few bits vary, else in
+// pieces the sorted form allows (distinct targets that no other step of the
+// piece reads), each fused or step by step.  Operations queued after the run
+// stay queued after it.
 sqs_status flush_run(sqs_state* st) {
-  if (st->run_gates.empty()) return SQS_OK;
-  std::vector<Gate1> gates;
-  gates.swap(st->run_gates);
+  if (st->run.empty()) return SQS_OK;
+  std::vector<sqs_state::Held> run;
+  run.swap(st->run);
   std::vector<HostOp> after;
   after.swap(st->pending);
   st->pending.swap(st->run_pre);
-  st->run_tmask[0] = st->run_tmask[1] = st->run_reads[0] = st->run_reads[1] = 0;
+  const uint64_t tmask[2] = {st->run_tmask[0], st->run_tmask[1]};
+  drop_run(st);
   sqs_status s = SQS_OK;
-  if (gates.size() >= 2 && fuse_pays(st, gates)) {
-    s = run_group(st, gates);
+  uint64_t vary[2];
+  run_vary(run.back().g, tmask, vary);
+  const int slot_bits = bits_set(vary);
+  bool addressed = run.size() >= 2 && slot_bits <= (int)sqs::kMaxSlotBits &&
+                   slots_pay(st, run, slot_bits);
+  if (addressed && st->captured) {
+    // The output must fit where the graph expects it (run_slots would move it).
+    const uint64_t k = (uint64_t)bits_set(tmask);
+    auto fits = [&] {
+      return std::min<double>(std::ldexp((double)st->ub, (int)k), std::ldexp(1.0, slot_bits)) <=
+             (double)st->alt.cap;
+    };
+    if (!fits()) s = sync_bound(st);
+    addressed = s == SQS_OK && fits();
+  }
+  if (s != SQS_OK) {
+  } else if (addressed) {
+    s = run_slots(st, run, tmask);
   } else {
-    for (size_t j = 0; j < gates.size() && s == SQS_OK; ++j)
-      s = run_branching(st, gates[j]);  // the queued operations go with the first
+    std::vector<Gate1> part;
+    uint64_t pt[2] = {0, 0}, pr[2] = {0, 0};
+    for (size_t i = 0; i < run.size() && s == SQS_OK; ++i) {
+      const Gate1& g = run[i].g;
+      uint64_t reads[2], t[2] = {0, 0};
+      step_reads(g, reads);
+      t[g.t >> 6] = 1ull << (g.t & 63);
+      const bool joins = !part.empty() && !run[i].after_phase && !g.fold_sign &&
+                         !part.back().fold_sign && !((pt[0] | pr[0]) & t[0]) &&
+                         !((pt[1] | pr[1]) & t[1]) && !(reads[0] & pt[0]) && !(reads[1] & pt[1]);
+      if (!joins) {
+        s = run_steps(st, part);
+        if (s != SQS_OK) break;
+        part.clear();
+        pt[0] = pt[1] = pr[0] = pr[1] = 0;
+        if (run[i].after_phase) st->pending.push_back(run[i].phase);
+      }
+      part.push_back(g);
+      for (int w = 0; w < 2; ++w) {
+        pt[w] |= t[w];
+        pr[w] |= reads[w];
+      }
+    }
+    if (s == SQS_OK) s = run_steps(st, part);
   }
   if (st->pending.empty()) st->pending.swap(after);
   else st->pending.insert(st->pending.end(), after.begin(), after.end());
@@ -1382,33 +1645,57 @@ bool fusing(const sqs_state* st) {
 }
 
 // Holds an interference step in the open run, or closes the run and opens a
-// new one with it.  A step joins when nothing was queued since the run's
-// last step, its target is new to the run and read by no step of it, and it
-// reads (controls, angle register) none of the run's targets nor its own.
-// A copy-pair fold always runs alone: one pass with no partition is cheaper
-// than its share of a fused run.
+// new one with it.  A step joins when nothing was queued since the run's last
+// step, its target is new to the run and read by no step of it, and it reads
+// (controls, angle register, table address) none of the run's targets: the
+// sorted form.  While few enough key bits vary for an addressed run, a step on
+// any target joins, whatever it reads, one phase may lie between two steps,
+// and so may a copy-pair fold, which opens no run: alone it is one pass.
 sqs_status hold_step(sqs_state* st, const Gate1& g) {
-  uint64_t reads[2] = {g.cmask[0], g.cmask[1]};
-  if (g.mode == 1)
-    for (uint32_t b = 0; b < g.ang_w; ++b) {
-      const uint32_t q = g.ang_off + b;
-      if (q < 128) reads[q >> 6] |= 1ull << (q & 63);
-    }
+  uint64_t reads[2];
+  step_reads(g, reads);
   uint64_t tbit[2] = {0, 0};
   tbit[g.t >> 6] = 1ull << (g.t & 63);
-  const bool alone = (reads[0] & tbit[0]) || (reads[1] & tbit[1]) || g.fold_sign != 0;
-  const bool join = !st->run_gates.empty() && st->pending.empty() && !alone &&
-                    st->run_gates.size() < (size_t)sqs::kMaxRun &&
-                    !((st->run_tmask[0] | st->run_reads[0]) & tbit[0]) &&
-                    !((st->run_tmask[1] | st->run_reads[1]) & tbit[1]) &&
-                    !(reads[0] & st->run_tmask[0]) && !(reads[1] & st->run_tmask[1]);
+  const bool own = (reads[0] & tbit[0]) || (reads[1] & tbit[1]);
+  uint64_t targets[2] = {st->run_tmask[0] | tbit[0], st->run_tmask[1] | tbit[1]};
+  bool join = false, sorted_form = false, phase = false;
+  if (!st->run.empty() && !own) {
+    phase = st->pending.size() == 1 && st->pending[0].d.kind == sqs::OP_MUL &&
+            st->pending[0].d.sel_bit >= 128 && !g.defer_ops;
+    sorted_form = st->run_sorted_form && !phase && !g.fold_sign &&
+                  !((st->run_tmask[0] | st->run_reads[0]) & tbit[0]) &&
+                  !((st->run_tmask[1] | st->run_reads[1]) & tbit[1]) &&
+                  !(reads[0] & st->run_tmask[0]) && !(reads[1] & st->run_tmask[1]);
+    uint64_t vary[2];
+    run_vary(g, targets, vary);
+    const int bits = bits_set(vary);
+    const bool slots = bits <= (int)sqs::kMaxSlotBits;
+    // An addressed run leaves at least 256 groups when the state has them: a
+    // group is one CTA's, and with fewer the SMs idle (18 varying bits: 10
+    // targets a run 27 us, 12 targets 44 us).
+    const int most = slots && !(st->flags & SQS_FUSE_ALWAYS)
+                         ? std::max(9, std::min(sqs::kMaxRun, bits - 8))
+                         : sqs::kMaxRun;
+    join = bits_set(targets) <= most && (sorted_form || slots) &&
+           (st->pending.empty() || phase) &&
+           st->run_items + 1u + (phase ? 1u : 0u) <= (uint32_t)sqs::kMaxItems;
+  }
   if (!join) {
     sqs_status s = flush_run(st);
     if (s != SQS_OK) return s;
-    if (alone) return run_branching(st, g);
+    if (own || g.fold_sign != 0) return run_branching(st, g);
     st->run_pre.swap(st->pending);
   }
-  st->run_gates.push_back(g);
+  sqs_state::Held h;
+  h.g = g;
+  h.after_phase = join && phase;
+  if (h.after_phase) {
+    h.phase = st->pending[0];
+    st->pending.clear();
+  }
+  st->run_items += h.after_phase ? 2u : 1u;
+  if (join) st->run_sorted_form = sorted_form;
+  st->run.push_back(h);
   for (int w = 0; w < 2; ++w) {
     st->run_tmask[w] |= tbit[w];
     st->run_reads[w] |= reads[w];
@@ -1426,6 +1713,7 @@ void history_reset(sqs_state* st, bool known_zero) {
   st->reads_since.assign(n, 0);
   st->arith_since.assign(n, 0);
   st->const_val.assign(n, known_zero ? 0 : -1);
+  st->known_val.assign(n, known_zero ? 0 : -1);
   st->pair_sign.assign(n, 0);
   st->n_branch = 0;
   st->last_target = -1;
@@ -1439,13 +1727,14 @@ void for_bits(const uint64_t m[2], uint32_t nbits, F f) {
 
 // Every predicate bit known constant and equal to the required value?
 // 1: always holds, 0: never holds, -1: unknown.
-int predicate_known(const sqs_state* st, const uint64_t pm[2], const uint64_t pv[2]) {
+int predicate_known(const sqs_state* st, const std::vector<int8_t>& val, const uint64_t pm[2],
+                    const uint64_t pv[2]) {
   int res = 1;
   for (uint32_t q = 0; q < st->total_bits; ++q) {
     if (!((pm[q >> 6] >> (q & 63)) & 1ull)) continue;
     const int want = (int)((pv[q >> 6] >> (q & 63)) & 1ull);
-    if (st->const_val[q] < 0) res = res == 0 ? 0 : -1;
-    else if (st->const_val[q] != want) res = 0;
+    if (val[q] < 0) res = res == 0 ? 0 : -1;
+    else if (val[q] != want) res = 0;
   }
   return res;
 }
@@ -1453,9 +1742,23 @@ int predicate_known(const sqs_state* st, const uint64_t pm[2], const uint64_t pv
 void note_field_write(sqs_state* st, uint32_t off, uint32_t w, bool arith) {
   for (uint32_t b = 0; b < w; ++b) {
     st->writes_since[off + b]++;
-    st->const_val[off + b] = -1;
+    st->const_val[off + b] = st->known_val[off + b] = -1;
     if (arith) st->arith_since[off + b] = 1;
   }
+}
+
+// The value of a field whose every bit is known constant (a counter register
+// that steps add to stays known), and setting one.
+bool field_known(const sqs_state* st, uint32_t off, uint32_t w, uint64_t& v) {
+  v = 0;
+  for (uint32_t b = 0; b < w; ++b) {
+    if (st->known_val[off + b] < 0) return false;
+    v |= (uint64_t)st->known_val[off + b] << b;
+  }
+  return true;
+}
+void set_field_known(sqs_state* st, uint32_t off, uint32_t w, uint64_t v) {
+  for (uint32_t b = 0; b < w; ++b) st->known_val[off + b] = (int8_t)((v >> b) & 1ull);
 }
 
 void note_field_read(sqs_state* st, uint32_t off, uint32_t w) {
@@ -1507,26 +1810,41 @@ void note_op(sqs_state* st, const HostOp& h) {
   switch (d.kind) {
     case sqs::OP_XOR:
     case sqs::OP_MUL_XOR: {
-      const int known = predicate_known(st, d.pmask, d.pval);
-      for_bits(d.xmask, st->total_bits, [&](uint32_t q) {
-        st->writes_since[q]++;
-        if (st->const_val[q] >= 0) {
-          if (known == 1) st->const_val[q] ^= 1;
-          else if (known < 0) st->const_val[q] = -1;
-        }
-      });
+      for (std::vector<int8_t>* val : {&st->const_val, &st->known_val}) {
+        const int known = predicate_known(st, *val, d.pmask, d.pval);
+        for_bits(d.xmask, st->total_bits, [&](uint32_t q) {
+          if ((*val)[q] < 0) return;
+          if (known == 1) (*val)[q] ^= 1;
+          else if (known < 0) (*val)[q] = -1;
+        });
+      }
+      for_bits(d.xmask, st->total_bits, [&](uint32_t q) { st->writes_since[q]++; });
       if (d.kind == sqs::OP_MUL_XOR && d.sel_bit < 128) st->reads_since[d.sel_bit]++;
       break;
     }
     case sqs::OP_ADD_REG:
-    case sqs::OP_SUB_REG:
+    case sqs::OP_SUB_REG: {
+      uint64_t dst, src;
+      const bool known = predicate_known(st, st->known_val, d.pmask, d.pval) == 1 &&
+                         field_known(st, d.dst_off, d.dst_w, dst) &&
+                         field_known(st, d.src_off, d.src_w, src);
       note_field_read(st, d.src_off, d.src_w);
       note_field_write(st, d.dst_off, d.dst_w, true);
+      if (known)
+        set_field_known(st, d.dst_off, d.dst_w, d.kind == sqs::OP_ADD_REG ? dst + src : dst - src);
       break;
+    }
     case sqs::OP_ADD_CONST:
-    case sqs::OP_MUL_CONST:
+    case sqs::OP_MUL_CONST: {
+      uint64_t dst;
+      const bool known = predicate_known(st, st->known_val, d.pmask, d.pval) == 1 &&
+                         field_known(st, d.dst_off, d.dst_w, dst);
       note_field_write(st, d.dst_off, d.dst_w, true);
+      if (known)
+        set_field_known(st, d.dst_off, d.dst_w,
+                        d.kind == sqs::OP_ADD_CONST ? dst + d.constant : dst * d.constant);
       break;
+    }
     case sqs::OP_MUL_ADD:
     case sqs::OP_DIV_XOR:
       note_field_read(st, d.src_off, d.src_w);
@@ -1551,6 +1869,10 @@ void note_op(sqs_state* st, const HostOp& h) {
 
 void push_op(sqs_state* st, const HostOp& h) {
   note_op(st, h);
+  // An operation that no step can join the held run across ends it now.  A
+  // phase may lie between two steps, and a load may commute with the next.
+  const bool between = (h.d.kind == sqs::OP_MUL && h.d.sel_bit >= 128) || h.d.kind == sqs::OP_QRAM;
+  if (!st->run.empty() && !between) flush_run(st);  // an error is sticky: the next call returns it
   st->pending.push_back(h);
 }
 
@@ -1590,11 +1912,13 @@ void note_branch(sqs_state* st, const Gate1& g) {
   if (g.mode == 1)
     for (uint32_t b = 0; b < g.ang_w; ++b)
       if (g.ang_off + b < st->total_bits) st->pair_sign[g.ang_off + b] = 0;
+  if (g.atab)
+    for (uint32_t b = 0; b < g.atab_w; ++b) st->pair_sign[g.atab_off + b] = 0;
   const uint32_t t = g.t;
   st->last_branch[t] = st->n_branch++;
   st->writes_since[t] = st->reads_since[t] = 0;
   st->arith_since[t] = 0;
-  st->const_val[t] = -1;
+  st->const_val[t] = st->known_val[t] = -1;
   st->last_target = t;
 }
 
@@ -1658,7 +1982,49 @@ constexpr size_t kLazyMax = 64;  // interference steps queued per learned-sizing
 sqs_status run_lazy(sqs_state* st);
 
 // Queues (learned mode) or runs (exact mode) one interference step.
+sqs_status issue_step(sqs_state* st, const Gate1& g_in, uint32_t n_ctrl);
+
+// Marks the bits of a queued load's data field constant as they were before
+// it, or not known constant (the load executes).
+void set_load_field(sqs_state* st, const HostOp& h, bool before) {
+  for (uint32_t b = 0; b < h.d.dst_w; ++b)
+    st->known_val[h.d.dst_off + b] =
+        before && ((h.was_const >> b) & 1ull) ? (int8_t)((h.was_value >> b) & 1ull) : (int8_t)-1;
+}
+
+// Issues an interference step.  A register-valued rotation right after a QRAM
+// load into its angle register commutes with the load when no entry of the
+// table depends on the target qubit (a rotation angle looked up at an address
+// that the rotated qubit is no part of, or at a prefix): the step then reads
+// the entry itself (Gate1::atab), and the load stays queued past it, where
+// the unload that usually follows cancels it (qram()).  A load, a rotation
+// and an unload are then one step that writes the target bit only: nothing
+// is queued before it, and the angle register stays known constant.
 sqs_status issue_branching(sqs_state* st, const Gate1& g_in, uint32_t n_ctrl) {
+  if (g_in.mode != 1 || st->pending.empty() || (st->flags & SQS_MERGE_PLAIN))
+    return issue_step(st, g_in, n_ctrl);
+  const HostOp load = st->pending.back();
+  const DevOp& d = load.d;
+  const uint32_t q = g_in.t - d.src_off;  // address bit of the target (wraps when below)
+  if (d.kind != sqs::OP_QRAM || d.pmask[0] || d.pmask[1] || d.dst_off != g_in.ang_off ||
+      d.dst_w != g_in.ang_w || (g_in.t >= d.src_off && q < d.src_w && ((load.varies >> q) & 1ull)))
+    return issue_step(st, g_in, n_ctrl);
+  Gate1 g = g_in;
+  g.atab = d.table;
+  g.atab_n = d.n_entries;
+  g.atab_bytes = (uint32_t)d.constant;
+  g.atab_off = d.src_off;
+  g.atab_w = d.src_w;
+  g.atab_varies = load.varies;
+  st->pending.pop_back();
+  set_load_field(st, load, true);
+  const sqs_status s = issue_step(st, g, n_ctrl);
+  set_load_field(st, load, false);
+  st->pending.push_back(load);
+  return s;
+}
+
+sqs_status issue_step(sqs_state* st, const Gate1& g_in, uint32_t n_ctrl) {
   float x[SQS_PRED_FEATURES];
   Gate1 g = g_in;
   features(st, g, n_ctrl, x);
@@ -1666,7 +2032,7 @@ sqs_status issue_branching(sqs_state* st, const Gate1& g_in, uint32_t n_ctrl) {
   // constant over the whole state has no partner anywhere; a copy-paired bit
   // has every partner, holding +-1 times the branch's own amplitude.
   const bool plain = (st->flags & SQS_MERGE_PLAIN) != 0;
-  const int8_t b0 = st->const_val[g.t];
+  const int8_t b0 = st->known_val[g.t];
   g.no_partners = (!plain && b0 >= 0) ? 1u : 0u;
   g.fold_sign = plain ? 0 : st->pair_sign[g.t];
   g.defer_ops = defer_ops_ok(st, g) ? 1u : 0u;
@@ -1697,7 +2063,7 @@ sqs_status issue_branching(sqs_state* st, const Gate1& g_in, uint32_t n_ctrl) {
   // An expansion that always acts (no controls that can fail) with
   // U[1][b0] = +-U[0][b0] leaves every branch paired with +-1 times itself.
   int8_t new_sign = 0;
-  if (b0 >= 0 && g.mode != 1 && predicate_known(st, g.cmask, g.cval) == 1) {
+  if (b0 >= 0 && g.mode != 1 && predicate_known(st, st->known_val, g.cmask, g.cval) == 1) {
     // Compared as numbers (0.0 == -0.0): the children U[r][b0] * a then
     // agree, or agree after a sign flip, in every nonzero component, and a
     // signed zero sums like an unsigned one.
@@ -1706,9 +2072,11 @@ sqs_status issue_branching(sqs_state* st, const Gate1& g_in, uint32_t n_ctrl) {
     if (r0[0] == r1[0] && r0[1] == r1[1]) new_sign = 1;
     else if (r0[0] == -r1[0] && r0[1] == -r1[1]) new_sign = -1;
   }
-  g.vary[0] = g.vary[1] = 0ull;
-  for (uint32_t q = 0; q < st->total_bits; ++q)
-    if (st->const_val[q] < 0) g.vary[q >> 6] |= 1ull << (q & 63);
+  g.vary[0] = g.vary[1] = g.fixed[0] = g.fixed[1] = 0ull;
+  for (uint32_t q = 0; q < st->total_bits; ++q) {
+    if (st->known_val[q] < 0) g.vary[q >> 6] |= 1ull << (q & 63);
+    else if (st->known_val[q] > 0) g.fixed[q >> 6] |= 1ull << (q & 63);
+  }
   note_branch(st, g);
   st->pair_sign[g.t] = new_sign;
   if ((st->flags & SQS_SIZING_LEARNED) && st->predictor) {
@@ -1749,6 +2117,29 @@ double grow_factor(float y) {
 sqs_status run_lazy(sqs_state* st) {
   if (st->lazy.empty()) return SQS_OK;
   const size_t n = st->lazy.size();
+  {
+    // While the hard bound stays small no prediction is needed, and none is
+    // waited for: buffers of that size cost less than the waits.
+    uint64_t bound = st->ub, most = bound;
+    for (const auto& q : st->lazy) {
+      bound = std::min(vary_cap(st, q.g), 2 * bound);
+      most = std::max(most, bound);
+    }
+    if (most <= small_bound(st)) {
+      std::vector<sqs_state::Lazy> steps;
+      steps.swap(st->lazy);
+      std::vector<HostOp> tail;
+      tail.swap(st->pending);
+      sqs_status s = SQS_OK;
+      for (size_t i = 0; i < n && s == SQS_OK; ++i) {
+        st->pending.swap(steps[i].ops);
+        s = run_branching(st, steps[i].g);
+      }
+      st->stats.learned_steps += n;
+      st->pending.swap(tail);
+      return s;
+    }
+  }
   std::vector<float> X(n * SQS_PRED_FEATURES), Y(n);
   for (size_t i = 0; i < n; ++i)
     std::memcpy(&X[i * SQS_PRED_FEATURES], st->lazy[i].x, sizeof(st->lazy[i].x));
@@ -2021,6 +2412,7 @@ HostSnap take_snap(const sqs_state* st) {
   h.reads_since = st->reads_since;
   h.arith_since = st->arith_since;
   h.const_val = st->const_val;
+  h.known_val = st->known_val;
   h.pair_sign = st->pair_sign;
   h.n_branch = st->n_branch;
   h.last_target = st->last_target;
@@ -2039,6 +2431,7 @@ void put_snap(sqs_state* st, const HostSnap& h) {
   st->reads_since = h.reads_since;
   st->arith_since = h.arith_since;
   st->const_val = h.const_val;
+  st->known_val = h.known_val;
   st->pair_sign = h.pair_sign;
   st->n_branch = h.n_branch;
   st->last_target = h.last_target;
@@ -2072,7 +2465,7 @@ sqs_status sort_copy(sqs_state* st, uint64_t n, const uint64_t keep[2], Store** 
   std::vector<uint32_t> shifts;
   for (uint32_t q = 0; q < st->total_bits;) {
     const bool kept = (keep[q >> 6] >> (q & 63)) & 1ull;
-    if (!kept || st->const_val[q] >= 0) {
+    if (!kept || st->known_val[q] >= 0) {
       ++q;
       continue;
     }
@@ -2252,6 +2645,8 @@ void sqs_state_destroy(sqs_state* st) {
   dfree(st, st->ctl);
   dfree(st, st->scratch);
   dfree(st, st->sort_buf);
+  dfree(st, st->slot_amp);
+  dfree(st, st->slot_pres);
   for (auto& t : st->ang_tabs) dfree(st, t.dev);
   for (auto& kv : st->tune)
     for (cudaEvent_t e : kv.second.ev)
@@ -2274,9 +2669,7 @@ sqs_status sqs_state_reset(sqs_state* st) {
   if (!st) return SQS_ERR_ARG;
   st->pending.clear();
   st->lazy.clear();
-  st->run_gates.clear();
-  st->run_pre.clear();
-  st->run_tmask[0] = st->run_tmask[1] = st->run_reads[0] = st->run_reads[1] = 0;
+  drop_run(st);
   st->sticky = SQS_OK;
   st->err.clear();
   st->cur_slot = 0;
@@ -2489,12 +2882,32 @@ sqs_status sqs_table_create(sqs_state* st, const void* host_entries, uint64_t n_
     cudaError_t e = cudaMemcpyAsync(t->dev, host_entries, n_entries * entry_bytes,
                                     cudaMemcpyHostToDevice, st->stream);
     // The host buffer belongs to the caller: finish the copy before returning.
+    // Which address bits the entries depend on, found once on the device.
+    unsigned long long bits = 0;
+    uint32_t nb = 0;
+    while (nb < 63 && (1ull << nb) < n_entries) ++nb;
+    s = ensure_scratch(st, sizeof(bits));
+    if (s != SQS_OK) {
+      cudaStreamSynchronize(st->stream);
+      dfree(st, t->dev);
+      delete t;
+      return s;
+    }
+    if (e == cudaSuccess) e = cudaMemsetAsync(st->scratch, 0, sizeof(bits), st->stream);
+    if (e == cudaSuccess)
+      e = sqs::launch_table_bits(st->stream, st->sm_count, t->dev, n_entries, entry_bytes, nb,
+                                 (unsigned long long*)st->scratch);
+    if (e == cudaSuccess)
+      e = cudaMemcpyAsync(&bits, st->scratch, sizeof(bits), cudaMemcpyDeviceToHost, st->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(st->stream);
     if (e != cudaSuccess) {
       dfree(st, t->dev);
       delete t;
       return cuda_fail(st, e, "table upload");
     }
+    // An address bit past the entries matters unless every entry is 0.
+    const uint64_t in = (1ull << nb) - 1ull;
+    t->varies = (bits & in) | ((bits >> 63) ? ~in : 0ull);
   }
   st->tables.push_back(t);
   *out = t;
@@ -2524,6 +2937,22 @@ static sqs_status qram(sqs_state* st, uint32_t addr_reg, uint32_t n_addr, uint32
   o.d.table = t->dev;
   o.d.n_entries = t->n;
   o.d.constant = t->bytes;
+  o.varies = t->varies;
+  for (uint32_t b = 0; b < o.d.dst_w; ++b) {
+    const int8_t c = st->known_val[o.d.dst_off + b];
+    if (c >= 0) o.was_const |= 1ull << b;
+    if (c > 0) o.was_value |= 1ull << b;
+  }
+  // The map is its own inverse: the same load twice in a row is no operation.
+  if (!st->pending.empty() && !(st->flags & SQS_MERGE_PLAIN)) {
+    const HostOp last = st->pending.back();
+    if (last.d.kind == sqs::OP_QRAM && std::memcmp(&last.d, &o.d, sizeof(DevOp)) == 0) {
+      note_op(st, o);
+      st->pending.pop_back();
+      set_load_field(st, last, true);
+      return SQS_OK;
+    }
+  }
   push_op(st, o);
   return SQS_OK;
 }
@@ -2796,9 +3225,7 @@ sqs_status sqs_import(sqs_state* st, const uint64_t* keys, const double* amps, u
   // The imported state replaces the current one: queued operations and a
   // held run are dropped with it.
   st->pending.clear();
-  st->run_gates.clear();
-  st->run_pre.clear();
-  st->run_tmask[0] = st->run_tmask[1] = st->run_reads[0] = st->run_reads[1] = 0;
+  drop_run(st);
   if (!ensure_store(st, st->cur, std::max<uint64_t>(n, 1)))
     return fail(st, SQS_ERR_OOM, "import");
   st->cur.set_dense();
@@ -3006,6 +3433,7 @@ sqs_status sqs_capture_end(sqs_state* st, sqs_graph** out) {
   g->exit = std::move(exit_snap);
   g->launches = launches;
   *out = g;
+  st->captured = true;
   return SQS_OK;
 }
 
@@ -3022,6 +3450,7 @@ sqs_status sqs_graph_launch(sqs_state* st, sqs_graph* g) {
       return fail(st, SQS_ERR_STATE, "the state's buffers changed since the capture");
   st->pending.clear();
   st->lazy.clear();
+  drop_run(st);
   put_snap(st, g->entry);
   cudaError_t e = cudaGraphLaunch(g->exec, st->stream);
   if (e != cudaSuccess) return cuda_fail(st, e, "graph launch");

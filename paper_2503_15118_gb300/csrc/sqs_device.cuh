@@ -272,11 +272,82 @@ __device__ __forceinline__ void for_each_live(const Arr& a, uint64_t n_dense, F 
   }
 }
 
+// Visits this CTA's units of `unit` slots of `in` -- slices of segments, or
+// of the dense array -- and calls body(base, lim) with every thread for each
+// unit holding live slots (lim > 0).  Units are handed out round-robin (unit
+// u to CTA u mod gridDim.x), in spread order over the parts of a segment.
+// For a segmented array the CTA checks blockDim.x of its candidate units at
+// once, one count load per thread, and lists the non-empty ones in shared
+// memory (list: blockDim.x entries): the count loads of empty units overlap
+// instead of forming a chain, which matters when the segment list is sized
+// for a bound far above the count (a graph's static bound).
+template <class F>
+__device__ __forceinline__ void for_units(const Arr& in, uint64_t n_dense, uint32_t unit,
+                                          uint16_t* list, unsigned int* n_list, F&& body) {
+  if (!in.seg_cnt) {
+    const uint64_t units = (n_dense + unit - 1) / unit;
+    for (uint64_t u = blockIdx.x; u < units; u += gridDim.x) {
+      const uint64_t base = u * unit;
+      body(base, (uint32_t)(n_dense - base < unit ? n_dense - base : unit));
+    }
+    return;
+  }
+  const uint32_t per_seg = ((1u << in.seg_log2) + unit - 1) / unit;
+  const uint32_t l = log2_pow2(per_seg);
+  const uint64_t units = (uint64_t)in.n_seg * per_seg;
+  for (uint64_t k0 = 0; blockIdx.x + k0 * gridDim.x < units; k0 += blockDim.x) {
+    if (threadIdx.x == 0) *n_list = 0u;
+    __syncthreads();
+    const uint64_t u = blockIdx.x + (k0 + threadIdx.x) * gridDim.x;
+    if (u < units) {
+      const uint64_t v = spread_visit(u, l);
+      const uint32_t sg = (uint32_t)(v / per_seg);
+      const uint32_t off = (uint32_t)(v - (uint64_t)sg * per_seg) * unit;
+      if (off < in.seg_cnt[sg]) list[atomicAdd(n_list, 1u)] = (uint16_t)threadIdx.x;
+    }
+    __syncthreads();
+    const uint32_t n = *n_list;
+    for (uint32_t i = 0; i < n; ++i) {
+      const uint64_t v = spread_visit(blockIdx.x + (k0 + list[i]) * gridDim.x, l);
+      const uint32_t sg = (uint32_t)(v / per_seg);
+      const uint32_t off = (uint32_t)(v - (uint64_t)sg * per_seg) * unit;
+      const uint32_t cnt = in.seg_cnt[sg];
+      body(((uint64_t)sg << in.seg_log2) + off, cnt - off < unit ? cnt - off : unit);
+    }
+    __syncthreads();  // the list is rebuilt for the next candidates
+  }
+}
+
 // ---- errors --------------------------------------------------------------------
 __device__ __forceinline__ void raise_err(Ctl* ctl, unsigned int bit, uint32_t seq,
                                           unsigned long long need) {
   if (atomicOr(&ctl->err, bit) == 0u) ctl->err_where = seq;
   atomicMax(&ctl->need, need);
+}
+
+// ---- QRAM tables -------------------------------------------------------------------
+// Entry `addr` of a table of n entries of eb bytes; 0 past its end.
+__device__ __forceinline__ uint64_t table_word(const void* t, uint64_t n, uint32_t eb,
+                                               uint64_t addr) {
+  if (addr >= n) return 0ull;
+  switch (eb) {
+    case 1: return __ldg((const uint8_t*)t + addr);
+    case 2: return __ldg((const uint16_t*)t + addr);
+    case 4: return __ldg((const uint32_t*)t + addr);
+    default: return __ldg((const unsigned long long*)t + addr);
+  }
+}
+
+// Value of the angle register of a mode-1 step on branch k (0 for other
+// modes), the word of a load the step stands before included.
+template <class K>
+__device__ __forceinline__ uint64_t angle_value(const Gate1& g, K k) {
+  if (g.mode != 1) return 0ull;
+  uint64_t v = get_field(k, g.ang_off, g.ang_w);
+  if (g.atab)
+    v ^= table_word(g.atab, g.atab_n, g.atab_bytes, get_field(k, g.atab_off, g.atab_w)) &
+         wmask(g.ang_w);
+  return v;
 }
 
 // ---- fused operation run ---------------------------------------------------------
@@ -326,16 +397,8 @@ __device__ __forceinline__ bool apply_ops(uint32_t n_ops, const DevOp* ops, cons
       idx = 0;
     } else if (kind == OP_QRAM) {
       if (on) {
-        const uint64_t addr = get_field(k, op.src_off, op.src_w);
-        uint64_t d = 0;
-        if (addr < op.n_entries) {
-          switch ((uint32_t)op.constant) {
-            case 1: d = __ldg((const uint8_t*)op.table + addr); break;
-            case 2: d = __ldg((const uint16_t*)op.table + addr); break;
-            case 4: d = __ldg((const uint32_t*)op.table + addr); break;
-            default: d = __ldg((const unsigned long long*)op.table + addr); break;
-          }
-        }
+        const uint64_t d = table_word(op.table, op.n_entries, (uint32_t)op.constant,
+                                      get_field(k, op.src_off, op.src_w));
         k = set_field<K>(k, op.dst_off, op.dst_w, get_field(k, op.dst_off, op.dst_w) ^ d);
       }
     } else if (kind == OP_SWAP) {
@@ -430,16 +493,7 @@ __device__ __forceinline__ void apply_ops_n(uint32_t n_ops, const DevOp* ops, co
 #pragma unroll
       for (int q = 0; q < NI; ++q) {
         if (live[q] && (k[q] & pm) == pv) {
-          const uint64_t addr = get_field(k[q], soff, sw);
-          uint64_t d = 0;
-          if (addr < n_ent) {
-            switch (eb) {
-              case 1: d = __ldg((const uint8_t*)tbl + addr); break;
-              case 2: d = __ldg((const uint16_t*)tbl + addr); break;
-              case 4: d = __ldg((const uint32_t*)tbl + addr); break;
-              default: d = __ldg((const unsigned long long*)tbl + addr); break;
-            }
-          }
+          const uint64_t d = table_word(tbl, n_ent, eb, get_field(k[q], soff, sw));
           k[q] = set_field<K>(k[q], doff, dw, get_field(k[q], doff, dw) ^ d);
         }
       }

@@ -288,7 +288,7 @@ __global__ void __launch_bounds__(kGroupThreads, 2)
             if (!h0) a0 = a1;  // unread for an absent member; keeps the operands defined
             if (!h1) a1 = a0;
           }
-          const uint64_t av = act && g.mode == 1 ? get_field(rest, g.ang_off, g.ang_w) : 0ull;
+          const uint64_t av = act ? angle_value(g, rest) : 0ull;
           step_pair<AT>(g, av, act, h0, a0, h1, a1, o0, o1);
           if (act) {
             const bool k0 = keep_amp(o0, g.eps, g.epsf, g.eps2);
@@ -342,7 +342,10 @@ __global__ void __launch_bounds__(kGroupThreads, 2)
 
 __global__ void k_group_peak(Ctl* ctl, uint32_t k) {
   if (threadIdx.x == 0 && blockIdx.x == 0)
-    for (uint32_t j = 0; j < k; ++j) atomicMax(&ctl->peak, ctl->stage[j]);
+    for (uint32_t j = 0; j < k; ++j) {
+      atomicMax(&ctl->peak, ctl->stage[j]);
+      ctl->stage[j] = 0;
+    }
 }
 
 template <int KW, class AT>

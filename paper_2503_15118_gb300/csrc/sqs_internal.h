@@ -84,6 +84,8 @@ struct Arr {
   uint32_t n_seg;
 };
 
+constexpr int kMaxItems = 32;  // steps and phases of one fused run
+
 // Device control block.  The total branch count of the current array lives
 // in a small ring: an operation that writes a new array adds into cnt[out]
 // and clears cnt[(out + 1) & 3] for the operation after it.
@@ -96,9 +98,11 @@ struct Ctl {
   double norm2;
   unsigned long long groups;     // fused run: coherent groups of its input
   unsigned long long items;      // fused run: branches of its input (after the queued run)
-  unsigned long long stage[16];  // fused run: branches after each of its operations
+  unsigned long long stage[kMaxItems];  // fused run: branches after each of its items (zero between runs)
   unsigned int buckets;          // bucket merge: buckets the partition filled
   unsigned int pair_next;        // bucket merge: next bucket a pair CTA takes (the partition zeroes it)
+  unsigned int run_done;         // addressed run: CTAs that finished (zero between runs)
+  unsigned int run_next;         // addressed run: next area a CTA takes (zero between runs)
 };
 
 constexpr unsigned int kErrCapacity = 1u;  // output array too small
@@ -126,6 +130,7 @@ struct Gate1 {            // the interference operation of one merge step
   uint32_t defer_ops;
   uint32_t issue_call;  // host only: the API call that issued the step (trace attribution)
   uint64_t vary[2];       // key bits not known constant over the state (sort digits)
+  uint64_t fixed[2];      // host only: the values of the other bits
   // Copy-pair fold: +1 / -1 when every branch's partner across the target bit
   // is known to exist with amplitude exactly +1 / -1 times its own; 0 otherwise.
   int32_t fold_sign;
@@ -145,6 +150,15 @@ struct Gate1 {            // the interference operation of one merge step
   // into digit 0 (device table owned by the state; null: direct sincos).
   const double2* ang_tab;
   uint32_t ang_digits;
+  // Mode 1, rotation between a QRAM load into the angle register and its
+  // unload: the angle value is the register XOR the word the load would have
+  // put there, entry `address field` of atab (0 past its end).  The host sets
+  // it only when no entry depends on the target bit, so that the load commutes
+  // with the step.  null: the register alone.
+  const void* atab;
+  uint64_t atab_n;
+  uint32_t atab_off, atab_w, atab_bytes;
+  uint64_t atab_varies;  // host only: address bits some entry depends on
 };
 
 // A fused run of interference operations on distinct target bits (Sec.
@@ -159,6 +173,30 @@ struct GroupRun {
   uint32_t pad;
   uint64_t tmask[2];     // union of the target bits
   Gate1 g[kMaxRun];
+};
+
+// A fused run by direct addressing (sqs_run.cu).  The varying key bits, packed
+// by `mv` (bits [src, src + len) of the key at [dst, dst + len) of the slot,
+// never across a key word), number a slot; `base` holds the other bits.
+struct BitMove {
+  uint8_t src, dst, len, pad;
+};
+constexpr int kMaxMoves = 28;       // a slot has at most kMaxSlotBits bits
+constexpr uint32_t kMaxSlotBits = 24;  // 2^24 slots: 285 MB in FP64
+struct SlotMap {
+  uint32_t n, pad;
+  uint64_t base[2];
+  BitMove mv[kMaxMoves];
+};
+// One item: an interference step on slot bit j, or (phase) the factor
+// g.u[0] + i g.u[1], on the slots with (slot & smask) == sval.
+struct RunItem {
+  uint32_t phase, j, smask, sval;
+  Gate1 g;
+};
+struct RunProg {
+  uint32_t n, area_log2, n_areas, pad;
+  RunItem it[kMaxItems];
 };
 
 struct Launch {
@@ -177,6 +215,11 @@ struct Launch {
 // Fills tab[j << 16 | d] = (cos, sin)(scale / 2 * d * 2^(16 j) + (j == 0 ? offset / 2 : 0)).
 cudaError_t launch_angle_table(cudaStream_t s, double2* tab, uint32_t digits, double scale,
                                double offset);
+// Address bits the n entries (eb bytes each, 2^nb >= n) of a table depend on:
+// ORs bit b < nb into *out when flipping address bit b changes some entry
+// (entries past the end read 0), bit 63 when any entry is nonzero.
+cudaError_t launch_table_bits(cudaStream_t s, int sm_count, const void* t, uint64_t n, uint32_t eb,
+                              uint32_t nb, unsigned long long* out);
 cudaError_t launch_init(const Launch& L, Ctl* ctl, Arr a, int slot, bool amp32);
 cudaError_t launch_apply_inplace(const Launch& L, int kw, bool amp32, Ctl* ctl, Arr a, int slot,
                                  const OpList& ops);
@@ -291,6 +334,18 @@ cudaError_t launch_group_count(const Launch& L, int kw, Ctl* ctl, Arr in,
 cudaError_t launch_group(const Launch& L, int kw, bool amp32, Ctl* ctl, Arr in,
                          const unsigned long long* n_ptr, uint32_t tile_len, uint64_t n_tiles,
                          Arr out, int out_slot, const GroupRun& run);
+// Fused run by direct addressing: the queued operations and the scatter into
+// amp[slot] with pres[slot] = 1 (all zero before), then the run itself over
+// the 2^area_log2-slot areas: survivors appended to the dense `out` (count in
+// cnt[out_slot]), pres zeroed, the peak raised to the largest count after a
+// step.
+uint32_t run_area_log2(uint32_t k);
+cudaError_t launch_slot_scatter(const Launch& L, int kw, bool amp32, Ctl* ctl, Arr in, int in_slot,
+                                const OpList& ops, const SlotMap& map, void* amp, uint8_t* pres);
+cudaError_t launch_slot_run(const Launch& L, int kw, bool amp32, Ctl* ctl, void* amp,
+                            uint8_t* pres, const SlotMap& map, const RunProg& prog, Arr out,
+                            int out_slot);
+
 // Raises a kernel's dynamic shared-memory limit to `smem` bytes on the
 // current device, once per device.  The attribute is per device; the
 // bitmask of devices already configured is shared by host threads, so it is

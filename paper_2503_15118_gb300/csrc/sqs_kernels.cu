@@ -42,56 +42,12 @@ __global__ void k_init(Ctl* ctl, Arr a, int slot) {
     ctl->err = 0;
     ctl->err_where = 0;
     ctl->norm2 = 0;
+    for (int i = 0; i < kMaxItems; ++i) ctl->stage[i] = 0;
+    ctl->run_done = ctl->run_next = 0;
   }
 }
 
 // ---------------------------------------------------------------------------
-
-// Visits this CTA's units of `unit` slots of `in` -- slices of segments, or
-// of the dense array -- and calls body(base, lim) with every thread for each
-// unit holding live slots (lim > 0).  Units are handed out round-robin (unit
-// u to CTA u mod gridDim.x), in spread order over the parts of a segment.
-// For a segmented array the CTA checks blockDim.x of its candidate units at
-// once, one count load per thread, and lists the non-empty ones in shared
-// memory (list: blockDim.x entries): the count loads of empty units overlap
-// instead of forming a chain, which matters when the segment list is sized
-// for a bound far above the count (a graph's static bound).
-template <class F>
-__device__ __forceinline__ void for_units(const Arr& in, uint64_t n_dense, uint32_t unit,
-                                          uint16_t* list, unsigned int* n_list, F&& body) {
-  if (!in.seg_cnt) {
-    const uint64_t units = (n_dense + unit - 1) / unit;
-    for (uint64_t u = blockIdx.x; u < units; u += gridDim.x) {
-      const uint64_t base = u * unit;
-      body(base, (uint32_t)(n_dense - base < unit ? n_dense - base : unit));
-    }
-    return;
-  }
-  const uint32_t per_seg = ((1u << in.seg_log2) + unit - 1) / unit;
-  const uint32_t l = log2_pow2(per_seg);
-  const uint64_t units = (uint64_t)in.n_seg * per_seg;
-  for (uint64_t k0 = 0; blockIdx.x + k0 * gridDim.x < units; k0 += blockDim.x) {
-    if (threadIdx.x == 0) *n_list = 0u;
-    __syncthreads();
-    const uint64_t u = blockIdx.x + (k0 + threadIdx.x) * gridDim.x;
-    if (u < units) {
-      const uint64_t v = spread_visit(u, l);
-      const uint32_t sg = (uint32_t)(v / per_seg);
-      const uint32_t off = (uint32_t)(v - (uint64_t)sg * per_seg) * unit;
-      if (off < in.seg_cnt[sg]) list[atomicAdd(n_list, 1u)] = (uint16_t)threadIdx.x;
-    }
-    __syncthreads();
-    const uint32_t n = *n_list;
-    for (uint32_t i = 0; i < n; ++i) {
-      const uint64_t v = spread_visit(blockIdx.x + (k0 + list[i]) * gridDim.x, l);
-      const uint32_t sg = (uint32_t)(v / per_seg);
-      const uint32_t off = (uint32_t)(v - (uint64_t)sg * per_seg) * unit;
-      const uint32_t cnt = in.seg_cnt[sg];
-      body(((uint64_t)sg << in.seg_log2) + off, cnt - off < unit ? cnt - off : unit);
-    }
-    __syncthreads();  // the list is rebuilt for the next candidates
-  }
-}
 
 // Op-major over kApplyILP branches per thread: each operation's descriptor
 // is read once for four branches (the interpreter's instruction count, not
@@ -419,7 +375,7 @@ __global__ void __launch_bounds__(kPairThreads, 3)
           const int j = partner[i];
           k0 = k & ~bmask;
           k1 = k | bmask;
-          const uint64_t av = g.mode == 1 ? get_field(k0, g.ang_off, g.ang_w) : 0ull;
+          const uint64_t av = angle_value(g, k0);
           if (!kt)
             children<AT>(g, av, true, ai, j >= 0, j >= 0 ? samp[j] : ai, o0, o1);
           else
@@ -549,7 +505,7 @@ __global__ void __launch_bounds__(kStreamThreads, 4)
             const bool kt = (k[q] & bmask) != (K)0;
             k0[q] = k[q] & ~bmask;
             k1[q] = k[q] | bmask;
-            const uint64_t av = g.mode == 1 ? get_field(k0[q], g.ang_off, g.ang_w) : 0ull;
+            const uint64_t av = angle_value(g, k0[q]);
             if (g.fold_sign == 0) {
               if (!kt)
                 children<AT>(g, av, true, v[q], false, v[q], o0[q], o1[q]);
@@ -782,7 +738,7 @@ __global__ void __launch_bounds__(kStreamThreads, 3)
           }
           if (__any_sync(0xffffffffu, live[q] && !kill)) {
             if (live[q] && !kill) {
-              const uint64_t avv = g.mode == 1 ? get_field(k0[q], g.ang_off, g.ang_w) : 0ull;
+              const uint64_t avv = angle_value(g, k0[q]);
               children<AT>(g, avv, true, v[q], true, a1, o0[q], o1[q]);
               keep0 = keep_amp(o0[q], g.eps, g.epsf, g.eps2);
               keep1 = keep_amp(o1[q], g.eps, g.epsf, g.eps2);
@@ -1087,7 +1043,7 @@ __global__ void __launch_bounds__(kStreamThreads, 4)
             const bool kt = (k[q] & bmask) != (K)0;
             k0[q] = k[q] & ~bmask;
             k1[q] = k[q] | bmask;
-            const uint64_t av = g.mode == 1 ? get_field(k0[q], g.ang_off, g.ang_w) : 0ull;
+            const uint64_t av = angle_value(g, k0[q]);
             if (g.fold_sign == 0) {
               if (!kt)
                 children<AT>(g, av, true, v[q], false, v[q], o0[q], o1[q]);
@@ -1285,7 +1241,7 @@ __global__ void __launch_bounds__(kStreamThreads, 4)
         }
         if (__any_sync(0xffffffffu, live[q] && !kill)) {
           if (live[q] && !kill) {
-            const uint64_t avv = g.mode == 1 ? get_field(k[q], g.ang_off, g.ang_w) : 0ull;
+            const uint64_t avv = angle_value(g, k[q]);
             children<AT>(g, avv, true, v[q], true, a1, o0[q], o1[q]);
             keep0 = keep_amp(o0[q], g.eps, g.epsf, g.eps2);
             keep1 = keep_amp(o1[q], g.eps, g.epsf, g.eps2);
@@ -1756,7 +1712,7 @@ __global__ void __launch_bounds__(kPairCThreads)
           const uint32_t oidx = ((uint32_t)pj - 1u) & (kSliceCap - 1u);
           aj = *map_rank(samp + oidx, orank);
         }
-        const uint64_t av = g.mode == 1 ? get_field(k0, g.ang_off, g.ang_w) : 0ull;
+        const uint64_t av = angle_value(g, k0);
         if (!kt)
           children<AT>(g, av, true, ai, pj >= 0, aj, o0, o1);
         else
@@ -1878,6 +1834,34 @@ __global__ void k_angle_table(double2* tab, uint32_t digits, double scale, doubl
 cudaError_t launch_angle_table(cudaStream_t s, double2* tab, uint32_t digits, double scale,
                                double offset) {
   k_angle_table<<<256, 256, 0, s>>>(tab, digits, scale, offset);
+  return cudaGetLastError();
+}
+
+// Address bits the entries of a table depend on: bit b of *out is set when
+// some entry differs from the one at the address with bit b flipped (0 past
+// the end), for b < nb; bit 63 when any entry is nonzero.  One pass over the
+// table's own entries, the partners from L2; bits already found are skipped.
+__global__ void k_table_bits(const void* t, uint64_t n, uint32_t eb, uint32_t nb,
+                             unsigned long long* out) {
+  unsigned long long mine = 0ull;
+  const unsigned long long all = (1ull << nb) - 1ull;
+  for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
+       i += (uint64_t)gridDim.x * blockDim.x) {
+    const uint64_t v = table_word(t, n, eb, i);
+    if (v) mine |= 1ull << 63;
+    for (unsigned long long m = all & ~mine; m; m &= m - 1ull) {
+      const uint32_t b = (uint32_t)__ffsll((long long)m) - 1u;
+      if (table_word(t, n, eb, i ^ (1ull << b)) != v) mine |= 1ull << b;
+    }
+  }
+  for (int o = 16; o > 0; o >>= 1) mine |= __shfl_xor_sync(0xffffffffu, mine, o);
+  if ((threadIdx.x & 31u) == 0 && mine) atomicOr(out, mine);
+}
+
+cudaError_t launch_table_bits(cudaStream_t s, int sm_count, const void* t, uint64_t n, uint32_t eb,
+                              uint32_t nb, unsigned long long* out) {
+  const uint64_t want = (n + 255) / 256, cap = (uint64_t)sm_count * 8;
+  k_table_bits<<<(int)(want < cap ? want : cap), 256, 0, s>>>(t, n, eb, nb, out);
   return cudaGetLastError();
 }
 

@@ -1,0 +1,375 @@
+// Fused runs by direct addressing (Sec. II.D.2: the branches that agree on
+// every bit a run does not write form a coherent group, and the run acts on
+// each group by itself).
+//
+// When few key bits vary over a state, a branch's group and its place in the
+// group can be addressed instead of sorted for: the varying bits, packed with
+// the run's targets lowest, number a slot, the group a range of 2^k slots.
+//   k_slot_scatter  applies the queued operations and stores every branch's
+//                   amplitude at its slot, with a presence byte: no sort, no
+//                   counters, no atomics.
+//   k_slot_run      takes areas of whole groups (up to 2^12 slots) into shared
+//                   memory and applies the run's items one after another:
+//                   interference steps and phases.  Per step the pairs with a
+//                   member present and the controls met are listed first (one
+//                   ballot per 32 pairs of presence bits), pairs of two members
+//                   apart from single ones, so that every lane of the FP64
+//                   sequence holds a pair that acts; survivors are appended to
+//                   the dense output.
+// Each step evaluates children() with the presence flags of its pair and
+// prunes with keep_amp(), so the result is that of the steps one by one, bit
+// for bit.  Because a pair's full key is known from its slot, a step may read
+// (controls, angle register, table address) the targets of other steps of the
+// run and a target may come again, which the sorted form (sqs_group.cu) does
+// not allow.
+//
+// What bounds it: FP64 issue of the rotations (12 FP64 instructions a pair and
+// register-valued step) while the areas hold branches, latency of a step's two
+// barriers while they do not; DRAM is idle.  Measured, rotations with their
+// loads and unloads as one step included: an N = 1024 walk step (0.9 M branches
+// on average, 98 steps) 8.4 -> 2.1 ms, three steps of a 128-system walk in
+// non-Hermitian form 10.4 -> 2.6 ms, two of 64 systems batched 14.3 -> 2.4 ms,
+// where partition and pair took 73 us a step at 10^6 branches and 15 us at the
+// smallest.
+#include <cuda_runtime.h>
+#include <stdint.h>
+
+#include "sqs_device.cuh"
+#include "sqs_internal.h"
+
+namespace sqs {
+namespace {
+
+constexpr int kRunThreads = 512;
+constexpr uint32_t kAreaLog2Max = 12;
+static_assert(kMaxRun <= (int)kAreaLog2Max, "a group fits the area");
+
+// The slot of key k (bits moved run by run), and the key of a slot.
+template <class K>
+__device__ __forceinline__ uint32_t slot_of(const SlotMap& m, K k) {
+  const uint64_t w0 = lo64(k), w1 = hi64(k);
+  uint32_t s = 0;
+#pragma unroll 1
+  for (uint32_t i = 0; i < m.n; ++i) {
+    const BitMove v = m.mv[i];
+    const uint64_t w = v.src < 64 ? w0 : w1;
+    s |= ((uint32_t)(w >> (v.src & 63u)) & ((1u << v.len) - 1u)) << v.dst;
+  }
+  return s;
+}
+template <int KW>
+__device__ __forceinline__ typename KT<KW>::T key_of(const SlotMap& m, uint32_t s) {
+  uint64_t w0 = m.base[0], w1 = m.base[1];
+#pragma unroll 1
+  for (uint32_t i = 0; i < m.n; ++i) {
+    const BitMove v = m.mv[i];
+    const uint64_t f = (uint64_t)((s >> v.dst) & ((1u << v.len) - 1u)) << (v.src & 63u);
+    if (KW == 1 || v.src < 64)
+      w0 |= f;
+    else
+      w1 |= f;
+  }
+  return mk<KW>(w0, w1);
+}
+
+constexpr int kScatterILP = 4;
+
+template <int KW, class AT, bool OPS>
+__global__ void __launch_bounds__(kStreamThreads)
+    k_slot_scatter(Ctl* ctl, Arr in, int in_slot, const __grid_constant__ OpList ops,
+                   const __grid_constant__ SlotMap map, AT* amp, uint8_t* pres) {
+  typedef typename KT<KW>::T K;
+  __shared__ AT tab[OPS ? kTabEntries : 1];
+  __shared__ DevOp sops[OPS ? kMaxOps : 1];
+  __shared__ uint16_t ulist[kStreamThreads];
+  __shared__ unsigned int n_ulist;
+  if (ctl->err) return;
+  if (OPS) load_ops(ops, sops, tab);
+  const uint64_t n_dense = ctl->cnt[in_slot];
+  if (blockIdx.x == 0 && threadIdx.x == 0) atomicMax(&ctl->peak, n_dense);
+  for_units(in, n_dense, kScatterILP * blockDim.x, ulist, &n_ulist,
+            [&](uint64_t base, uint32_t lim) {
+    K k[kScatterILP];
+    AT v[kScatterILP];
+    bool live[kScatterILP];
+#pragma unroll
+    for (int q = 0; q < kScatterILP; ++q) {
+      const uint32_t j = q * blockDim.x + threadIdx.x;
+      live[q] = j < lim;
+      k[q] = 0;
+      v[q].x = v[q].y = 0;
+      if (live[q]) {
+        k[q] = ld_key<KW>(in, base + j);
+        v[q] = ((const AT*)in.amp)[base + j];
+      }
+    }
+    if (OPS) apply_ops_n<KW, AT, kScatterILP>(ops.n, sops, tab, k, v, live);
+#pragma unroll
+    for (int q = 0; q < kScatterILP; ++q) {
+      if (live[q]) {
+        const uint32_t s = slot_of(map, k[q]);
+        amp[s] = v[q];
+        pres[s] = 1;
+      }
+    }
+  });
+}
+
+// Shared memory of one k_slot_run CTA (dynamic): the area's amplitudes, then
+//   pres   presence bits, 32 slots a word
+//   list   u16 per pair: pairs of two members from the front, single ones
+//          from the back
+//   wbase  survivors before each presence word (emission)
+template <class AT>
+constexpr size_t run_smem_bytes(uint32_t area_log2) {
+  return ((size_t)sizeof(AT) << area_log2) + ((size_t)8 << (area_log2 - 5)) +
+         ((size_t)2 << (area_log2 - 1));
+}
+
+template <int KW, class AT>
+__global__ void __launch_bounds__(kRunThreads, 2)
+    k_slot_run(Ctl* ctl, AT* gamp, uint8_t* gpres, const __grid_constant__ SlotMap map,
+               const __grid_constant__ RunProg prog, Arr out, int out_slot, uint32_t seq) {
+  typedef typename KT<KW>::T K;
+  extern __shared__ __align__(16) unsigned char smem[];
+  __shared__ unsigned int lc[2][2];  // list counters: [parity][two members, single]
+  __shared__ unsigned int stage[kMaxItems];
+  __shared__ unsigned int wsum[4];
+  __shared__ unsigned long long base_out;
+  __shared__ unsigned int last, next;
+  const uint32_t area = 1u << prog.area_log2, npairs = area >> 1, nwords = area >> 5;
+  AT* amp = (AT*)smem;
+  uint32_t* pres = (uint32_t*)(smem + ((size_t)sizeof(AT) << prog.area_log2));
+  uint32_t* wbase = pres + nwords;
+  uint16_t* list = (uint16_t*)(wbase + nwords);
+  const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5;
+  const unsigned int lt = (1u << lane) - 1u;
+  // After an error (an earlier kernel's) the presence bytes are still cleared:
+  // they are zero between runs.
+  const bool dead = ctl->err != 0u;
+  if (blockIdx.x == 0 && threadIdx.x == 0) ctl->cnt[(out_slot + 1) & 3] = 0;
+  for (uint32_t i = threadIdx.x; i < kMaxItems; i += blockDim.x) stage[i] = 0u;
+  if (threadIdx.x < 4) lc[threadIdx.x >> 1][threadIdx.x & 1u] = 0u;
+  uint32_t par = 0;
+  // Areas are drawn one at a time (the next index while the current area is
+  // processed): branches cluster in some of them, and with a fixed share per
+  // CTA half the SMs idled (a 64-system walk batch: 580 us a run).
+  if (threadIdx.x == 0) next = atomicAdd(&ctl->run_next, 1u);
+  __syncthreads();
+  for (uint32_t b = next; b < prog.n_areas; b = next) {
+    uint32_t drawn = 0u;
+    if (threadIdx.x == 0) drawn = atomicAdd(&ctl->run_next, 1u);
+    const uint32_t s0g = b << prog.area_log2;  // first slot of the area
+    // 1. Presence bytes to bits (16 slots a thread), cleared behind.
+    bool some = false;
+    if (threadIdx.x < area / 16u) {
+      uint4* const src = (uint4*)(gpres + s0g) + threadIdx.x;
+      const uint4 v = *src;
+      unsigned int m = 0u;
+      if (v.x | v.y | v.z | v.w) {
+        // Bytes are 0 or 1: the multiply gathers a word's four into its top nibble.
+        m = ((v.x * 0x10204080u) >> 28) | (((v.y * 0x10204080u) >> 28) << 4) |
+            (((v.z * 0x10204080u) >> 28) << 8) | (((v.w * 0x10204080u) >> 28) << 12);
+        *src = make_uint4(0u, 0u, 0u, 0u);
+        some = true;
+      }
+      ((uint16_t*)pres)[threadIdx.x] = (uint16_t)m;
+    }
+    const bool empty = !__syncthreads_or(some);  // every thread has read `next`
+    if (threadIdx.x == 0) next = drawn;
+    __syncthreads();
+    if (empty || dead) continue;
+#pragma unroll 4
+    for (uint32_t s = threadIdx.x; s < area; s += blockDim.x)
+      if ((pres[s >> 5] >> (s & 31u)) & 1u) amp[s] = gamp[s0g + s];
+    __syncthreads();
+    // 2. The run's items.
+    for (uint32_t i = 0; i < prog.n; ++i) {
+      const RunItem& it = prog.it[i];
+      const uint32_t smask = it.smask, sval = it.sval;
+      if (it.phase) {
+        AT f;
+        to_amp(f, make_double2(it.g.u[0], it.g.u[1]));
+        for (uint32_t s = threadIdx.x; s < area; s += blockDim.x)
+          if (((pres[s >> 5] >> (s & 31u)) & 1u) && ((s0g + s) & smask) == sval)
+            amp[s] = cmul(amp[s], f);
+        __syncthreads();
+        continue;
+      }
+      const Gate1& g = it.g;
+      const uint32_t low = (1u << it.j) - 1u;
+      // The pairs that act.  (npairs is a multiple of 32: whole warps.)
+      for (uint32_t p = threadIdx.x; p < npairs; p += blockDim.x) {
+        const uint32_t s0 = ((p & ~low) << 1) | (p & low), s1 = s0 | (1u << it.j);
+        const unsigned int h0 = (pres[s0 >> 5] >> (s0 & 31u)) & 1u;
+        const unsigned int h1 = (pres[s1 >> 5] >> (s1 & 31u)) & 1u;
+        const bool act = (h0 | h1) && ((s0g + s0) & smask) == sval;
+        const unsigned int b2 = __ballot_sync(0xffffffffu, act && (h0 & h1));
+        const unsigned int b1 = __ballot_sync(0xffffffffu, act && !(h0 & h1));
+        if (b1 | b2) {
+          unsigned int at2 = 0, at1 = 0;
+          if (lane == 0) {
+            if (b2) at2 = atomicAdd(&lc[par][0], (unsigned int)__popc(b2));
+            if (b1) at1 = atomicAdd(&lc[par][1], (unsigned int)__popc(b1));
+          }
+          at2 = __shfl_sync(0xffffffffu, at2, 0);
+          at1 = __shfl_sync(0xffffffffu, at1, 0);
+          if ((b2 >> lane) & 1u) list[at2 + __popc(b2 & lt)] = (uint16_t)p;
+          if ((b1 >> lane) & 1u) list[npairs - 1u - (at1 + __popc(b1 & lt))] = (uint16_t)p;
+        }
+      }
+      __syncthreads();
+      const uint32_t n2 = lc[par][0], n1 = lc[par][1];
+      par ^= 1u;
+      if (threadIdx.x < 2) lc[par][threadIdx.x] = 0u;  // the next step's
+      const uint32_t n2w = (n2 + 31u) & ~31u;
+      for (uint32_t q = threadIdx.x; q < n2w + n1; q += blockDim.x) {
+        const bool two = q < n2;
+        if (!two && q < n2w) continue;
+        const uint32_t p = two ? list[q] : list[npairs - 1u - (q - n2w)];
+        const uint32_t s0 = ((p & ~low) << 1) | (p & low), s1 = s0 | (1u << it.j);
+        const uint32_t m0 = 1u << (s0 & 31u), m1 = 1u << (s1 & 31u);
+        const uint64_t av = g.mode == 1 ? angle_value(g, key_of<KW>(map, s0g + s0)) : 0ull;
+        bool h0 = true, h1 = true;
+        AT o0, o1;
+        if (two) {
+          children<AT>(g, av, true, amp[s0], true, amp[s1], o0, o1);
+        } else {
+          h0 = (pres[s0 >> 5] & m0) != 0u;
+          h1 = !h0;
+          const AT a = amp[h0 ? s0 : s1];
+          if (h0)
+            children<AT>(g, av, true, a, false, a, o0, o1);
+          else
+            children<AT>(g, av, false, a, true, a, o0, o1);
+        }
+        const bool k0 = keep_amp(o0, g.eps, g.epsf, g.eps2);
+        const bool k1 = keep_amp(o1, g.eps, g.epsf, g.eps2);
+        amp[s0] = o0;
+        amp[s1] = o1;
+        if (k0 != h0) atomicXor(&pres[s0 >> 5], m0);
+        if (k1 != h1) atomicXor(&pres[s1 >> 5], m1);
+      }
+      __syncthreads();
+      // Branches after the step (the words change again only after the next
+      // step's list barrier).
+      if (threadIdx.x < nwords) {
+        unsigned int c = __popc(pres[threadIdx.x]);
+        for (int o = 16; o > 0; o >>= 1) c += __shfl_xor_sync(0xffffffffu, c, o);
+        if (lane == 0 && c) atomicAdd(&stage[i], c);
+      }
+    }
+    // 3. Survivors to the dense output.
+    unsigned int c = 0, incl = 0;
+    if (threadIdx.x < nwords) {
+      c = incl = __popc(pres[threadIdx.x]);
+      for (int o = 1; o < 32; o <<= 1) {
+        const unsigned int y = __shfl_up_sync(0xffffffffu, incl, o);
+        if (lane >= (uint32_t)o) incl += y;
+      }
+      if (lane == 31) wsum[warp] = incl;
+    }
+    __syncthreads();
+    if (threadIdx.x < nwords) {
+      unsigned int before = incl - c;
+      for (uint32_t w = 0; w < warp; ++w) before += wsum[w];
+      wbase[threadIdx.x] = before;
+      if (threadIdx.x == nwords - 1u) {
+        const unsigned int sum = before + c;
+        base_out = sum ? atomicAdd(&ctl->cnt[out_slot], (unsigned long long)sum) : 0ull;
+        if (sum && base_out + sum > out.cap) raise_err(ctl, kErrCapacity, seq, base_out + sum);
+      }
+    }
+    __syncthreads();
+    const unsigned long long ob = base_out;
+#pragma unroll 2
+    for (uint32_t s = threadIdx.x; s < area; s += blockDim.x) {
+      const uint32_t w = pres[s >> 5];
+      if ((w >> lane) & 1u) {  // s & 31 == lane
+        const uint64_t pos = ob + wbase[s >> 5] + __popc(w & lt);
+        if (pos < out.cap) {
+          st_key<KW>(out, pos, key_of<KW>(map, s0g + s));
+          ((AT*)out.amp)[pos] = amp[s];
+        }
+      }
+    }
+    __syncthreads();  // the area is reused
+  }
+  // 4. The counts after each step; the last CTA raises the peak and clears
+  //    them for the next run.
+  for (uint32_t i = threadIdx.x; i < prog.n; i += blockDim.x)
+    if (stage[i]) atomicAdd(&ctl->stage[i], (unsigned long long)stage[i]);
+  __threadfence();
+  __syncthreads();
+  if (threadIdx.x == 0) last = atomicAdd(&ctl->run_done, 1u) == gridDim.x - 1u;
+  __syncthreads();
+  if (last) {
+    __threadfence();
+    for (uint32_t i = threadIdx.x; i < prog.n; i += blockDim.x) {
+      const unsigned long long v = atomicExch(&ctl->stage[i], 0ull);
+      if (v) atomicMax(&ctl->peak, v);
+    }
+    if (threadIdx.x == 0) ctl->run_done = ctl->run_next = 0u;
+  }
+}
+
+template <int KW, class AT>
+cudaError_t scatter_t(const Launch& L, Ctl* ctl, Arr in, int in_slot, const OpList& ops,
+                      const SlotMap& map, void* amp, uint8_t* pres) {
+  const uint64_t per = (uint64_t)kScatterILP * kStreamThreads;
+  uint64_t grid = (L.n_hint + per - 1) / per;
+  const uint64_t cap = (uint64_t)L.sm_count * 8;
+  grid = grid < 1 ? 1 : (grid > cap ? cap : grid);
+  if (ops.n)
+    k_slot_scatter<KW, AT, true><<<(int)grid, kStreamThreads, 0, L.stream>>>(
+        ctl, in, in_slot, ops, map, (AT*)amp, pres);
+  else
+    k_slot_scatter<KW, AT, false><<<(int)grid, kStreamThreads, 0, L.stream>>>(
+        ctl, in, in_slot, ops, map, (AT*)amp, pres);
+  return cudaGetLastError();
+}
+
+template <int KW, class AT>
+cudaError_t run_t(const Launch& L, Ctl* ctl, void* amp, uint8_t* pres, const SlotMap& map,
+                  const RunProg& prog, Arr out, int out_slot) {
+  static std::atomic<unsigned long long> configured{0};  // opt-in above 48 KB, per device
+  cudaError_t e = ensure_smem_optin((const void*)k_slot_run<KW, AT>,
+                                    run_smem_bytes<AT>(kAreaLog2Max), configured);
+  if (e != cudaSuccess) return e;
+  const uint32_t wave = (uint32_t)L.sm_count * 2u;
+  const uint32_t grid = prog.n_areas < wave ? prog.n_areas : wave;
+  k_slot_run<KW, AT><<<grid, kRunThreads, run_smem_bytes<AT>(prog.area_log2), L.stream>>>(
+      ctl, (AT*)amp, pres, map, prog, out, out_slot, L.seq);
+  return cudaGetLastError();
+}
+
+}  // namespace
+
+cudaError_t launch_slot_scatter(const Launch& L, int kw, bool amp32, Ctl* ctl, Arr in, int in_slot,
+                                const OpList& ops, const SlotMap& map, void* amp, uint8_t* pres) {
+  if (kw == 2)
+    return amp32 ? scatter_t<2, float2>(L, ctl, in, in_slot, ops, map, amp, pres)
+                 : scatter_t<2, double2>(L, ctl, in, in_slot, ops, map, amp, pres);
+  return amp32 ? scatter_t<1, float2>(L, ctl, in, in_slot, ops, map, amp, pres)
+               : scatter_t<1, double2>(L, ctl, in, in_slot, ops, map, amp, pres);
+}
+
+// Slots per shared-memory area: one group, at least 2^10 slots (a full block's
+// work per step).  More groups to an area mean fewer barriers, but also fewer
+// areas to balance over the SMs: a 64-system walk batch spends 191 us a run
+// with 2^12 slots, 149 us with the smallest areas, the N = 1024 walk the same.
+uint32_t run_area_log2(uint32_t k) { return k > 10u ? k : 10u; }
+
+cudaError_t launch_slot_run(const Launch& L, int kw, bool amp32, Ctl* ctl, void* amp,
+                            uint8_t* pres, const SlotMap& map, const RunProg& prog, Arr out,
+                            int out_slot) {
+  if (prog.n > (uint32_t)kMaxItems || prog.area_log2 > kAreaLog2Max || prog.area_log2 < 10u)
+    return cudaErrorInvalidValue;
+  if (kw == 2)
+    return amp32 ? run_t<2, float2>(L, ctl, amp, pres, map, prog, out, out_slot)
+                 : run_t<2, double2>(L, ctl, amp, pres, map, prog, out, out_slot);
+  return amp32 ? run_t<1, float2>(L, ctl, amp, pres, map, prog, out, out_slot)
+               : run_t<1, double2>(L, ctl, amp, pres, map, prog, out, out_slot);
+}
+
+}  // namespace sqs

@@ -360,7 +360,7 @@ __global__ void __launch_bounds__(kStreamThreads)
             const bool kt = (k & bmask) != (K)0;
             k0 = p;
             k1 = p | bmask;
-            const uint64_t av = g.mode == 1 ? get_field(k0, g.ang_off, g.ang_w) : 0ull;
+            const uint64_t av = angle_value(g, k0);
             if (has_p) {
               const AT ap = ((const AT*)in.amp)[i + 1];
               if (!kt)
