@@ -815,8 +815,11 @@ sqs_status run_hashed(sqs_state* st, const Gate1& g, double est_in, int64_t rec_
   cudaError_t e;
   {
     Traced tr(st, SQS_K_PARTITION);
+    uint64_t tbit[2] = {0ull, 0ull};
+    tbit[g.t >> 6] = 1ull << (g.t & 63);
     e = sqs::launch_partition(launch_of(st, in_slots), st->kw, st->amp32, st->ctl,
-                              st->cur.view(), st->cur_slot, L, g, st->bk.view(), (uint32_t)target);
+                              st->cur.view(), st->cur_slot, L, tbit, st->bk.view(),
+                              (uint32_t)target);
   }
   if (e != cudaSuccess) return cuda_fail(st, e, "partition launch");
   {
@@ -1433,49 +1436,44 @@ bool slots_pay(const sqs_state* st, const std::vector<sqs_state::Held>& run, int
   return fused < alone;
 }
 
-// The held run (k targets) by direct addressing: the queued operations and
-// the scatter of every branch to its slot, then every group transformed in
-// shared memory.  No host wait: the output holds at most one branch per slot,
-// or 2^k per input branch.
-sqs_status run_slots(sqs_state* st, const std::vector<sqs_state::Held>& run,
-                     const uint64_t tmask[2]) {
-  TraceCall attribution(st, run[0].g.issue_call);
-  sqs_status s = run_pending(st, true);  // leaves the fused operations in ops_buf
-  if (s != SQS_OK) return st->sticky = s;
-  const Gate1& last = run.back().g;
-  uint64_t vary[2];
-  run_vary(last, tmask, vary);
-  const uint32_t bits = (uint32_t)bits_set(vary), k = (uint32_t)bits_set(tmask);
-  const uint64_t slots = 1ull << bits;
-
-  // Slot layout: the targets in key order in the low k bits, then the others.
-  sqs::SlotMap map;
+// Slot layout and items of a run (st->run_prog): the targets in key order in
+// the low bits of the slot, then the other bits of `vary` (none: a bucketed
+// run, whose slots number a group's members and whose predicates on other bits
+// are tested on the group's key).
+void build_run(sqs_state* st, const std::vector<sqs_state::Held>& run, const uint64_t tmask[2],
+               const uint64_t* vary, sqs::SlotMap& map) {
   std::memset(&map, 0, sizeof(map));
-  uint8_t at[128];  // slot bit of each varying key bit
+  const uint64_t in[2] = {vary ? vary[0] : tmask[0], vary ? vary[1] : tmask[1]};
+  uint8_t at[128];  // slot bit of each key bit in the slot
   uint32_t pos = 0;
   for (int pass = 0; pass < 2; ++pass)
     for (uint32_t q = 0; q < st->total_bits; ++q) {
-      const bool v = (vary[q >> 6] >> (q & 63)) & 1ull, t = (tmask[q >> 6] >> (q & 63)) & 1ull;
+      const bool v = (in[q >> 6] >> (q & 63)) & 1ull, t = (tmask[q >> 6] >> (q & 63)) & 1ull;
       if (!v || t != (pass == 0)) continue;
       at[q] = (uint8_t)pos;
       sqs::BitMove* m = map.n ? &map.mv[map.n - 1] : nullptr;
-      if (m && m->src + m->len == q && m->dst + m->len == pos && (q & 63))
+      if (m && m->src + m->len == (int)q && m->dst + m->len == (int)pos && (q & 63))
         m->len++;
       else
         map.mv[map.n++] = sqs::BitMove{(uint8_t)q, (uint8_t)pos, 1, 0};
       ++pos;
     }
-  for (int w = 0; w < 2; ++w) map.base[w] = last.fixed[w] & ~vary[w];
+  if (vary)
+    for (int w = 0; w < 2; ++w) map.base[w] = run.back().g.fixed[w] & ~vary[w];
   // A predicate over the key as one over the slot; false when a constant bit
   // fails it.
   auto slot_pred = [&](const uint64_t pm[2], const uint64_t pv[2], sqs::RunItem& it) {
     it.smask = it.sval = 0;
+    it.rmask[0] = it.rmask[1] = it.rval[0] = it.rval[1] = 0;
     for (uint32_t q = 0; q < st->total_bits; ++q) {
       if (!((pm[q >> 6] >> (q & 63)) & 1ull)) continue;
-      const uint32_t want = (uint32_t)((pv[q >> 6] >> (q & 63)) & 1ull);
-      if ((vary[q >> 6] >> (q & 63)) & 1ull) {
+      const uint64_t want = (pv[q >> 6] >> (q & 63)) & 1ull;
+      if ((in[q >> 6] >> (q & 63)) & 1ull) {
         it.smask |= 1u << at[q];
-        it.sval |= want << at[q];
+        it.sval |= (uint32_t)want << at[q];
+      } else if (!vary) {
+        it.rmask[q >> 6] |= 1ull << (q & 63);
+        it.rval[q >> 6] |= want << (q & 63);
       } else if (((map.base[q >> 6] >> (q & 63)) & 1ull) != want) {
         return false;
       }
@@ -1484,8 +1482,9 @@ sqs_status run_slots(sqs_state* st, const std::vector<sqs_state::Held>& run,
   };
   sqs::RunProg& prog = st->run_prog;
   prog.n = 0;
-  for (const auto& h : run) {
-    if (h.after_phase) {
+  for (size_t i = 0; i < run.size(); ++i) {
+    const auto& h = run[i];
+    if (h.after_phase && i > 0) {  // before the first step a phase is queued instead
       sqs::RunItem& it = prog.it[prog.n];
       std::memset(&it, 0, sizeof(it));
       if (slot_pred(h.phase.d.pmask, h.phase.d.pval, it)) {
@@ -1501,6 +1500,26 @@ sqs_status run_slots(sqs_state* st, const std::vector<sqs_state::Held>& run,
     it.g = h.g;
     if (slot_pred(h.g.cmask, h.g.cval, it)) ++prog.n;  // else it acts on no branch
   }
+}
+
+// The held run (k targets) by direct addressing: the queued operations and
+// the scatter of every branch to its slot, then every group transformed in
+// shared memory.  No host wait: the output holds at most one branch per slot,
+// or 2^k per input branch.
+sqs_status run_slots(sqs_state* st, const std::vector<sqs_state::Held>& run,
+                     const uint64_t tmask[2]) {
+  TraceCall attribution(st, run[0].g.issue_call);
+  sqs_status s = run_pending(st, true);  // leaves the fused operations in ops_buf
+  if (s != SQS_OK) return st->sticky = s;
+  const Gate1& last = run.back().g;
+  uint64_t vary[2];
+  run_vary(last, tmask, vary);
+  const uint32_t bits = (uint32_t)bits_set(vary), k = (uint32_t)bits_set(tmask);
+  const uint64_t slots = 1ull << bits;
+
+  sqs::SlotMap map;
+  build_run(st, run, tmask, vary, map);
+  sqs::RunProg& prog = st->run_prog;
   prog.area_log2 = sqs::run_area_log2(k);
   prog.n_areas = bits > prog.area_log2 ? 1u << (bits - prog.area_log2) : 1u;
   const uint64_t want = (uint64_t)prog.n_areas << prog.area_log2;
@@ -1548,6 +1567,83 @@ sqs_status run_slots(sqs_state* st, const std::vector<sqs_state::Held>& run,
   return SQS_OK;
 }
 
+// Steps on few targets over hash buckets (k_partition with the targets cleared,
+// k_bucket_run): any state, whatever its keys.  *taken stays false, with
+// nothing done, when the output -- up to 2^k branches per input branch -- would
+// need more memory than it should: a quarter of what is free, or, after a graph
+// capture, any move of the buffers.
+sqs_status run_bucketed(sqs_state* st, const std::vector<sqs_state::Held>& run,
+                        const uint64_t tmask[2], bool& taken) {
+  taken = false;
+  const uint32_t k = (uint32_t)bits_set(tmask);
+  // Groups come whole, up to 2^k branches: lower fills than the pair merge's
+  // keep an overflow of the 2048 slots (64 groups where 16 are the mean) as
+  // far away, e^-80 a bucket for k = 4, e^-55 for k = 5.
+  const uint64_t fill = k <= 4 ? 512 : 384;
+  auto grown = [&] {
+    uint64_t vary[2];
+    run_vary(run.back().g, tmask, vary);
+    const uint64_t cap =
+        std::min<uint64_t>(max_branches(st), 1ull << std::min(bits_set(vary), 62));
+    return st->ub > (cap >> k) ? cap : st->ub << k;
+  };
+  auto buckets = [&] { return std::max<uint64_t>(1, (st->ub + fill - 1) / fill); };
+  auto fits = [&] {
+    return grown() <= st->alt.cap && (buckets() << kBucketLog2) <= st->bk.cap;
+  };
+  if (!fits() && st->ub > small_bound(st)) {
+    sqs_status s = sync_bound(st);  // the bound outgrew the allocation: exact count
+    if (s != SQS_OK) return s;
+  }
+  if (buckets() > 0x7fffffffull) return SQS_OK;
+  if (!fits()) {
+    if (st->captured) return SQS_OK;
+    size_t free_b = 0, total_b = 0;
+    if (cudaMemGetInfo(&free_b, &total_b) != cudaSuccess) {
+      cudaGetLastError();
+      return SQS_OK;
+    }
+    const double rb = (double)(8 * st->kw + amp_bytes(st));
+    if (rb * ((double)grown() + (double)(buckets() << kBucketLog2)) > (double)free_b / 4)
+      return SQS_OK;
+  }
+  taken = true;
+  TraceCall attribution(st, run[0].g.issue_call);
+  sqs_status s = run_pending(st, true);  // leaves the fused operations in ops_buf
+  if (s != SQS_OK) return st->sticky = s;
+  const uint64_t out_need = grown(), B = buckets();
+  if ((st->bk.cap < (B << kBucketLog2) && !ensure_store(st, st->bk, B << kBucketLog2)) ||
+      (st->alt.cap < out_need && !ensure_store(st, st->alt, out_need)))
+    return st->sticky = fail(st, SQS_ERR_OOM, "cannot allocate %llu branches",
+                             (unsigned long long)out_need);
+  sqs::SlotMap map;
+  build_run(st, run, tmask, nullptr, map);
+  st->bk.set_segments(kBucketLog2, (uint32_t)B);
+  st->alt.set_dense();
+  const uint64_t in_slots = st->cur.slots(st->ub);
+  const int out_slot = (st->cur_slot + 1) & 3;
+  cudaError_t e;
+  {
+    Traced tr(st, SQS_K_PARTITION);
+    e = sqs::launch_partition(launch_of(st, in_slots), st->kw, st->amp32, st->ctl, st->cur.view(),
+                              st->cur_slot, st->ops_buf, tmask, st->bk.view(), (uint32_t)fill);
+  }
+  if (e != cudaSuccess) return cuda_fail(st, e, "partition launch");
+  {
+    Traced tr(st, SQS_K_GROUP);
+    e = sqs::launch_bucket_run(launch_of(st, in_slots), st->kw, st->amp32, st->ctl,
+                               st->bk.view(), map, st->run_prog, k, tmask, st->alt.view(),
+                               out_slot);
+  }
+  if (e != cudaSuccess) return cuda_fail(st, e, "bucket run launch");
+  std::swap(st->cur, st->alt);
+  st->cur_slot = out_slot;
+  st->ub = out_need;
+  st->stats.runs_fused++;
+  st->stats.steps_fused += run.size();
+  return SQS_OK;
+}
+
 // Reads of a step besides its target: controls, angle bits, and the table
 // address bits that some entry depends on.
 void step_reads(const Gate1& g, uint64_t reads[2]) {
@@ -1563,20 +1659,83 @@ void step_reads(const Gate1& g, uint64_t reads[2]) {
       if ((g.atab_varies >> b) & 1ull) add(g.atab_off + b);
 }
 
-// A run of steps with nothing between them, in the sorted form's terms:
-// fused when that pays, else one by one.
-sqs_status run_steps(sqs_state* st, const std::vector<Gate1>& gates) {
-  if (gates.size() >= 2 && fuse_pays(st, gates)) return run_group(st, gates);
+// Runs held steps that are not addressed.  In pieces the sorted form allows
+// (distinct targets no other step of the piece reads, no phase, no fold) where
+// sorting them pays; what is left, on a state too wide to address, in pieces
+// of up to kMaxHashRun targets over hash buckets when at least three launches
+// are saved; else step by step.
+sqs_status run_pieces(sqs_state* st, const std::vector<sqs_state::Held>& run, bool wide) {
   sqs_status s = SQS_OK;
-  for (size_t j = 0; j < gates.size() && s == SQS_OK; ++j)
-    s = run_branching(st, gates[j]);  // the queued operations go with the first
+  auto tbit = [](const Gate1& g, uint64_t t[2]) {
+    t[0] = t[1] = 0;
+    t[g.t >> 6] = 1ull << (g.t & 63);
+  };
+  auto alone = [&](const sqs_state::Held* h, size_t n) {
+    for (size_t i = 0; i < n && s == SQS_OK; ++i) {
+      if (h[i].after_phase && i > 0) st->pending.push_back(h[i].phase);
+      s = run_branching(st, h[i].g);  // the queued operations go with the first
+    }
+  };
+  auto bucketed = [&](const sqs_state::Held* h, size_t n) {
+    while (n && s == SQS_OK) {
+      uint64_t tm[2] = {0, 0}, t[2];
+      size_t m = 0;
+      double launches = 0.0;
+      for (; m < n; ++m) {
+        tbit(h[m].g, t);
+        const uint64_t both[2] = {tm[0] | t[0], tm[1] | t[1]};
+        if (bits_set(both) > sqs::kMaxHashRun) break;
+        tm[0] = both[0];
+        tm[1] = both[1];
+        launches += h[m].g.no_partners || h[m].g.fold_sign ? 1.0 : 2.0;
+      }
+      bool taken = false;
+      if (wide && m >= 2 && launches >= 3.0)
+        s = run_bucketed(st, std::vector<sqs_state::Held>(h, h + m), tm, taken);
+      if (s == SQS_OK && !taken) alone(h, m);
+      if (m < n && h[m].after_phase && s == SQS_OK) st->pending.push_back(h[m].phase);
+      h += m;
+      n -= m;
+    }
+  };
+  size_t from = 0;  // first step not yet run
+  while (from < run.size() && s == SQS_OK) {
+    // The longest sorted-form piece that starts here.
+    uint64_t pt[2] = {0, 0}, pr[2] = {0, 0}, t[2], reads[2];
+    size_t end = from;
+    std::vector<Gate1> gates;
+    for (; end < run.size(); ++end) {
+      const Gate1& g = run[end].g;
+      step_reads(g, reads);
+      tbit(g, t);
+      if (end > from &&
+          (run[end].after_phase || g.fold_sign || gates.back().fold_sign ||
+           ((pt[0] | pr[0]) & t[0]) || ((pt[1] | pr[1]) & t[1]) || (reads[0] & pt[0]) ||
+           (reads[1] & pt[1])))
+        break;
+      gates.push_back(g);
+      for (int w = 0; w < 2; ++w) {
+        pt[w] |= t[w];
+        pr[w] |= reads[w];
+      }
+    }
+    if (gates.size() >= 2 && fuse_pays(st, gates)) {
+      s = run_group(st, gates);
+    } else if (wide) {
+      end = run.size();  // bucketed pieces may go on past it
+      bucketed(&run[from], end - from);
+    } else {
+      alone(&run[from], end - from);
+    }
+    if (end < run.size() && run[end].after_phase && s == SQS_OK)
+      st->pending.push_back(run[end].phase);
+    from = end;
+  }
   return s;
 }
 
 // Executes the held run: by direct addressing where few bits vary, else in
-// pieces the sorted form allows (distinct targets that no other step of the
-// piece reads), each fused or step by step.  Operations queued after the run
-// stay queued after it.
+// pieces (run_pieces).  Operations queued after the run stay queued after it.
 sqs_status flush_run(sqs_state* st) {
   if (st->run.empty()) return SQS_OK;
   std::vector<sqs_state::Held> run;
@@ -1606,30 +1765,7 @@ sqs_status flush_run(sqs_state* st) {
   } else if (addressed) {
     s = run_slots(st, run, tmask);
   } else {
-    std::vector<Gate1> part;
-    uint64_t pt[2] = {0, 0}, pr[2] = {0, 0};
-    for (size_t i = 0; i < run.size() && s == SQS_OK; ++i) {
-      const Gate1& g = run[i].g;
-      uint64_t reads[2], t[2] = {0, 0};
-      step_reads(g, reads);
-      t[g.t >> 6] = 1ull << (g.t & 63);
-      const bool joins = !part.empty() && !run[i].after_phase && !g.fold_sign &&
-                         !part.back().fold_sign && !((pt[0] | pr[0]) & t[0]) &&
-                         !((pt[1] | pr[1]) & t[1]) && !(reads[0] & pt[0]) && !(reads[1] & pt[1]);
-      if (!joins) {
-        s = run_steps(st, part);
-        if (s != SQS_OK) break;
-        part.clear();
-        pt[0] = pt[1] = pr[0] = pr[1] = 0;
-        if (run[i].after_phase) st->pending.push_back(run[i].phase);
-      }
-      part.push_back(g);
-      for (int w = 0; w < 2; ++w) {
-        pt[w] |= t[w];
-        pr[w] |= reads[w];
-      }
-    }
-    if (s == SQS_OK) s = run_steps(st, part);
+    s = run_pieces(st, run, slot_bits > (int)sqs::kMaxSlotBits);
   }
   if (st->pending.empty()) st->pending.swap(after);
   else st->pending.insert(st->pending.end(), after.begin(), after.end());
@@ -1648,9 +1784,10 @@ bool fusing(const sqs_state* st) {
 // new one with it.  A step joins when nothing was queued since the run's last
 // step, its target is new to the run and read by no step of it, and it reads
 // (controls, angle register, table address) none of the run's targets: the
-// sorted form.  While few enough key bits vary for an addressed run, a step on
-// any target joins, whatever it reads, one phase may lie between two steps,
-// and so may a copy-pair fold, which opens no run: alone it is one pass.
+// sorted form.  A step on any target joins whatever it reads, one phase may lie
+// between two steps and so may a copy-pair fold (which opens no run: alone it
+// is one pass) while few enough key bits vary for an addressed run, or while
+// the targets are few enough for a bucketed one.
 sqs_status hold_step(sqs_state* st, const Gate1& g) {
   uint64_t reads[2];
   step_reads(g, reads);
@@ -1676,7 +1813,8 @@ sqs_status hold_step(sqs_state* st, const Gate1& g) {
     const int most = slots && !(st->flags & SQS_FUSE_ALWAYS)
                          ? std::max(9, std::min(sqs::kMaxRun, bits - 8))
                          : sqs::kMaxRun;
-    join = bits_set(targets) <= most && (sorted_form || slots) &&
+    join = bits_set(targets) <= most &&
+           (sorted_form || slots || bits_set(targets) <= sqs::kMaxHashRun) &&
            (st->pending.empty() || phase) &&
            st->run_items + 1u + (phase ? 1u : 0u) <= (uint32_t)sqs::kMaxItems;
   }

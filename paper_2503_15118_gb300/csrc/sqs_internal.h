@@ -190,8 +190,11 @@ struct SlotMap {
 };
 // One item: an interference step on slot bit j, or (phase) the factor
 // g.u[0] + i g.u[1], on the slots with (slot & smask) == sval.
+// Bucketed runs: the slot bits are those of the index in the group, and the
+// rest of the group's key must match rval under rmask as well.
 struct RunItem {
   uint32_t phase, j, smask, sval;
+  uint64_t rmask[2], rval[2];
   Gate1 g;
 };
 struct RunProg {
@@ -228,7 +231,8 @@ cudaError_t launch_apply_inplace(const Launch& L, int kw, bool amp32, Ctl* ctl, 
 cudaError_t launch_apply_compact(const Launch& L, int kw, bool amp32, Ctl* ctl, Arr in,
                                  int in_slot, Arr out, int out_slot, const OpList& ops);
 // Streams `in` through the run and scatters every branch into the hash bucket
-// of its pair class (key with the target bit cleared).  bk is segmented with
+// of its pair class or group (key with the bits of `clear` cleared: the
+// target's, or a run's targets').  bk is segmented with
 // bk.n_seg buckets of 2^bk.seg_log2 slots, counters zero on entry.
 // Buckets follow the device count: ceil(count / fill_target) of them, at
 // most bk.n_seg (the host's bound; fill_target 0 keeps bk.n_seg); the pair
@@ -245,7 +249,8 @@ cudaError_t launch_apply_compact(const Launch& L, int kw, bool amp32, Ctl* ctl, 
 // either way.
 constexpr uint32_t kBucketCntLog2 = 5;
 cudaError_t launch_partition(const Launch& L, int kw, bool amp32, Ctl* ctl, Arr in, int in_slot,
-                             const OpList& ops, const Gate1& g, Arr bk, uint32_t fill_target);
+                             const OpList& ops, const uint64_t clear[2], Arr bk,
+                             uint32_t fill_target);
 
 // Radix-sort merge (sqs_sort.cu).  One LSD pass: digit `shift` of the
 // pair-class key (key with bit t deleted) of `in` -> `out` (dense), stable.
@@ -345,6 +350,15 @@ cudaError_t launch_slot_scatter(const Launch& L, int kw, bool amp32, Ctl* ctl, A
 cudaError_t launch_slot_run(const Launch& L, int kw, bool amp32, Ctl* ctl, void* amp,
                             uint8_t* pres, const SlotMap& map, const RunProg& prog, Arr out,
                             int out_slot);
+
+// Fused run of few targets over hash buckets (launch_partition with the
+// targets as its clear mask): every group of a bucket laid out as 2^k slots in
+// shared memory and run; `map` moves the targets between key and slot index.
+// Clears the bucket counters; output and counts as launch_slot_run.
+constexpr int kMaxHashRun = 5;
+cudaError_t launch_bucket_run(const Launch& L, int kw, bool amp32, Ctl* ctl, Arr bk,
+                              const SlotMap& map, const RunProg& prog, uint32_t k,
+                              const uint64_t tmask[2], Arr out, int out_slot);
 
 // Raises a kernel's dynamic shared-memory limit to `smem` bytes on the
 // current device, once per device.  The attribute is per device; the

@@ -165,8 +165,8 @@ constexpr int kPartILP = 4;
 
 template <int KW, class AT>
 __global__ void __launch_bounds__(kStreamThreads)
-    k_partition(Ctl* ctl, Arr in, int in_slot, const __grid_constant__ OpList ops, Gate1 g,
-                Arr bk, uint32_t seq, uint32_t fill_target) {
+    k_partition(Ctl* ctl, Arr in, int in_slot, const __grid_constant__ OpList ops, uint64_t clear0,
+                uint64_t clear1, Arr bk, uint32_t seq, uint32_t fill_target) {
   typedef typename KT<KW>::T K;
   __shared__ AT tab[kTabEntries];
   __shared__ DevOp sops[kMaxOps];
@@ -185,7 +185,7 @@ __global__ void __launch_bounds__(kStreamThreads)
     ctl->buckets = n_buckets;
     ctl->pair_next = 0u;
   }
-  const K bmask = bit_mask<KW>(g.t);
+  const K bmask = mk<KW>(clear0, clear1);
   const uint32_t C = 1u << bk.seg_log2;
   __shared__ uint16_t ulist[kStreamThreads];
   __shared__ unsigned int n_ulist;
@@ -1961,11 +1961,12 @@ cudaError_t launch_fold(const Launch& L, int kw, bool amp32, Ctl* ctl, Arr in, i
 }
 
 cudaError_t launch_partition(const Launch& L, int kw, bool amp32, Ctl* ctl, Arr in, int in_slot,
-                             const OpList& ops, const Gate1& g, Arr bk, uint32_t fill_target) {
+                             const OpList& ops, const uint64_t clear[2], Arr bk,
+                             uint32_t fill_target) {
   const int grid = stream_grid(L, kStreamThreads);
 #define SQS_PT(KW_, AT_)                                                                \
-  k_partition<KW_, AT_><<<grid, kStreamThreads, 0, L.stream>>>(ctl, in, in_slot, ops, g, \
-                                                               bk, L.seq, fill_target)
+  k_partition<KW_, AT_><<<grid, kStreamThreads, 0, L.stream>>>(             \
+      ctl, in, in_slot, ops, clear[0], clear[1], bk, L.seq, fill_target)
   SQS_DISPATCH(kw, amp32, SQS_PT);
 #undef SQS_PT
   return cudaGetLastError();

@@ -115,52 +115,236 @@ __global__ void __launch_bounds__(kStreamThreads)
   });
 }
 
-// Shared memory of one k_slot_run CTA (dynamic): the area's amplitudes, then
+// Shared state of a CTA that runs items over an area of slots.  Dynamic: the
+// area's amplitudes, then
 //   pres   presence bits, 32 slots a word
+//   wbase  survivors before each presence word (emission)
 //   list   u16 per pair: pairs of two members from the front, single ones
 //          from the back
-//   wbase  survivors before each presence word (emission)
 template <class AT>
-constexpr size_t run_smem_bytes(uint32_t area_log2) {
+__host__ __device__ constexpr size_t run_smem_bytes(uint32_t area_log2) {
   return ((size_t)sizeof(AT) << area_log2) + ((size_t)8 << (area_log2 - 5)) +
          ((size_t)2 << (area_log2 - 1));
 }
+template <class AT>
+struct Area {
+  uint32_t log2;
+  AT* amp;
+  uint32_t *pres, *wbase;
+  uint16_t* list;
+  __device__ Area(unsigned char* smem, uint32_t area_log2) : log2(area_log2) {
+    amp = (AT*)smem;
+    pres = (uint32_t*)(smem + ((size_t)sizeof(AT) << area_log2));
+    wbase = pres + (1u << (area_log2 - 5));
+    list = (uint16_t*)(wbase + (1u << (area_log2 - 5)));
+  }
+};
+struct RunShared {
+  unsigned int lc[2][2];  // list counters: [parity][two members, single]
+  unsigned int stage[kMaxItems];
+  unsigned int wsum[4];
+  unsigned long long base_out;
+  unsigned int last, next, dead;
+};
+
+// Applies the run's items to the area, one after another.  keys.ok(it, s)
+// tells whether item it acts on slot s, a present one or the other of its pair
+// (its predicate; the same for both), keys.key(s) the key of slot s.  Called by the whole CTA with the
+// area's amplitudes and presence bits written and a barrier passed; returns
+// past a barrier.
+template <int KW, class AT, class Keys>
+__device__ __forceinline__ void run_items(const RunProg& prog, const Area<AT>& A, RunShared& sh,
+                                          uint32_t& par, const Keys& keys) {
+  const uint32_t area = 1u << A.log2, npairs = area >> 1, nwords = area >> 5;
+  AT* const amp = A.amp;
+  uint32_t* const pres = A.pres;
+  uint16_t* const list = A.list;
+  const uint32_t lane = threadIdx.x & 31u;
+  const unsigned int lt = (1u << lane) - 1u;
+  for (uint32_t i = 0; i < prog.n; ++i) {
+    const RunItem& it = prog.it[i];
+    if (it.phase) {
+      AT f;
+      to_amp(f, make_double2(it.g.u[0], it.g.u[1]));
+      for (uint32_t s = threadIdx.x; s < area; s += blockDim.x)
+        if (((pres[s >> 5] >> (s & 31u)) & 1u) && keys.ok(it, s)) amp[s] = cmul(amp[s], f);
+      __syncthreads();
+      continue;
+    }
+    const Gate1& g = it.g;
+    const uint32_t low = (1u << it.j) - 1u;
+    // The pairs that act.  (npairs is a multiple of 32: whole warps.)
+    for (uint32_t p = threadIdx.x; p < npairs; p += blockDim.x) {
+      const uint32_t s0 = ((p & ~low) << 1) | (p & low), s1 = s0 | (1u << it.j);
+      const unsigned int h0 = (pres[s0 >> 5] >> (s0 & 31u)) & 1u;
+      const unsigned int h1 = (pres[s1 >> 5] >> (s1 & 31u)) & 1u;
+      const bool act = (h0 | h1) && keys.ok(it, s0);
+      const unsigned int b2 = __ballot_sync(0xffffffffu, act && (h0 & h1));
+      const unsigned int b1 = __ballot_sync(0xffffffffu, act && !(h0 & h1));
+      if (b1 | b2) {
+        unsigned int at2 = 0, at1 = 0;
+        if (lane == 0) {
+          if (b2) at2 = atomicAdd(&sh.lc[par][0], (unsigned int)__popc(b2));
+          if (b1) at1 = atomicAdd(&sh.lc[par][1], (unsigned int)__popc(b1));
+        }
+        at2 = __shfl_sync(0xffffffffu, at2, 0);
+        at1 = __shfl_sync(0xffffffffu, at1, 0);
+        if ((b2 >> lane) & 1u) list[at2 + __popc(b2 & lt)] = (uint16_t)p;
+        if ((b1 >> lane) & 1u) list[npairs - 1u - (at1 + __popc(b1 & lt))] = (uint16_t)p;
+      }
+    }
+    __syncthreads();
+    const uint32_t n2 = sh.lc[par][0], n1 = sh.lc[par][1];
+    par ^= 1u;
+    if (threadIdx.x < 2) sh.lc[par][threadIdx.x] = 0u;  // the next step's
+    const uint32_t n2w = (n2 + 31u) & ~31u;
+    for (uint32_t q = threadIdx.x; q < n2w + n1; q += blockDim.x) {
+      const bool two = q < n2;
+      if (!two && q < n2w) continue;
+      const uint32_t p = two ? list[q] : list[npairs - 1u - (q - n2w)];
+      const uint32_t s0 = ((p & ~low) << 1) | (p & low), s1 = s0 | (1u << it.j);
+      const uint32_t m0 = 1u << (s0 & 31u), m1 = 1u << (s1 & 31u);
+      const uint64_t av = g.mode == 1 ? angle_value(g, keys.key(s0)) : 0ull;
+      bool h0 = true, h1 = true;
+      AT o0, o1;
+      if (two) {
+        children<AT>(g, av, true, amp[s0], true, amp[s1], o0, o1);
+      } else {
+        h0 = (pres[s0 >> 5] & m0) != 0u;
+        h1 = !h0;
+        const AT a = amp[h0 ? s0 : s1];
+        if (h0)
+          children<AT>(g, av, true, a, false, a, o0, o1);
+        else
+          children<AT>(g, av, false, a, true, a, o0, o1);
+      }
+      const bool k0 = keep_amp(o0, g.eps, g.epsf, g.eps2);
+      const bool k1 = keep_amp(o1, g.eps, g.epsf, g.eps2);
+      amp[s0] = o0;
+      amp[s1] = o1;
+      if (k0 != h0) atomicXor(&pres[s0 >> 5], m0);
+      if (k1 != h1) atomicXor(&pres[s1 >> 5], m1);
+    }
+    __syncthreads();
+    // Branches after the step (the words change again only after the next
+    // step's list barrier).
+    if (threadIdx.x < nwords) {
+      unsigned int c = __popc(pres[threadIdx.x]);
+      for (int o = 16; o > 0; o >>= 1) c += __shfl_xor_sync(0xffffffffu, c, o);
+      if (lane == 0 && c) atomicAdd(&sh.stage[i], c);
+    }
+  }
+}
+
+// Appends the area's survivors to the dense output; ends with a barrier.
+template <int KW, class AT, class Keys>
+__device__ __forceinline__ void emit_area(Ctl* ctl, const Area<AT>& A, RunShared& sh,
+                                          const Keys& keys, const Arr& out, int out_slot,
+                                          uint32_t seq) {
+  const uint32_t area = 1u << A.log2, nwords = area >> 5;
+  const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5;
+  const unsigned int lt = (1u << lane) - 1u;
+  unsigned int c = 0, incl = 0;
+  if (threadIdx.x < nwords) {
+    c = incl = __popc(A.pres[threadIdx.x]);
+    for (int o = 1; o < 32; o <<= 1) {
+      const unsigned int y = __shfl_up_sync(0xffffffffu, incl, o);
+      if (lane >= (uint32_t)o) incl += y;
+    }
+    if (lane == 31) sh.wsum[warp] = incl;
+  }
+  __syncthreads();
+  if (threadIdx.x < nwords) {
+    unsigned int before = incl - c;
+    for (uint32_t w = 0; w < warp; ++w) before += sh.wsum[w];
+    A.wbase[threadIdx.x] = before;
+    if (threadIdx.x == nwords - 1u) {
+      const unsigned int sum = before + c;
+      sh.base_out = sum ? atomicAdd(&ctl->cnt[out_slot], (unsigned long long)sum) : 0ull;
+      if (sum && sh.base_out + sum > out.cap)
+        raise_err(ctl, kErrCapacity, seq, sh.base_out + sum);
+    }
+  }
+  __syncthreads();
+  const unsigned long long ob = sh.base_out;
+#pragma unroll 2
+  for (uint32_t s = threadIdx.x; s < area; s += blockDim.x) {
+    const uint32_t w = A.pres[s >> 5];
+    if ((w >> lane) & 1u) {  // s & 31 == lane
+      const uint64_t pos = ob + A.wbase[s >> 5] + __popc(w & lt);
+      if (pos < out.cap) {
+        st_key<KW>(out, pos, keys.key(s));
+        ((AT*)out.amp)[pos] = A.amp[s];
+      }
+    }
+  }
+  __syncthreads();  // the area is reused
+}
+
+// The counts after each step; the last CTA raises the peak and clears them
+// (and the work counter) for the next run.
+__device__ __forceinline__ void finish_run(Ctl* ctl, const RunProg& prog, RunShared& sh) {
+  for (uint32_t i = threadIdx.x; i < prog.n; i += blockDim.x)
+    if (sh.stage[i]) atomicAdd(&ctl->stage[i], (unsigned long long)sh.stage[i]);
+  __threadfence();
+  __syncthreads();
+  if (threadIdx.x == 0) sh.last = atomicAdd(&ctl->run_done, 1u) == gridDim.x - 1u;
+  __syncthreads();
+  if (sh.last) {
+    __threadfence();
+    for (uint32_t i = threadIdx.x; i < prog.n; i += blockDim.x) {
+      const unsigned long long v = atomicExch(&ctl->stage[i], 0ull);
+      if (v) atomicMax(&ctl->peak, v);
+    }
+    if (threadIdx.x == 0) ctl->run_done = ctl->run_next = 0u;
+  }
+}
+
+__device__ __forceinline__ void begin_run(Ctl* ctl, RunShared& sh, int out_slot) {
+  if (blockIdx.x == 0 && threadIdx.x == 0) ctl->cnt[(out_slot + 1) & 3] = 0;
+  for (uint32_t i = threadIdx.x; i < kMaxItems; i += blockDim.x) sh.stage[i] = 0u;
+  if (threadIdx.x < 4) sh.lc[threadIdx.x >> 1][threadIdx.x & 1u] = 0u;
+  // Work is drawn one piece at a time (the next index while the current piece
+  // is processed): branches cluster in some areas, and with a fixed share per
+  // CTA half the SMs idled (a 64-system walk batch: 580 us a run).
+  if (threadIdx.x == 0) {
+    sh.next = atomicAdd(&ctl->run_next, 1u);
+    sh.dead = ctl->err;  // one answer for the CTA: another may raise an error any time
+  }
+  __syncthreads();
+}
+
+// Slots of an addressed run: predicates are masks of the slot number.
+template <int KW>
+struct SlotKeys {
+  const SlotMap& map;
+  uint32_t first;  // slot of the area's slot 0
+  __device__ __forceinline__ bool ok(const RunItem& it, uint32_t s) const {
+    return ((first + s) & it.smask) == it.sval;
+  }
+  __device__ __forceinline__ typename KT<KW>::T key(uint32_t s) const {
+    return key_of<KW>(map, first + s);
+  }
+};
 
 template <int KW, class AT>
 __global__ void __launch_bounds__(kRunThreads, 2)
     k_slot_run(Ctl* ctl, AT* gamp, uint8_t* gpres, const __grid_constant__ SlotMap map,
                const __grid_constant__ RunProg prog, Arr out, int out_slot, uint32_t seq) {
-  typedef typename KT<KW>::T K;
   extern __shared__ __align__(16) unsigned char smem[];
-  __shared__ unsigned int lc[2][2];  // list counters: [parity][two members, single]
-  __shared__ unsigned int stage[kMaxItems];
-  __shared__ unsigned int wsum[4];
-  __shared__ unsigned long long base_out;
-  __shared__ unsigned int last, next;
-  const uint32_t area = 1u << prog.area_log2, npairs = area >> 1, nwords = area >> 5;
-  AT* amp = (AT*)smem;
-  uint32_t* pres = (uint32_t*)(smem + ((size_t)sizeof(AT) << prog.area_log2));
-  uint32_t* wbase = pres + nwords;
-  uint16_t* list = (uint16_t*)(wbase + nwords);
-  const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5;
-  const unsigned int lt = (1u << lane) - 1u;
-  // After an error (an earlier kernel's) the presence bytes are still cleared:
-  // they are zero between runs.
-  const bool dead = ctl->err != 0u;
-  if (blockIdx.x == 0 && threadIdx.x == 0) ctl->cnt[(out_slot + 1) & 3] = 0;
-  for (uint32_t i = threadIdx.x; i < kMaxItems; i += blockDim.x) stage[i] = 0u;
-  if (threadIdx.x < 4) lc[threadIdx.x >> 1][threadIdx.x & 1u] = 0u;
+  __shared__ RunShared sh;
+  const Area<AT> A(smem, prog.area_log2);
+  const uint32_t area = 1u << prog.area_log2;
   uint32_t par = 0;
-  // Areas are drawn one at a time (the next index while the current area is
-  // processed): branches cluster in some of them, and with a fixed share per
-  // CTA half the SMs idled (a 64-system walk batch: 580 us a run).
-  if (threadIdx.x == 0) next = atomicAdd(&ctl->run_next, 1u);
-  __syncthreads();
-  for (uint32_t b = next; b < prog.n_areas; b = next) {
+  begin_run(ctl, sh, out_slot);
+  // After an error the presence bytes are still cleared: they are zero between
+  // runs.
+  const bool dead = sh.dead != 0u;
+  for (uint32_t b = sh.next; b < prog.n_areas; b = sh.next) {
     uint32_t drawn = 0u;
     if (threadIdx.x == 0) drawn = atomicAdd(&ctl->run_next, 1u);
     const uint32_t s0g = b << prog.area_log2;  // first slot of the area
-    // 1. Presence bytes to bits (16 slots a thread), cleared behind.
+    // Presence bytes to bits (16 slots a thread), cleared behind.
     bool some = false;
     if (threadIdx.x < area / 16u) {
       uint4* const src = (uint4*)(gpres + s0g) + threadIdx.x;
@@ -173,144 +357,158 @@ __global__ void __launch_bounds__(kRunThreads, 2)
         *src = make_uint4(0u, 0u, 0u, 0u);
         some = true;
       }
-      ((uint16_t*)pres)[threadIdx.x] = (uint16_t)m;
+      ((uint16_t*)A.pres)[threadIdx.x] = (uint16_t)m;
     }
     const bool empty = !__syncthreads_or(some);  // every thread has read `next`
-    if (threadIdx.x == 0) next = drawn;
+    if (threadIdx.x == 0) sh.next = drawn;
     __syncthreads();
     if (empty || dead) continue;
 #pragma unroll 4
     for (uint32_t s = threadIdx.x; s < area; s += blockDim.x)
-      if ((pres[s >> 5] >> (s & 31u)) & 1u) amp[s] = gamp[s0g + s];
+      if ((A.pres[s >> 5] >> (s & 31u)) & 1u) A.amp[s] = gamp[s0g + s];
     __syncthreads();
-    // 2. The run's items.
-    for (uint32_t i = 0; i < prog.n; ++i) {
-      const RunItem& it = prog.it[i];
-      const uint32_t smask = it.smask, sval = it.sval;
-      if (it.phase) {
-        AT f;
-        to_amp(f, make_double2(it.g.u[0], it.g.u[1]));
-        for (uint32_t s = threadIdx.x; s < area; s += blockDim.x)
-          if (((pres[s >> 5] >> (s & 31u)) & 1u) && ((s0g + s) & smask) == sval)
-            amp[s] = cmul(amp[s], f);
-        __syncthreads();
-        continue;
+    const SlotKeys<KW> keys{map, s0g};
+    run_items<KW, AT>(prog, A, sh, par, keys);
+    emit_area<KW, AT>(ctl, A, sh, keys, out, out_slot, seq);
+  }
+  finish_run(ctl, prog, sh);
+}
+
+// ---------------------------------------------------------------------------
+// Bucketed runs: where too many key bits vary to address slots, k_partition
+// scatters the branches by a hash of the key with the run's few targets
+// cleared, so that every group (at most 2^kMaxHashRun branches) lies in one
+// bucket.  k_bucket_run numbers a bucket's groups through an open-addressing
+// table in shared memory (over the amplitude area, which is free then), lays
+// batches of them out as 2^k slots each and runs the items as above.  A round
+// of the QRAM workload (4 rotations and their inverses on 2^20 two-word
+// branches, 2^24 in between) took 8 partitions and 8 pair launches, 3.6 ms;
+// the state in between now never leaves shared memory.
+constexpr uint32_t kBucketCap = 2048;
+constexpr uint32_t kBucketTable = 2 * kBucketCap;
+constexpr uint32_t kBucketAreaLog2 = 12;
+
+template <int KW, class AT>
+struct BucketSmem {
+  typedef typename KT<KW>::T K;
+  static constexpr size_t key_off = run_smem_bytes<AT>(kBucketAreaLog2);
+  static constexpr size_t gid_off = key_off + kBucketCap * sizeof(K);
+  static constexpr size_t rep_off = gid_off + kBucketCap * 2;
+  static constexpr size_t bytes = rep_off + kBucketCap * 2;
+  static_assert(kBucketTable * 4 <= (sizeof(AT) << kBucketAreaLog2), "the table fits the area");
+  static_assert(bytes <= 112u * 1024u, "two CTAs per SM");
+};
+
+// Slots of a batch of groups: slot (group, index) with the group's first
+// branch as its representative.
+template <int KW>
+struct GroupKeys {
+  typedef typename KT<KW>::T K;
+  const SlotMap& map;  // moves between the k index bits and the key
+  const K* skey;
+  const uint16_t* rep;  // of the batch's groups
+  uint32_t k;
+  K tmask;
+  __device__ __forceinline__ K rest(uint32_t s) const { return skey[rep[s >> k]] & ~tmask; }
+  __device__ __forceinline__ bool ok(const RunItem& it, uint32_t s) const {
+    if ((s & it.smask) != it.sval) return false;
+    if ((it.rmask[0] | it.rmask[1]) == 0ull) return true;
+    return (rest(s) & mk<KW>(it.rmask[0], it.rmask[1])) == mk<KW>(it.rval[0], it.rval[1]);
+  }
+  __device__ __forceinline__ K key(uint32_t s) const {
+    return rest(s) | key_of<KW>(map, s & ((1u << k) - 1u));
+  }
+};
+
+template <int KW, class AT>
+__global__ void __launch_bounds__(kRunThreads, 2)
+    k_bucket_run(Ctl* ctl, Arr bk, const __grid_constant__ SlotMap map,
+                 const __grid_constant__ RunProg prog, uint32_t k, uint64_t tm0, uint64_t tm1,
+                 Arr out, int out_slot, uint32_t seq) {
+  typedef typename KT<KW>::T K;
+  typedef BucketSmem<KW, AT> L;
+  extern __shared__ __align__(16) unsigned char smem[];
+  __shared__ RunShared sh;
+  __shared__ unsigned int n_groups;
+  const Area<AT> A(smem, kBucketAreaLog2);
+  K* const skey = (K*)(smem + L::key_off);
+  uint16_t* const gid = (uint16_t*)(smem + L::gid_off);
+  uint16_t* const rep = (uint16_t*)(smem + L::rep_off);
+  unsigned int* const slot = (unsigned int*)smem;  // over the area
+  const K tmask = mk<KW>(tm0, tm1);
+  const uint32_t per_batch = 1u << (kBucketAreaLog2 - k);
+  uint32_t par = 0;
+  begin_run(ctl, sh, out_slot);
+  const uint32_t nb = sh.dead ? 0u : ctl->buckets;
+  for (uint32_t b = sh.next; b < nb; b = sh.next) {
+    uint32_t drawn = 0u;
+    if (threadIdx.x == 0) {
+      drawn = atomicAdd(&ctl->run_next, 1u);
+      n_groups = 0u;
+    }
+    unsigned int* const bcnt = &bk.seg_cnt[(uint64_t)b << kBucketCntLog2];
+    const uint32_t cnt = *bcnt;
+    const uint32_t n = cnt > kBucketCap ? 0u : cnt;  // overflow: flagged by the partition
+    const uint64_t base = (uint64_t)b << bk.seg_log2;
+    // 1. Keys, and the group of every branch: first its representative (the
+    //    branch that claimed the group's table slot), then the group's number.
+    for (uint32_t i = threadIdx.x; i < n; i += blockDim.x) skey[i] = ld_key<KW>(bk, base + i);
+    for (uint32_t i = threadIdx.x; i < kBucketTable; i += blockDim.x) slot[i] = 0u;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+      sh.next = drawn;
+      *bcnt = 0u;  // the bucket is clean for the next use
+    }
+    for (uint32_t i = threadIdx.x; i < n; i += blockDim.x) {
+      const K p = skey[i] & ~tmask;
+      uint32_t h = (uint32_t)khash(p) & (kBucketTable - 1u);
+      // n <= half the table: a free slot or the group is found within it.
+      for (uint32_t probe = 0; probe < kBucketTable; ++probe) {
+        const unsigned int old = atomicCAS(&slot[h], 0u, i + 1u);
+        if (old == 0u) {
+          const unsigned int id = atomicAdd(&n_groups, 1u);
+          rep[id] = (uint16_t)i;
+          break;
+        }
+        if ((skey[old - 1u] & ~tmask) == p) break;
+        h = (h + 1u) & (kBucketTable - 1u);
       }
-      const Gate1& g = it.g;
-      const uint32_t low = (1u << it.j) - 1u;
-      // The pairs that act.  (npairs is a multiple of 32: whole warps.)
-      for (uint32_t p = threadIdx.x; p < npairs; p += blockDim.x) {
-        const uint32_t s0 = ((p & ~low) << 1) | (p & low), s1 = s0 | (1u << it.j);
-        const unsigned int h0 = (pres[s0 >> 5] >> (s0 & 31u)) & 1u;
-        const unsigned int h1 = (pres[s1 >> 5] >> (s1 & 31u)) & 1u;
-        const bool act = (h0 | h1) && ((s0g + s0) & smask) == sval;
-        const unsigned int b2 = __ballot_sync(0xffffffffu, act && (h0 & h1));
-        const unsigned int b1 = __ballot_sync(0xffffffffu, act && !(h0 & h1));
-        if (b1 | b2) {
-          unsigned int at2 = 0, at1 = 0;
-          if (lane == 0) {
-            if (b2) at2 = atomicAdd(&lc[par][0], (unsigned int)__popc(b2));
-            if (b1) at1 = atomicAdd(&lc[par][1], (unsigned int)__popc(b1));
-          }
-          at2 = __shfl_sync(0xffffffffu, at2, 0);
-          at1 = __shfl_sync(0xffffffffu, at1, 0);
-          if ((b2 >> lane) & 1u) list[at2 + __popc(b2 & lt)] = (uint16_t)p;
-          if ((b1 >> lane) & 1u) list[npairs - 1u - (at1 + __popc(b1 & lt))] = (uint16_t)p;
+      gid[i] = (uint16_t)h;  // the group's table slot
+    }
+    __syncthreads();
+    const uint32_t G = n_groups;
+    // Table slot -> group number (a slot holds its representative).
+    for (uint32_t q = threadIdx.x; q < G; q += blockDim.x) {
+      const K p = skey[rep[q]] & ~tmask;
+      uint32_t h = (uint32_t)khash(p) & (kBucketTable - 1u);
+      while (slot[h] != (unsigned int)rep[q] + 1u) h = (h + 1u) & (kBucketTable - 1u);
+      slot[h] = (q << 16) | 0x8000u;  // no branch index: read as a number below
+    }
+    __syncthreads();
+    for (uint32_t i = threadIdx.x; i < n; i += blockDim.x) gid[i] = (uint16_t)(slot[gid[i]] >> 16);
+    __syncthreads();
+    // 2. Batches of whole groups.
+    for (uint32_t g0 = 0; g0 < G; g0 += per_batch) {
+      const uint32_t gn = G - g0 < per_batch ? G - g0 : per_batch;
+      for (uint32_t w = threadIdx.x; w < (1u << (kBucketAreaLog2 - 5)); w += blockDim.x)
+        A.pres[w] = 0u;
+      __syncthreads();
+      for (uint32_t i = threadIdx.x; i < n; i += blockDim.x) {
+        const uint32_t q = (uint32_t)gid[i] - g0;  // wraps below the batch
+        if (q < gn) {
+          const uint32_t s = (q << k) | slot_of(map, skey[i]);
+          A.amp[s] = ((const AT*)bk.amp)[base + i];
+          atomicOr(&A.pres[s >> 5], 1u << (s & 31u));
         }
       }
       __syncthreads();
-      const uint32_t n2 = lc[par][0], n1 = lc[par][1];
-      par ^= 1u;
-      if (threadIdx.x < 2) lc[par][threadIdx.x] = 0u;  // the next step's
-      const uint32_t n2w = (n2 + 31u) & ~31u;
-      for (uint32_t q = threadIdx.x; q < n2w + n1; q += blockDim.x) {
-        const bool two = q < n2;
-        if (!two && q < n2w) continue;
-        const uint32_t p = two ? list[q] : list[npairs - 1u - (q - n2w)];
-        const uint32_t s0 = ((p & ~low) << 1) | (p & low), s1 = s0 | (1u << it.j);
-        const uint32_t m0 = 1u << (s0 & 31u), m1 = 1u << (s1 & 31u);
-        const uint64_t av = g.mode == 1 ? angle_value(g, key_of<KW>(map, s0g + s0)) : 0ull;
-        bool h0 = true, h1 = true;
-        AT o0, o1;
-        if (two) {
-          children<AT>(g, av, true, amp[s0], true, amp[s1], o0, o1);
-        } else {
-          h0 = (pres[s0 >> 5] & m0) != 0u;
-          h1 = !h0;
-          const AT a = amp[h0 ? s0 : s1];
-          if (h0)
-            children<AT>(g, av, true, a, false, a, o0, o1);
-          else
-            children<AT>(g, av, false, a, true, a, o0, o1);
-        }
-        const bool k0 = keep_amp(o0, g.eps, g.epsf, g.eps2);
-        const bool k1 = keep_amp(o1, g.eps, g.epsf, g.eps2);
-        amp[s0] = o0;
-        amp[s1] = o1;
-        if (k0 != h0) atomicXor(&pres[s0 >> 5], m0);
-        if (k1 != h1) atomicXor(&pres[s1 >> 5], m1);
-      }
-      __syncthreads();
-      // Branches after the step (the words change again only after the next
-      // step's list barrier).
-      if (threadIdx.x < nwords) {
-        unsigned int c = __popc(pres[threadIdx.x]);
-        for (int o = 16; o > 0; o >>= 1) c += __shfl_xor_sync(0xffffffffu, c, o);
-        if (lane == 0 && c) atomicAdd(&stage[i], c);
-      }
+      const GroupKeys<KW> keys{map, skey, rep + g0, k, tmask};
+      run_items<KW, AT>(prog, A, sh, par, keys);
+      emit_area<KW, AT>(ctl, A, sh, keys, out, out_slot, seq);
     }
-    // 3. Survivors to the dense output.
-    unsigned int c = 0, incl = 0;
-    if (threadIdx.x < nwords) {
-      c = incl = __popc(pres[threadIdx.x]);
-      for (int o = 1; o < 32; o <<= 1) {
-        const unsigned int y = __shfl_up_sync(0xffffffffu, incl, o);
-        if (lane >= (uint32_t)o) incl += y;
-      }
-      if (lane == 31) wsum[warp] = incl;
-    }
-    __syncthreads();
-    if (threadIdx.x < nwords) {
-      unsigned int before = incl - c;
-      for (uint32_t w = 0; w < warp; ++w) before += wsum[w];
-      wbase[threadIdx.x] = before;
-      if (threadIdx.x == nwords - 1u) {
-        const unsigned int sum = before + c;
-        base_out = sum ? atomicAdd(&ctl->cnt[out_slot], (unsigned long long)sum) : 0ull;
-        if (sum && base_out + sum > out.cap) raise_err(ctl, kErrCapacity, seq, base_out + sum);
-      }
-    }
-    __syncthreads();
-    const unsigned long long ob = base_out;
-#pragma unroll 2
-    for (uint32_t s = threadIdx.x; s < area; s += blockDim.x) {
-      const uint32_t w = pres[s >> 5];
-      if ((w >> lane) & 1u) {  // s & 31 == lane
-        const uint64_t pos = ob + wbase[s >> 5] + __popc(w & lt);
-        if (pos < out.cap) {
-          st_key<KW>(out, pos, key_of<KW>(map, s0g + s));
-          ((AT*)out.amp)[pos] = amp[s];
-        }
-      }
-    }
-    __syncthreads();  // the area is reused
+    if (G == 0) __syncthreads();  // every thread has left the shared state
   }
-  // 4. The counts after each step; the last CTA raises the peak and clears
-  //    them for the next run.
-  for (uint32_t i = threadIdx.x; i < prog.n; i += blockDim.x)
-    if (stage[i]) atomicAdd(&ctl->stage[i], (unsigned long long)stage[i]);
-  __threadfence();
-  __syncthreads();
-  if (threadIdx.x == 0) last = atomicAdd(&ctl->run_done, 1u) == gridDim.x - 1u;
-  __syncthreads();
-  if (last) {
-    __threadfence();
-    for (uint32_t i = threadIdx.x; i < prog.n; i += blockDim.x) {
-      const unsigned long long v = atomicExch(&ctl->stage[i], 0ull);
-      if (v) atomicMax(&ctl->peak, v);
-    }
-    if (threadIdx.x == 0) ctl->run_done = ctl->run_next = 0u;
-  }
+  finish_run(ctl, prog, sh);
 }
 
 template <int KW, class AT>
@@ -343,7 +541,34 @@ cudaError_t run_t(const Launch& L, Ctl* ctl, void* amp, uint8_t* pres, const Slo
   return cudaGetLastError();
 }
 
+template <int KW, class AT>
+cudaError_t bucket_t(const Launch& L, Ctl* ctl, Arr bk, const SlotMap& map, const RunProg& prog,
+                     uint32_t k, const uint64_t tmask[2], Arr out, int out_slot) {
+  static std::atomic<unsigned long long> configured{0};  // opt-in above 48 KB, per device
+  const size_t smem = BucketSmem<KW, AT>::bytes;
+  cudaError_t e = ensure_smem_optin((const void*)k_bucket_run<KW, AT>, smem, configured);
+  if (e != cudaSuccess) return e;
+  const uint32_t wave = (uint32_t)L.sm_count * 2u;
+  const uint32_t grid = bk.n_seg < wave ? bk.n_seg : wave;
+  k_bucket_run<KW, AT><<<grid ? grid : 1u, kRunThreads, smem, L.stream>>>(
+      ctl, bk, map, prog, k, tmask[0], tmask[1], out, out_slot, L.seq);
+  return cudaGetLastError();
+}
+
 }  // namespace
+
+cudaError_t launch_bucket_run(const Launch& L, int kw, bool amp32, Ctl* ctl, Arr bk,
+                              const SlotMap& map, const RunProg& prog, uint32_t k,
+                              const uint64_t tmask[2], Arr out, int out_slot) {
+  if (prog.n > (uint32_t)kMaxItems || k > (uint32_t)kMaxHashRun ||
+      (1u << bk.seg_log2) != kBucketCap)
+    return cudaErrorInvalidValue;
+  if (kw == 2)
+    return amp32 ? bucket_t<2, float2>(L, ctl, bk, map, prog, k, tmask, out, out_slot)
+                 : bucket_t<2, double2>(L, ctl, bk, map, prog, k, tmask, out, out_slot);
+  return amp32 ? bucket_t<1, float2>(L, ctl, bk, map, prog, k, tmask, out, out_slot)
+               : bucket_t<1, double2>(L, ctl, bk, map, prog, k, tmask, out, out_slot);
+}
 
 cudaError_t launch_slot_scatter(const Launch& L, int kw, bool amp32, Ctl* ctl, Arr in, int in_slot,
                                 const OpList& ops, const SlotMap& map, void* amp, uint8_t* pres) {
