@@ -1662,8 +1662,8 @@ void step_reads(const Gate1& g, uint64_t reads[2]) {
 // Runs held steps that are not addressed.  In pieces the sorted form allows
 // (distinct targets no other step of the piece reads, no phase, no fold) where
 // sorting them pays; what is left, on a state too wide to address, in pieces
-// of up to kMaxHashRun targets over hash buckets when at least three launches
-// are saved; else step by step.
+// of up to kMaxHashRun targets over hash buckets (two launches) in place of at
+// least five; else step by step.
 sqs_status run_pieces(sqs_state* st, const std::vector<sqs_state::Held>& run, bool wide) {
   sqs_status s = SQS_OK;
   auto tbit = [](const Gate1& g, uint64_t t[2]) {
@@ -1690,7 +1690,7 @@ sqs_status run_pieces(sqs_state* st, const std::vector<sqs_state::Held>& run, bo
         launches += h[m].g.no_partners || h[m].g.fold_sign ? 1.0 : 2.0;
       }
       bool taken = false;
-      if (wide && m >= 2 && launches >= 3.0)
+      if (wide && m >= 2 && launches >= 5.0)
         s = run_bucketed(st, std::vector<sqs_state::Held>(h, h + m), tm, taken);
       if (s == SQS_OK && !taken) alone(h, m);
       if (m < n && h[m].after_phase && s == SQS_OK) st->pending.push_back(h[m].phase);
