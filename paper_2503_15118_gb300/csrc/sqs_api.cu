@@ -2623,7 +2623,7 @@ sqs_status sort_copy(sqs_state* st, uint64_t n, const uint64_t keep[2], Store** 
   const uint64_t tilesN = std::max<uint64_t>(1, (n + tile - 1) / tile);
   unsigned int *hist, *part;
   unsigned long long* n_dev;
-  sqs_status s = sort_scratch(st, std::max(tiles0, tilesN), hist, part, n_dev, rb);
+  sqs_status s = sort_scratch(st, std::max(tiles0, 2 * tilesN), hist, part, n_dev, rb);
   if (s != SQS_OK) return s;
   if ((st->bk.cap < n && !ensure_store(st, st->bk, n)) ||
       (st->alt.cap < n && !ensure_store(st, st->alt, n)))
@@ -2641,7 +2641,17 @@ sqs_status sort_copy(sqs_state* st, uint64_t n, const uint64_t keep[2], Store** 
   const uint32_t npass = (uint32_t)shifts.size();
   cudaError_t e = cudaSuccess;
   if (timed) tune_begin(st, tkey);
-  for (uint32_t p = 0; p < npass && e == cudaSuccess; ++p) {
+  const bool small = rb == 8 && npass <= 16 && n <= sqs::small_sort_max(st->sm_count);
+  if (small) {
+    // One launch for all passes: latency, not bandwidth, bounds a small sort.
+    for (Store* b : buf) b->set_dense();
+    Traced tr(st, SQS_K_SORT);
+    e = sqs::launch_rsort_small(launch_of(st, n), st->kw, st->amp32, st->ctl, src, n,
+                                buf[0]->view(), buf[1]->view(), shifts.data(), npass, hist, part,
+                                n_dev, whole ? nullptr : cm, t_none);
+    n_ptr = n_dev;
+  }
+  for (uint32_t p = 0; !small && p < npass && e == cudaSuccess; ++p) {
     Store& dst = *buf[p & 1];
     dst.set_dense();
     Traced tr(st, SQS_K_SORT);
@@ -3337,9 +3347,8 @@ sqs_status sqs_export(sqs_state* st, uint64_t* keys, double* amps, uint64_t cap,
       e = cudaMemcpyAsync(amps, src->amp, cnt * 16, cudaMemcpyDeviceToHost, st->stream);
     }
   }
-  if (e == cudaSuccess) e = cudaStreamSynchronize(st->stream);
   if (e != cudaSuccess) return cuda_fail(st, e, "export");
-  return SQS_OK;
+  return sync_ctl(st);  // waits; a sort that gave up is an error, not an export
 }
 
 sqs_status sqs_import(sqs_state* st, const uint64_t* keys, const double* amps, uint64_t n) {

@@ -273,6 +273,16 @@ cudaError_t launch_rsort_pass(const Launch& L, int kw, bool amp32, Ctl* ctl, Arr
                               uint32_t shift, unsigned int* hist, unsigned int* part,
                               unsigned long long* n_dev, Arr out,
                               const uint64_t* clear_mask = nullptr, int radix_bits = 8);
+// A whole sort in one cooperative launch, for n <= small_sort_max() branches:
+// n_pass 8-bit digits at shifts[] of the key with the bits of clear_mask cleared
+// (null: with bit t deleted), from `in` (dense or segmented) by turns into buf0
+// (first) and buf1, both of at least n slots.  hist holds 2^9 counters per tile
+// of sort_tile() branches, bar one; *n_dev receives n.
+uint64_t small_sort_max(int sm_count);
+cudaError_t launch_rsort_small(const Launch& L, int kw, bool amp32, Ctl* ctl, Arr in, uint64_t n,
+                               Arr buf0, Arr buf1, const uint32_t* shifts, uint32_t n_pass,
+                               unsigned int* hist, unsigned int* bar, unsigned long long* n_dev,
+                               const uint64_t* clear_mask, uint32_t t);
 // Combines neighbours of the sorted array `in` (*n_ptr branches): chunk c of
 // 2^sort_merge_chunk_log2() branches becomes segment c of `out` (twice the
 // size).  Adds the count into cnt[out_slot], clears cnt[(out_slot + 1) & 3].

@@ -315,6 +315,198 @@ __global__ void __launch_bounds__(kSortThreads)
   }
 }
 
+// A whole LSD sort in one cooperative launch, for states that fit one tile per
+// SM.  Every pass of the kernels above is four launches, each a few microseconds
+// of latency at these sizes.  Here CTA t keeps tile t's branches in registers from its
+// histogram to its scatter, and a grid barrier -- bounded: after kGridWait polls
+// it records an error and the grid returns -- separates the phases.  An export
+// of 65536 one-word branches (8 passes) takes 140 us in place of 276, of 4000
+// branches 130 in place of 252; past one tile per SM the passes above are
+// bound by their traffic.  Same order as the passes above
+// (stable; a segmented input is laid out dense in segment order first).
+constexpr uint32_t kGridWait = 1u << 21;  // about a second
+constexpr int kSmallPasses = 16;  // 128 bits by 8
+struct SmallSort {
+  uint32_t n_pass;
+  uint32_t shift[kSmallPasses];
+};
+
+// All CTAs of the grid; false (for every thread) when the wait ran out.
+__device__ __forceinline__ bool grid_barrier(unsigned int* bar, unsigned int& phase,
+                                             unsigned int* ok) {
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    ++phase;
+    const unsigned int target = phase * gridDim.x;
+    __threadfence();
+    atomicAdd(bar, 1u);
+    uint32_t it = 0;
+    unsigned int seen;
+    do {
+      asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(seen) : "l"(bar) : "memory");
+    } while (seen < target && ++it < kGridWait);
+    __threadfence();
+    *ok = seen >= target;
+  }
+  __syncthreads();
+  return *ok != 0u;
+}
+
+template <int KW, class AT>
+__global__ void __launch_bounds__(kSortThreads)
+    k_rsort_small(Ctl* ctl, Arr in, uint64_t n, Arr buf0, Arr buf1, const SmallSort passes,
+                  unsigned int* hist, unsigned int* bar, unsigned long long* n_dev, uint32_t seq,
+                  uint64_t cm0, uint64_t cm1, uint32_t t) {
+  typedef typename KT<KW>::T K;
+  constexpr uint32_t R = 256;
+  const K cm = mk<KW>(cm0, cm1);
+  extern __shared__ __align__(16) unsigned char smem[];
+  K* skey = (K*)smem;
+  AT* samp = (AT*)(smem + (size_t)kSortTile * sizeof(K));
+  unsigned int* whist = (unsigned int*)(samp + kSortTile);  // [kSortWarps][R]
+  unsigned int* tbase = whist + kSortWarps * R;
+  unsigned int* gofs = tbase + R;
+  uint16_t* sdig = (uint16_t*)(gofs + R);
+  __shared__ unsigned int wsum[kSortWarps], wsum2[kSortWarps], ok, carry;
+  const unsigned int lane = threadIdx.x & 31u, warp = threadIdx.x >> 5;
+  const unsigned int lt = (1u << lane) - 1u;
+  const uint32_t T = gridDim.x;
+  unsigned int phase = 0;
+  if (blockIdx.x == 0 && threadIdx.x == 0) *n_dev = n;
+  auto give_up = [&] {
+    if (threadIdx.x == 0) raise_err(ctl, kErrProbe, seq, 0);
+  };
+  const Arr* src = &in;
+  if (in.seg_cnt) {
+    // Dense copy into the buffer the first pass does not write.
+    const Arr& dst = buf1;
+    if (threadIdx.x == 0) carry = 0u;
+    __syncthreads();
+    for (uint32_t s0 = 0; s0 < in.n_seg; s0 += kSortThreads) {
+      const uint32_t sg = s0 + threadIdx.x;
+      const unsigned int c = sg < in.n_seg ? in.seg_cnt[sg] : 0u;
+      unsigned int incl = c;
+      for (int o = 1; o < 32; o <<= 1) {
+        const unsigned int y = __shfl_up_sync(0xffffffffu, incl, o);
+        if (lane >= (unsigned int)o) incl += y;
+      }
+      if (lane == 31u) wsum[warp] = incl;
+      __syncthreads();
+      unsigned int pre = carry + incl - c;
+      for (unsigned int w = 0; w < warp; ++w) pre += wsum[w];
+      gofs[threadIdx.x] = pre;   // first dense position of the segment
+      tbase[threadIdx.x] = c;
+      __syncthreads();
+      if (threadIdx.x == kSortThreads - 1) carry = pre + c;
+      // This CTA's segments of the chunk: s0 is a multiple of the chunk, so
+      // segment sg belongs to CTA sg mod T.
+      for (uint32_t q = (blockIdx.x + T - s0 % T) % T; q < kSortThreads; q += T) {
+        const uint32_t m = tbase[q];
+        const uint64_t from = (uint64_t)(s0 + q) << in.seg_log2;
+        for (uint32_t j = threadIdx.x; j < m; j += kSortThreads) {
+          st_key<KW>(dst, gofs[q] + j, ld_key<KW>(in, from + j));
+          ((AT*)dst.amp)[gofs[q] + j] = ((const AT*)in.amp)[from + j];
+        }
+      }
+      __syncthreads();
+    }
+    if (!grid_barrier(bar, phase, &ok)) return give_up();
+    src = &buf1;
+  }
+  const uint64_t base = (uint64_t)blockIdx.x * kSortTile;
+  const uint32_t lim = base < n ? (uint32_t)umin64(n - base, (uint64_t)kSortTile) : 0u;
+  for (uint32_t p = 0; p < passes.n_pass; ++p) {
+    const uint32_t shift = passes.shift[p];
+    const Arr& dst = (p & 1u) ? buf1 : buf0;
+    unsigned int* const h = hist + (size_t)(p & 1u) * T * R;
+    for (uint32_t i = threadIdx.x; i < kSortWarps * R; i += blockDim.x) whist[i] = 0u;
+    __syncthreads();
+    K k[kSortItems];
+    AT a[kSortItems];
+    uint32_t d[kSortItems], rk[kSortItems];
+#pragma unroll
+    for (int r = 0; r < kSortItems; ++r) {
+      const uint32_t j = warp * (32u * kSortItems) + (uint32_t)r * 32u + lane;
+      if (j < lim) {
+        k[r] = ld_key<KW>(*src, base + j);
+        a[r] = ((const AT*)src->amp)[base + j];
+      }
+    }
+#pragma unroll
+    for (int r = 0; r < kSortItems; ++r) {
+      const uint32_t j = warp * (32u * kSortItems) + (uint32_t)r * 32u + lane;
+      const bool live = j < lim;
+      // Dead lanes get a value no live lane has, so they match only themselves.
+      d[r] = live ? digit_of<8>(k[r], t, shift, cm) : R + lane;
+      const unsigned int peers = __match_any_sync(0xffffffffu, d[r]);
+      unsigned int before = 0u;
+      if (live) before = whist[warp * R + d[r]];
+      __syncwarp();
+      if (live && (peers & lt) == 0u) whist[warp * R + d[r]] = before + (unsigned int)__popc(peers);
+      __syncwarp();
+      rk[r] = before + (unsigned int)__popc(peers & lt);
+    }
+    __syncthreads();
+    // One digit a thread: the tile's count, and the warps' places in it.
+    unsigned int mine = 0u;
+    for (int w = 0; w < kSortWarps; ++w) {
+      const unsigned int c = whist[w * R + threadIdx.x];
+      whist[w * R + threadIdx.x] = mine;
+      mine += c;
+    }
+    h[(size_t)blockIdx.x * R + threadIdx.x] = mine;
+    if (!grid_barrier(bar, phase, &ok)) return give_up();
+    unsigned int before = 0u, total = 0u;
+#pragma unroll 8
+    for (uint32_t u = 0; u < T; ++u) {
+      const unsigned int c = __ldcg(&h[(size_t)u * R + threadIdx.x]);
+      before += u < blockIdx.x ? c : 0u;
+      total += c;
+    }
+    // Exclusive scans over the digits: of the tile's counts and the totals.
+    unsigned int i1 = mine, i2 = total;
+    for (int o = 1; o < 32; o <<= 1) {
+      const unsigned int y1 = __shfl_up_sync(0xffffffffu, i1, o);
+      const unsigned int y2 = __shfl_up_sync(0xffffffffu, i2, o);
+      if (lane >= (unsigned int)o) {
+        i1 += y1;
+        i2 += y2;
+      }
+    }
+    if (lane == 31u) {
+      wsum[warp] = i1;
+      wsum2[warp] = i2;
+    }
+    __syncthreads();
+    unsigned int pre1 = i1 - mine, pre2 = i2 - total;
+    for (unsigned int w = 0; w < warp; ++w) {
+      pre1 += wsum[w];
+      pre2 += wsum2[w];
+    }
+    tbase[threadIdx.x] = pre1;
+    gofs[threadIdx.x] = pre2 + before;
+    __syncthreads();
+#pragma unroll
+    for (int r = 0; r < kSortItems; ++r) {
+      if (d[r] < R) {
+        const uint32_t lp = tbase[d[r]] + whist[warp * R + d[r]] + rk[r];
+        skey[lp] = k[r];
+        samp[lp] = a[r];
+        sdig[lp] = (uint16_t)d[r];
+      }
+    }
+    __syncthreads();
+    for (uint32_t i = threadIdx.x; i < lim; i += blockDim.x) {
+      const uint32_t dg = sdig[i];
+      const uint64_t pos = (uint64_t)gofs[dg] + (i - tbase[dg]);
+      st_key<KW>(dst, pos, skey[i]);
+      ((AT*)dst.amp)[pos] = samp[i];
+    }
+    if (p + 1 < passes.n_pass && !grid_barrier(bar, phase, &ok)) return give_up();
+    src = &dst;
+  }
+}
+
 // The merge over the sorted array: the first member of each pair class
 // computes both children (Eq. of the 2x2 step, Sec. II.D.2) from itself and
 // its neighbour when the neighbour shares the class; chunk c of 2^12 sorted
@@ -496,6 +688,44 @@ cudaError_t launch_rsort_pass(const Launch& L, int kw, bool amp32, Ctl* ctl, Arr
     default:
       return cudaErrorInvalidValue;
   }
+}
+
+uint64_t small_sort_max(int sm_count) { return (uint64_t)sm_count * kSortTile; }
+
+template <int KW, class AT>
+static cudaError_t small_t(const Launch& L, Ctl* ctl, Arr in, uint64_t n, Arr buf0, Arr buf1,
+                           const uint32_t* shifts, uint32_t n_pass, unsigned int* hist,
+                           unsigned int* bar, unsigned long long* n_dev,
+                           const uint64_t* clear_mask, uint32_t t) {
+  const size_t smem = scatter_smem<KW, AT, 8>();
+  static std::atomic<unsigned long long> configured{0};  // opt-in above 48 KB, per device
+  cudaError_t e = ensure_smem_optin((const void*)k_rsort_small<KW, AT>, smem, configured);
+  if (e != cudaSuccess) return e;
+  e = cudaMemsetAsync(bar, 0, sizeof(unsigned int), L.stream);
+  if (e != cudaSuccess) return e;
+  SmallSort ps;
+  std::memset(&ps, 0, sizeof(ps));
+  ps.n_pass = n_pass;
+  for (uint32_t p = 0; p < n_pass; ++p) ps.shift[p] = shifts[p];
+  uint64_t cm0 = clear_mask ? clear_mask[0] : 0ull, cm1 = clear_mask ? clear_mask[1] : 0ull;
+  uint32_t seq = L.seq;
+  void* args[] = {&ctl, &in, &n, &buf0, &buf1, &ps, &hist, &bar, &n_dev, &seq, &cm0, &cm1, &t};
+  const uint64_t grid = (n + kSortTile - 1) / kSortTile;
+  return cudaLaunchCooperativeKernel((const void*)k_rsort_small<KW, AT>,
+                                     dim3((unsigned)(grid ? grid : 1)), dim3(kSortThreads), args,
+                                     smem, L.stream);
+}
+
+cudaError_t launch_rsort_small(const Launch& L, int kw, bool amp32, Ctl* ctl, Arr in, uint64_t n,
+                               Arr buf0, Arr buf1, const uint32_t* shifts, uint32_t n_pass,
+                               unsigned int* hist, unsigned int* bar, unsigned long long* n_dev,
+                               const uint64_t* clear_mask, uint32_t t) {
+  if (n_pass == 0 || n_pass > (uint32_t)kSmallPasses || n > small_sort_max(L.sm_count))
+    return cudaErrorInvalidValue;
+#define SQS_S(KW_, AT_) \
+  small_t<KW_, AT_>(L, ctl, in, n, buf0, buf1, shifts, n_pass, hist, bar, n_dev, clear_mask, t)
+  return SQS_SORT_DISPATCH(kw, amp32, SQS_S);
+#undef SQS_S
 }
 
 cudaError_t launch_rsort_merge(const Launch& L, int kw, bool amp32, Ctl* ctl, Arr in,
