@@ -756,6 +756,20 @@ sqs_status run_binned(sqs_state* st, const Gate1& g, uint64_t B1, int64_t rec_id
   return SQS_OK;
 }
 
+// After a merge into st->alt: the record of its counts, the buffers' roles, the
+// bound.
+sqs_status finish_merge(sqs_state* st, const Gate1& g, int out_slot, int64_t rec_idx) {
+  if (rec_idx >= 0) {
+    const cudaError_t e = sqs::launch_record(launch_of(st, 1), st->ctl, st->cur_slot, out_slot,
+                                             st->rec_dev + 2 * (size_t)rec_idx);
+    if (e != cudaSuccess) return cuda_fail(st, e, "record launch");
+  }
+  std::swap(st->cur, st->alt);
+  st->cur_slot = out_slot;
+  st->ub = bound_after(st, std::min(vary_cap(st, g), 2 * st->ub));
+  return SQS_OK;
+}
+
 // One interference step: fused pending run + partition + pair.  est_in < 0:
 // buckets sized from the hard bound st->ub (exact mode); otherwise from the
 // predicted input count est_in with a 20% margin (learned mode).
@@ -797,6 +811,25 @@ sqs_status run_hashed(sqs_state* st, const Gate1& g, double est_in, int64_t rec_
     return run_binned(st, g, B1, rec_idx);
   }
   st->stats.steps_hash++;
+  if (est_in < 0 && want <= sqs::merge_small_max()) {
+    // About 512 branches a CTA while the cluster can grow (16 CTAs at most).
+    uint32_t ctas = 1;
+    while (ctas < 16 && (uint64_t)ctas * (kBucketFill / 2) < want) ctas *= 2;
+    const uint64_t slots = (uint64_t)ctas << kSegLog2;
+    const bool fixed = st->captured || st->capturing;  // buffers stay where they are
+    if (st->alt.cap >= slots || (!fixed && ensure_store(st, st->alt, slots))) {
+      st->alt.set_segments(kSegLog2, ctas);
+      const int out_slot = (st->cur_slot + 1) & 3;
+      cudaError_t e;
+      {
+        Traced tr(st, SQS_K_PAIR);
+        e = sqs::launch_merge_small(launch_of(st, want), st->kw, st->amp32, st->ctl,
+                                    st->cur.view(), st->cur_slot, L, g, st->alt.view(), out_slot);
+      }
+      if (e != cudaSuccess) return cuda_fail(st, e, "merge launch");
+      return finish_merge(st, g, out_slot, rec_idx);
+    }
+  }
   // Learned mode grows buffers straight to the predicted peak (grow_hint_b),
   // or to this step's size when a predicted peak cannot be allocated.
   const uint64_t Bcap = std::max(B, st->grow_hint_b);
@@ -828,15 +861,7 @@ sqs_status run_hashed(sqs_state* st, const Gate1& g, double est_in, int64_t rec_
                          st->alt.view(), out_slot);
   }
   if (e != cudaSuccess) return cuda_fail(st, e, "pair launch");
-  if (rec_idx >= 0) {
-    e = sqs::launch_record(launch_of(st, 1), st->ctl, st->cur_slot, out_slot,
-                           st->rec_dev + 2 * (size_t)rec_idx);
-    if (e != cudaSuccess) return cuda_fail(st, e, "record launch");
-  }
-  std::swap(st->cur, st->alt);
-  st->cur_slot = out_slot;
-  st->ub = bound_after(st, std::min(vary_cap(st, g), 2 * st->ub));
-  return SQS_OK;
+  return finish_merge(st, g, out_slot, rec_idx);
 }
 
 // Digit windows of the radix-sort merge: start positions (in the pair-class
@@ -1436,6 +1461,24 @@ bool slots_pay(const sqs_state* st, const std::vector<sqs_state::Held>& run, int
   return fused < alone;
 }
 
+// Makes room for `want` slots of addressed runs.
+bool ensure_slots(sqs_state* st, uint64_t want) {
+  if (st->slot_cap >= want) return true;
+  dfree(st, st->slot_amp);
+  dfree(st, st->slot_pres);
+  st->slot_amp = dalloc(st, want * amp_bytes(st));
+  st->slot_pres = (uint8_t*)dalloc(st, want);
+  st->slot_cap = st->slot_amp && st->slot_pres ? want : 0;
+  if (!st->slot_cap) {
+    dfree(st, st->slot_amp);
+    dfree(st, st->slot_pres);
+    st->slot_amp = st->slot_pres = nullptr;
+    return false;
+  }
+  cudaMemsetAsync(st->slot_pres, 0, want, st->stream);
+  return true;
+}
+
 // Slot layout and items of a run (st->run_prog): the targets in key order in
 // the low bits of the slot, then the other bits of `vary` (none: a bucketed
 // run, whose slots number a group's members and whose predicates on other bits
@@ -1523,21 +1566,9 @@ sqs_status run_slots(sqs_state* st, const std::vector<sqs_state::Held>& run,
   prog.area_log2 = sqs::run_area_log2(k);
   prog.n_areas = bits > prog.area_log2 ? 1u << (bits - prog.area_log2) : 1u;
   const uint64_t want = (uint64_t)prog.n_areas << prog.area_log2;
-  if (st->slot_cap < want) {
-    dfree(st, st->slot_amp);
-    dfree(st, st->slot_pres);
-    st->slot_amp = dalloc(st, want * amp_bytes(st));
-    st->slot_pres = (uint8_t*)dalloc(st, want);
-    st->slot_cap = st->slot_amp && st->slot_pres ? want : 0;
-    if (!st->slot_cap) {
-      dfree(st, st->slot_amp);
-      dfree(st, st->slot_pres);
-      st->slot_amp = st->slot_pres = nullptr;
-      return st->sticky = fail(st, SQS_ERR_OOM, "cannot allocate %llu slots",
-                               (unsigned long long)want);
-    }
-    cudaMemsetAsync(st->slot_pres, 0, want, st->stream);
-  }
+  if (!ensure_slots(st, want))
+    return st->sticky = fail(st, SQS_ERR_OOM, "cannot allocate %llu slots",
+                             (unsigned long long)want);
   const uint64_t grown = st->ub > (slots >> k) ? slots : st->ub << k;
   if (st->alt.cap < grown && !ensure_store(st, st->alt, grown))
     return st->sticky = fail(st, SQS_ERR_OOM, "cannot allocate %llu branches",
@@ -1561,9 +1592,11 @@ sqs_status run_slots(sqs_state* st, const std::vector<sqs_state::Held>& run,
   if (e != cudaSuccess) return cuda_fail(st, e, "slot run launch");
   std::swap(st->cur, st->alt);
   st->cur_slot = out_slot;
-  st->ub = grown;
-  st->stats.runs_fused++;
-  st->stats.steps_fused += run.size();
+  st->ub = bound_after(st, grown);
+  if (!st->capturing) {  // nothing runs during a capture
+    st->stats.runs_fused++;
+    st->stats.steps_fused += run.size();
+  }
   return SQS_OK;
 }
 
@@ -1719,9 +1752,9 @@ sqs_status run_pieces(sqs_state* st, const std::vector<sqs_state::Held>& run, bo
         pr[w] |= reads[w];
       }
     }
-    if (gates.size() >= 2 && fuse_pays(st, gates)) {
+    if (gates.size() >= 2 && !st->capturing && fuse_pays(st, gates)) {
       s = run_group(st, gates);
-    } else if (wide) {
+    } else if (wide && !st->capturing) {
       end = run.size();  // bucketed pieces may go on past it
       bucketed(&run[from], end - from);
     } else {
@@ -1751,14 +1784,16 @@ sqs_status flush_run(sqs_state* st) {
   const int slot_bits = bits_set(vary);
   bool addressed = run.size() >= 2 && slot_bits <= (int)sqs::kMaxSlotBits &&
                    slots_pay(st, run, slot_bits);
-  if (addressed && st->captured) {
-    // The output must fit where the graph expects it (run_slots would move it).
-    const uint64_t k = (uint64_t)bits_set(tmask);
+  if (addressed && (st->captured || st->capturing)) {
+    // Output and slots must fit where the graph has them (run_slots would move
+    // them).
+    const int k = bits_set(tmask);
     auto fits = [&] {
-      return std::min<double>(std::ldexp((double)st->ub, (int)k), std::ldexp(1.0, slot_bits)) <=
-             (double)st->alt.cap;
+      const double grown = std::min(std::ldexp((double)st->ub, k), std::ldexp(1.0, slot_bits));
+      return grown <= (double)st->alt.cap &&
+             std::ldexp(1.0, std::max(slot_bits, 12)) <= (double)st->slot_cap;
     };
-    if (!fits()) s = sync_bound(st);
+    if (!fits() && !st->capturing) s = sync_bound(st);
     addressed = s == SQS_OK && fits();
   }
   if (s != SQS_OK) {
@@ -1772,12 +1807,12 @@ sqs_status flush_run(sqs_state* st) {
   return s;
 }
 
-// Fused runs wait for the device (the group count sizes the output), so a
-// graph capture runs every step alone.
+// In a graph capture only addressed runs fuse: the others wait for the device
+// (the group count, or the exact count, sizes their output).
 bool fusing(const sqs_state* st) {
   return !(st->flags & (SQS_FUSE_OFF | SQS_MERGE_PLAIN | SQS_MERGE_HASH | SQS_MERGE_SORT |
                         SQS_MERGE_CLUSTER)) &&
-         !st->recording && !st->capturing;
+         !st->recording;
 }
 
 // Holds an interference step in the open run, or closes the run and opens a
@@ -3537,6 +3572,16 @@ sqs_status sqs_capture_begin(sqs_state* st, uint64_t static_bound) {
   if (!ensure_store(st, st->cur, cap) || !ensure_store(st, st->alt, cap) ||
       !ensure_store(st, st->bk, B << kBucketLog2))
     return st->sticky = fail(st, SQS_ERR_OOM, "cannot size buffers for the capture");
+  // Slots for addressed runs: up to 2^20 (a circuit of 20 qubits), or eight per
+  // branch of the bound; a run over more of them takes its steps one by one.
+  if (fusing(st) && !st->captured) {
+    uint64_t slots = 1ull << 12;
+    while (slots < (1ull << std::min(st->total_bits, sqs::kMaxSlotBits)) &&
+           slots < std::max<uint64_t>(1ull << 20, 8 * static_bound))
+      slots <<= 1;
+    if (!ensure_slots(st, slots))
+      return st->sticky = fail(st, SQS_ERR_OOM, "cannot size buffers for the capture");
+  }
   s = sqs_state_reset(st);  // the state the graph starts from, now
   if (s != SQS_OK) return s;
   st->entry_snap = take_snap(st);

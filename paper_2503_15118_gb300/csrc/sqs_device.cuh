@@ -295,6 +295,15 @@ __device__ __forceinline__ void for_units(const Arr& in, uint64_t n_dense, uint3
   const uint32_t per_seg = ((1u << in.seg_log2) + unit - 1) / unit;
   const uint32_t l = log2_pow2(per_seg);
   const uint64_t units = (uint64_t)in.n_seg * per_seg;
+  if (units <= gridDim.x) {  // at most one unit a CTA: no list, one load
+    if (blockIdx.x >= units) return;
+    const uint64_t v = spread_visit(blockIdx.x, l);
+    const uint32_t sg = (uint32_t)(v / per_seg);
+    const uint32_t off = (uint32_t)(v - (uint64_t)sg * per_seg) * unit;
+    const uint32_t cnt = in.seg_cnt[sg];
+    if (off < cnt) body(((uint64_t)sg << in.seg_log2) + off, cnt - off < unit ? cnt - off : unit);
+    return;
+  }
   for (uint64_t k0 = 0; blockIdx.x + k0 * gridDim.x < units; k0 += blockDim.x) {
     if (threadIdx.x == 0) *n_list = 0u;
     __syncthreads();
@@ -362,7 +371,14 @@ __device__ __forceinline__ K arith_op(const DevOp& op, K k) {
   } else {
     const uint64_t a = get_field(k, op.src_off, op.src_w);
     const uint64_t b = get_field(k, op.src2_off, op.src2_w);
-    r = op.kind == OP_MUL_ADD ? d + a * b : d ^ (b ? a / b : 0ull);
+    // (A 64-bit division is a routine of some hundred instructions; fields of
+    // up to 32 bits take the 32-bit one.)
+    if (op.kind == OP_MUL_ADD)
+      r = d + a * b;
+    else if (op.src_w <= 32u && op.src2_w <= 32u)
+      r = d ^ (uint64_t)((uint32_t)b ? (uint32_t)a / (uint32_t)b : 0u);
+    else
+      r = d ^ (b ? a / b : 0ull);
   }
   return set_field<K>(k, op.dst_off, op.dst_w, r);
 }
@@ -430,20 +446,28 @@ __device__ __forceinline__ void apply_ops_n(uint32_t n_ops, const DevOp* ops, co
   uint32_t idx[NI];
 #pragma unroll
   for (int q = 0; q < NI; ++q) idx[q] = 0;
+  if (n_ops == 0u) return;
+  // The next operation's kind, predicate and mask are read while the current
+  // one is applied: over few branches a run is the latency of its operations.
+  uint32_t kind = ops[0].kind;
+  K pm = mk<KW>(ops[0].pmask[0], ops[0].pmask[1]);
+  K pv = mk<KW>(ops[0].pval[0], ops[0].pval[1]);
+  K xm = mk<KW>(ops[0].xmask[0], ops[0].xmask[1]);
 #pragma unroll 1
   for (uint32_t o = 0; o < n_ops; ++o) {
     const DevOp& op = ops[o];
-    const uint32_t kind = op.kind;
-    const K pm = mk<KW>(op.pmask[0], op.pmask[1]);
-    const K pv = mk<KW>(op.pval[0], op.pval[1]);
+    const DevOp& nx = ops[o + 1u < n_ops ? o + 1u : o];
+    const uint32_t kind_nx = nx.kind;
+    const K pm_nx = mk<KW>(nx.pmask[0], nx.pmask[1]);
+    const K pv_nx = mk<KW>(nx.pval[0], nx.pval[1]);
+    const K xm_nx = mk<KW>(nx.xmask[0], nx.xmask[1]);
     if (kind == OP_XOR) {
-      const K xm = mk<KW>(op.xmask[0], op.xmask[1]);
 #pragma unroll
       for (int q = 0; q < NI; ++q)
         if ((k[q] & pm) == pv) k[q] ^= xm;
     } else if (kind == OP_MUL || kind == OP_MUL_XOR) {
       const uint32_t sel = op.sel_bit, sh = op.shift;
-      const K xm = kind == OP_MUL_XOR ? mk<KW>(op.xmask[0], op.xmask[1]) : (K)0;
+      // (An OP_MUL's mask is zero.)
 #pragma unroll
       for (int q = 0; q < NI; ++q) {
         if ((k[q] & pm) == pv) {
@@ -517,20 +541,36 @@ __device__ __forceinline__ void apply_ops_n(uint32_t n_ops, const DevOp* ops, co
       for (int q = 0; q < NI; ++q)
         if ((k[q] & pm) == pv) k[q] = arith_op(op, k[q]);
     }
+    kind = kind_nx;
+    pm = pm_nx;
+    pv = pv_nx;
+    xm = xm_nx;
   }
+}
+
+// A kernel parameter's address as a generic one the compiler cannot trace back
+// to the parameter bank.  Read by lane-varying index from the bank itself, every
+// distinct address of a warp is a turn of its own (29 KB of operations and
+// factors: 5 us at the start of a kernel); through the generic address it is an
+// ordinary coalesced load.
+template <class T>
+__device__ __forceinline__ const T* param_ptr(const T* p) {
+  asm volatile("" : "+l"(p));
+  return p;
 }
 
 // Copies the launch's operations and factor table into shared memory: the
 // per-branch loop then reads them with broadcast shared loads instead of
 // indexed parameter-space loads.
-template <class AT>
-__device__ __forceinline__ void load_ops(const OpList& L, DevOp* ops, AT* tab) {
+template <class AT, class LT>
+__device__ __forceinline__ void load_ops(const LT& L, DevOp* ops, AT* tab) {
   static_assert(sizeof(DevOp) % 8 == 0, "DevOp copied as 8-byte words");
-  const uint64_t* src = (const uint64_t*)L.op;
+  const uint64_t* src = param_ptr((const uint64_t*)L.op);
+  const double2* factors = param_ptr(L.tab);
   uint64_t* dst = (uint64_t*)ops;
   const uint32_t words = L.n * (uint32_t)(sizeof(DevOp) / 8);
   for (uint32_t i = threadIdx.x; i < words; i += blockDim.x) dst[i] = src[i];
-  for (uint32_t i = threadIdx.x; i < L.n_tab; i += blockDim.x) to_amp(tab[i], L.tab[i]);
+  for (uint32_t i = threadIdx.x; i < L.n_tab; i += blockDim.x) to_amp(tab[i], factors[i]);
   __syncthreads();
 }
 
@@ -569,6 +609,37 @@ __device__ __forceinline__ bool mbar_try_wait(uint64_t* bar, uint32_t parity) {
 }
 
 constexpr int kStreamThreads = 256;
+
+// ---- programmatic dependent launch --------------------------------------------
+// A kernel launched by launch_next() may start while its predecessor on the
+// stream still runs: its launch, parameters and operation list (copied to
+// shared memory) then cost nothing.  pdl_next() at a kernel's start allows that
+// to its successor; pdl_wait() returns once the predecessor is complete and its
+// writes are visible, and comes before any access to global memory.
+__device__ __forceinline__ void pdl_next() {
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
+template <class... P, class... A>
+inline cudaError_t launch_next(void (*kern)(P...), uint64_t grid, int threads, size_t smem,
+                               cudaStream_t stream, const A&... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)grid);
+  cfg.blockDim = dim3((unsigned)threads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = stream;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  // By pointer: an operation list is 29 KB, copied once by the launch itself.
+  return [&](const P&... p) {
+    void* ptr[] = {(void*)&p...};
+    return cudaLaunchKernelExC(&cfg, (const void*)kern, ptr);
+  }(args...);
+}
 
 // ---------------------------------------------------------------------------
 // The 2x2 of one merge step on a pair class: children (o0, o1) of the

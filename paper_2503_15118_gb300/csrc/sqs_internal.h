@@ -53,19 +53,65 @@ struct DevOp {
   double eps, eps2;            // OP_PRUNE
 };
 
-constexpr int kMaxOps = 64;      // fused operations per launch
+constexpr int kMaxOps = 96;      // fused operations per launch (a parameter of 29 KB; 32 is the limit)
 constexpr int kTabEntries = 1024;  // folded factor entries per launch
 
-struct OpList {
+template <int N, int T>
+struct OpListOf {
+  static constexpr int kOps = N, kTab = T;
   uint32_t n;
   uint32_t touches_keys;  // some op changes keys
   uint32_t touches_amps;  // some op changes amplitudes
   uint32_t drops;         // some op may drop branches (OP_PRUNE)
   uint32_t n_tab;         // used entries of tab
   uint32_t pad[3];
-  DevOp op[kMaxOps];
-  double2 tab[kTabEntries];
+  DevOp op[N];
+  double2 tab[T];
 };
+typedef OpListOf<kMaxOps, kTabEntries> OpList;
+// The operations between two interference steps are a few as a rule.  A list of
+// at most 12 with 64 factors travels as a kernel parameter of 3 KB in place of
+// 29 KB, with shared tables to match: a 20-qubit circuit (20 launches) takes
+// 308 us in place of 319, a 59-qubit one on 2^19 branches 570 in place of 579.
+typedef OpListOf<12, 64> OpListSmall;
+inline bool fits_small(const OpList& L) {
+  return L.n <= (uint32_t)OpListSmall::kOps && L.n_tab <= (uint32_t)OpListSmall::kTab;
+}
+inline void copy_small(const OpList& L, OpListSmall& s) {
+  s.n = L.n;
+  s.touches_keys = L.touches_keys;
+  s.touches_amps = L.touches_amps;
+  s.drops = L.drops;
+  s.n_tab = L.n_tab;
+  for (uint32_t i = 0; i < L.n; ++i) s.op[i] = L.op[i];
+  for (uint32_t i = 0; i < L.n_tab; ++i) s.tab[i] = L.tab[i];
+}
+
+// The same run on bit planes (sqs_planes.cu): per operation, its predicate as a
+// list of planes (bit 7 set: the bit must be 0), and fields as first planes.
+struct PlaneOp {
+  uint64_t constant;
+  uint16_t ctrl;  // first predicate entry
+  uint16_t dst;   // OP_XOR: first of w entries of planes to flip; OP_MUL_XOR: the bit;
+                  // fields: first bit; OP_TABLE: first table entry
+  uint16_t src;
+  uint8_t kind, n_ctrl, w, src_w;  // OP_TABLE: w index bits
+  uint8_t sel, shift;              // OP_MUL*: selector bit (128: none), index bit
+  uint8_t pad[4];
+};
+static_assert(sizeof(PlaneOp) == 24, "copied as words");
+constexpr int kPlaneIdx = 10;    // bits of one factor index
+constexpr int kPlaneCtrl = 512;  // predicate bits of a list
+template <int T>
+struct PlaneListOf {
+  static constexpr int kTab = T;
+  uint32_t n, n_ctrl, n_tab, bits, touches_keys, pad;
+  PlaneOp op[kMaxOps];
+  uint8_t ctrl[kPlaneCtrl];
+  double2 tab[T];
+};
+typedef PlaneListOf<kTabEntries> PlaneList;
+typedef PlaneListOf<64> PlaneListSmall;
 
 // ---------------------------------------------------------------------------
 // Device memory views.
@@ -226,6 +272,10 @@ cudaError_t launch_table_bits(cudaStream_t s, int sm_count, const void* t, uint6
 cudaError_t launch_init(const Launch& L, Ctl* ctl, Arr a, int slot, bool amp32);
 cudaError_t launch_apply_inplace(const Launch& L, int kw, bool amp32, Ctl* ctl, Arr a, int slot,
                                  const OpList& ops);
+// The list on planes (false: not possible), and the in-place pass over it.
+bool plane_list(const OpList& L, uint32_t total_bits, PlaneList& p);
+cudaError_t launch_apply_planes(const Launch& L, int kw, bool amp32, Ctl* ctl, Arr a, int slot,
+                                const PlaneList& ops);
 // Streams `in` through the run into a segmented `out` (one segment per
 // 2^out.seg_log2 input slots), dropping pruned branches.
 cudaError_t launch_apply_compact(const Launch& L, int kw, bool amp32, Ctl* ctl, Arr in,
@@ -295,6 +345,12 @@ cudaError_t launch_rsort_merge(const Launch& L, int kw, bool amp32, Ctl* ctl, Ar
 // counter the partition zeroed (ctl->pair_next).  Resets the bucket counters.
 cudaError_t launch_pair(const Launch& L, int kw, bool amp32, Ctl* ctl, const Gate1& g, Arr bk,
                         Arr out, int out_slot);
+// The bucket merge in one launch, for at most merge_small_max() branches: a
+// cluster of out.n_seg CTAs (1, 2, 4, 8 or 16; at least one per 1024 branches),
+// whose survivors become the segments of `out` (2^12 slots each).
+uint64_t merge_small_max();
+cudaError_t launch_merge_small(const Launch& L, int kw, bool amp32, Ctl* ctl, Arr in, int in_slot,
+                               const OpList& ops, const Gate1& g, Arr out, int out_slot);
 // Interference step whose target bit is constant over the state (no pair can
 // exist): the fused run, then both children of every controlled branch,
 // appended to the dense array `out` (count in cnt[out_slot]; input chunks of

@@ -24,6 +24,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <type_traits>
+
 #include "sqs_device.cuh"
 #include "sqs_internal.h"
 
@@ -31,6 +33,8 @@ namespace sqs {
 
 template <class AT>
 __global__ void k_init(Ctl* ctl, Arr a, int slot) {
+  pdl_next();
+  pdl_wait();
   if (threadIdx.x == 0 && blockIdx.x == 0) {
     a.k0[0] = 0;
     if (a.k1) a.k1[0] = 0;
@@ -54,26 +58,28 @@ __global__ void k_init(Ctl* ctl, Arr a, int slot) {
 // memory, bounds a long run on a large state).
 constexpr int kApplyILP = 4;
 
-template <int KW, class AT, bool TK, bool TA>
+template <int KW, class AT, bool TK, bool TA, class LT, int NI>
 __global__ void __launch_bounds__(kStreamThreads)
-    k_apply_inplace(Ctl* ctl, Arr a, int slot, const __grid_constant__ OpList ops, uint32_t seq) {
+    k_apply_inplace(Ctl* ctl, Arr a, int slot, const __grid_constant__ LT ops, uint32_t seq) {
   typedef typename KT<KW>::T K;
-  __shared__ AT tab[kTabEntries];
-  __shared__ DevOp sops[kMaxOps];
-  if (ctl->err) return;
+  __shared__ AT tab[LT::kTab];
+  __shared__ DevOp sops[LT::kOps];
+  pdl_next();
   load_ops(ops, sops, tab);
+  pdl_wait();
+  if (ctl->err) return;
   const uint64_t n_dense = ctl->cnt[slot];
   if (blockIdx.x == 0 && threadIdx.x == 0) atomicMax(&ctl->peak, n_dense);
   __shared__ uint16_t ulist[kStreamThreads];
   __shared__ unsigned int n_ulist;
-  // Units of kApplyILP * blockDim slots: a slice of a segment, or of the
+  // Units of NI * blockDim slots: a slice of a segment, or of the
   // dense array.
-  for_units(a, n_dense, kApplyILP * blockDim.x, ulist, &n_ulist, [&](uint64_t base, uint32_t lim) {
-    K k[kApplyILP];
-    AT v[kApplyILP];
-    bool live[kApplyILP];
+  for_units(a, n_dense, NI * blockDim.x, ulist, &n_ulist, [&](uint64_t base, uint32_t lim) {
+    K k[NI];
+    AT v[NI];
+    bool live[NI];
 #pragma unroll
-    for (int q = 0; q < kApplyILP; ++q) {
+    for (int q = 0; q < NI; ++q) {
       const uint32_t j = q * blockDim.x + threadIdx.x;
       live[q] = j < lim;
       k[q] = 0;
@@ -83,9 +89,9 @@ __global__ void __launch_bounds__(kStreamThreads)
         if (TA) v[q] = ((const AT*)a.amp)[base + j];
       }
     }
-    apply_ops_n<KW, AT, kApplyILP>(ops.n, sops, tab, k, v, live);
+    apply_ops_n<KW, AT, NI>(ops.n, sops, tab, k, v, live);
 #pragma unroll
-    for (int q = 0; q < kApplyILP; ++q) {
+    for (int q = 0; q < NI; ++q) {
       const uint32_t j = q * blockDim.x + threadIdx.x;
       if (j < lim) {  // no operation of an in-place run drops a branch
         if (TK) st_key<KW>(a, base + j, k[q]);
@@ -104,8 +110,10 @@ __global__ void __launch_bounds__(kStreamThreads)
   __shared__ AT tab[kTabEntries];
   __shared__ DevOp sops[kMaxOps];
   __shared__ unsigned int seg_fill;
-  if (ctl->err) return;
+  pdl_next();
   load_ops(ops, sops, tab);
+  pdl_wait();
+  if (ctl->err) return;
   if (blockIdx.x == 0 && threadIdx.x == 0) {
     ctl->cnt[(out_slot + 1) & 3] = 0;
     atomicMax(&ctl->peak, ctl->cnt[in_slot]);
@@ -163,15 +171,17 @@ __global__ void __launch_bounds__(kStreamThreads)
 // bucket-counter atomics overlap instead of forming one long chain.
 constexpr int kPartILP = 4;
 
-template <int KW, class AT>
-__global__ void __launch_bounds__(kStreamThreads)
-    k_partition(Ctl* ctl, Arr in, int in_slot, const __grid_constant__ OpList ops, uint64_t clear0,
+template <int KW, class AT, class LT>
+__global__ void __launch_bounds__(kStreamThreads, KW == 1 ? 3 : 2)
+    k_partition(Ctl* ctl, Arr in, int in_slot, const __grid_constant__ LT ops, uint64_t clear0,
                 uint64_t clear1, Arr bk, uint32_t seq, uint32_t fill_target) {
   typedef typename KT<KW>::T K;
-  __shared__ AT tab[kTabEntries];
-  __shared__ DevOp sops[kMaxOps];
-  if (ctl->err) return;
+  __shared__ AT tab[LT::kTab];
+  __shared__ DevOp sops[LT::kOps];
+  pdl_next();
   load_ops(ops, sops, tab);
+  pdl_wait();
+  if (ctl->err) return;
   const uint64_t n_dense = ctl->cnt[in_slot];
   // Buckets from the device count, ceil(count / fill_target), at most the
   // host's bucket count (a bound, which may be far above the count, as
@@ -231,19 +241,154 @@ __global__ void __launch_bounds__(kStreamThreads)
   });
 }
 
+constexpr int kPairThreads = 512;
+
+// One bucket's pairing, by the whole CTA: branches [0, n) in skey / samp
+// (n <= C), partner[] all -1 and the table slot[0, 2C) cleared, a barrier
+// passed.  Pairs, 2x2, prune; the survivors go to segment b of `out`, its count
+// and the total's share are written.  Ends with a barrier.
+struct PairShared {
+  unsigned int fill, n_pairs, n_rest;
+};
+template <int KW, class AT>
+__device__ __forceinline__ void pair_bucket(Ctl* ctl, const Gate1& g, uint32_t n, uint32_t C,
+                                            typename KT<KW>::T* skey, AT* samp, unsigned int* slot,
+                                            int* partner, PairShared& sh, const Arr& out,
+                                            uint32_t b, int out_slot, uint32_t seq) {
+  typedef typename KT<KW>::T K;
+  const uint32_t S = 2u * C;
+  const K bmask = bit_mask<KW>(g.t);
+  const K cmask = mk<KW>(g.cmask[0], g.cmask[1]);
+  const K cval = mk<KW>(g.cval[0], g.cval[1]);
+  for (uint32_t i = threadIdx.x; i < n; i += blockDim.x) {
+    const K k = skey[i];
+    if ((k & cmask) != cval) continue;  // passes through unchanged
+    const K p = k & ~bmask;
+    uint32_t h = (uint32_t)khash(p) & (S - 1u);
+    // At most C entries live in 2C slots, so a free slot or the partner is
+    // always found within S probes; the bound only guards against misuse.
+    uint32_t probe = 0;
+    for (; probe < S; ++probe) {
+      const unsigned int old = atomicCAS(&slot[h], 0u, i + 1u);
+      if (old == 0u) break;
+      const uint32_t j = old - 1u;
+      if ((skey[j] & ~bmask) == p) {
+        partner[i] = (int)j;
+        partner[j] = (int)i;
+        break;
+      }
+      h = (h + 1u) & (S - 1u);
+    }
+    if (probe == S) raise_err(ctl, kErrProbe, seq, 0);
+  }
+  __syncthreads();
+
+  // Emitters: branches the controls leave alone, unpaired branches and the
+  // bit-0 member of each pair.  Listing them first (in the probe table, which
+  // is free now) keeps every lane of the arithmetic below busy.  The pairs
+  // are listed apart from the rest ([0, C) and [C, 2C) of the table), so a
+  // warp evaluates one form of the 2x2 (two members, or one): mixed, it
+  // would issue both FP64 sequences, each with part of its lanes.
+  unsigned int* emit = slot;
+  const uint32_t lane = threadIdx.x & 31u;
+  const unsigned int lt = (1u << lane) - 1u;
+  if (threadIdx.x == 0) sh.fill = sh.n_pairs = sh.n_rest = 0;
+  __syncthreads();
+  const uint32_t rounds_in = (n + blockDim.x - 1u) / blockDim.x;
+  for (uint32_t r = 0; r < rounds_in; ++r) {
+    const uint32_t i = r * blockDim.x + threadIdx.x;
+    bool ep = false, er = false;
+    if (i < n) {
+      const K k = skey[i];
+      const bool met = (k & cmask) == cval;
+      const bool kt = (k & bmask) != (K)0;
+      const bool paired = partner[i] >= 0;
+      ep = met && !kt && paired;
+      er = !met || !paired;
+    }
+    const unsigned int bp = __ballot_sync(0xffffffffu, ep);
+    const unsigned int br = __ballot_sync(0xffffffffu, er);
+    unsigned int wp = 0, wr = 0;
+    if (lane == 0) {
+      if (bp) wp = atomicAdd(&sh.n_pairs, (unsigned int)__popc(bp));
+      if (br) wr = atomicAdd(&sh.n_rest, (unsigned int)__popc(br));
+    }
+    wp = __shfl_sync(0xffffffffu, wp, 0);
+    wr = __shfl_sync(0xffffffffu, wr, 0);
+    if (ep) emit[wp + __popc(bp & lt)] = i;
+    if (er) emit[C + wr + __popc(br & lt)] = i;
+  }
+  __syncthreads();
+  const uint32_t np = sh.n_pairs;
+  const uint32_t ne = np + sh.n_rest;
+
+  const uint64_t obase = (uint64_t)b << out.seg_log2;
+  const uint32_t rounds = (ne + blockDim.x - 1u) / blockDim.x;
+  for (uint32_t r = 0; r < rounds; ++r) {
+    const uint32_t q = r * blockDim.x + threadIdx.x;
+    bool keep0 = false, keep1 = false;
+    K k0 = 0, k1 = 0;
+    AT o0, o1;
+    if (q < ne) {
+      const uint32_t i = q < np ? emit[q] : emit[C + (q - np)];
+      const K k = skey[i];
+      const AT ai = samp[i];
+      if ((k & cmask) != cval) {
+        keep0 = true;  // controls not met: the branch is unchanged
+        k0 = k;
+        o0 = ai;
+      } else {
+        const bool kt = (k & bmask) != (K)0;
+        const int j = partner[i];
+        k0 = k & ~bmask;
+        k1 = k | bmask;
+        const uint64_t av = angle_value(g, k0);
+        if (!kt)
+          children<AT>(g, av, true, ai, j >= 0, j >= 0 ? samp[j] : ai, o0, o1);
+        else
+          children<AT>(g, av, false, ai, true, ai, o0, o1);
+        keep0 = keep_amp(o0, g.eps, g.epsf, g.eps2);
+        keep1 = keep_amp(o1, g.eps, g.epsf, g.eps2);
+      }
+    }
+    const unsigned int b0 = __ballot_sync(0xffffffffu, keep0);
+    const unsigned int b1 = __ballot_sync(0xffffffffu, keep1);
+    const unsigned int tot = __popc(b0) + __popc(b1);
+    unsigned int wbase = 0;
+    if (lane == 0 && tot) wbase = atomicAdd(&sh.fill, tot);
+    wbase = __shfl_sync(0xffffffffu, wbase, 0);
+    if (keep0) {
+      const uint64_t pos = obase + wbase + __popc(b0 & lt);
+      st_key<KW>(out, pos, k0);
+      ((AT*)out.amp)[pos] = o0;
+    }
+    if (keep1) {
+      const uint64_t pos = obase + wbase + __popc(b0) + __popc(b1 & lt);
+      st_key<KW>(out, pos, k1);
+      ((AT*)out.amp)[pos] = o1;
+    }
+  }
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    out.seg_cnt[b] = sh.fill;
+    if (sh.fill) atomicAdd(&ctl->cnt[out_slot], (unsigned long long)sh.fill);
+  }
+  __syncthreads();  // the tables and the shared counts are reused
+}
+
 // Persistent: a resident wave of CTAs takes the buckets the partition used
 // (ctl->buckets, from the device count) one by one, so the launch does not
 // grow with the host's bucket bound (a graph sizes it for a static bound).
 // Shared memory: keys[C], amps[C] (storage type), slots[2C] (0 = empty, else
 // index + 1), partner[C].
-constexpr int kPairThreads = 512;
-
 template <int KW, class AT>
 __global__ void __launch_bounds__(kPairThreads, 3)
     k_pair(Ctl* ctl, Gate1 g, Arr bk, Arr out, int out_slot, uint32_t seq) {
   typedef typename KT<KW>::T K;
   extern __shared__ __align__(16) unsigned char smem[];
-  __shared__ unsigned int fill;
+  __shared__ PairShared sh;
+  pdl_next();
+  pdl_wait();
   if (ctl->err) return;
   const uint32_t C = 1u << bk.seg_log2;
   const uint32_t S = 2u * C;
@@ -284,130 +429,12 @@ __global__ void __launch_bounds__(kPairThreads, 3)
       partner[i] = -1;
     }
     for (uint32_t i = threadIdx.x; i < S; i += blockDim.x) slot[i] = 0u;
-    if (threadIdx.x == 0) fill = 0;
     __syncthreads();
     if (threadIdx.x == 0) *bcnt = 0u;  // bucket is clean for the next use
 
-    const K bmask = bit_mask<KW>(g.t);
-    const K cmask = mk<KW>(g.cmask[0], g.cmask[1]);
-    const K cval = mk<KW>(g.cval[0], g.cval[1]);
-    for (uint32_t i = threadIdx.x; i < n; i += blockDim.x) {
-      const K k = skey[i];
-      if ((k & cmask) != cval) continue;  // passes through unchanged
-      const K p = k & ~bmask;
-      uint32_t h = (uint32_t)khash(p) & (S - 1u);
-      // At most C entries live in 2C slots, so a free slot or the partner is
-      // always found within S probes; the bound only guards against misuse.
-      uint32_t probe = 0;
-      for (; probe < S; ++probe) {
-        const unsigned int old = atomicCAS(&slot[h], 0u, i + 1u);
-        if (old == 0u) break;
-        const uint32_t j = old - 1u;
-        if ((skey[j] & ~bmask) == p) {
-          partner[i] = (int)j;
-          partner[j] = (int)i;
-          break;
-        }
-        h = (h + 1u) & (S - 1u);
-      }
-      if (probe == S) raise_err(ctl, kErrProbe, seq, 0);
-    }
-    __syncthreads();
-
-    // Emitters: branches the controls leave alone, unpaired branches and the
-    // bit-0 member of each pair.  Listing them first (in the probe table, which
-    // is free now) keeps every lane of the arithmetic below busy.  The pairs
-    // are listed apart from the rest ([0, C) and [C, 2C) of the table), so a
-    // warp evaluates one form of the 2x2 (two members, or one): mixed, it
-    // would issue both FP64 sequences, each with part of its lanes.
-    unsigned int* emit = slot;
-    const uint32_t lane = threadIdx.x & 31u;
-    const unsigned int lt = (1u << lane) - 1u;
-    if (threadIdx.x == 0) fill = 0;
-    __shared__ unsigned int n_pairs, n_rest;
-    if (threadIdx.x == 0) n_pairs = n_rest = 0;
-    __syncthreads();
-    const uint32_t rounds_in = (n + blockDim.x - 1u) / blockDim.x;
-    for (uint32_t r = 0; r < rounds_in; ++r) {
-      const uint32_t i = r * blockDim.x + threadIdx.x;
-      bool ep = false, er = false;
-      if (i < n) {
-        const K k = skey[i];
-        const bool met = (k & cmask) == cval;
-        const bool kt = (k & bmask) != (K)0;
-        const bool paired = partner[i] >= 0;
-        ep = met && !kt && paired;
-        er = !met || !paired;
-      }
-      const unsigned int bp = __ballot_sync(0xffffffffu, ep);
-      const unsigned int br = __ballot_sync(0xffffffffu, er);
-      unsigned int wp = 0, wr = 0;
-      if (lane == 0) {
-        if (bp) wp = atomicAdd(&n_pairs, (unsigned int)__popc(bp));
-        if (br) wr = atomicAdd(&n_rest, (unsigned int)__popc(br));
-      }
-      wp = __shfl_sync(0xffffffffu, wp, 0);
-      wr = __shfl_sync(0xffffffffu, wr, 0);
-      if (ep) emit[wp + __popc(bp & lt)] = i;
-      if (er) emit[C + wr + __popc(br & lt)] = i;
-    }
-    __syncthreads();
-    const uint32_t np = n_pairs;
-    const uint32_t ne = np + n_rest;
-
-    const uint64_t obase = (uint64_t)b << out.seg_log2;
-    const uint32_t rounds = (ne + blockDim.x - 1u) / blockDim.x;
-    for (uint32_t r = 0; r < rounds; ++r) {
-      const uint32_t q = r * blockDim.x + threadIdx.x;
-      bool keep0 = false, keep1 = false;
-      K k0 = 0, k1 = 0;
-      AT o0, o1;
-      if (q < ne) {
-        const uint32_t i = q < np ? emit[q] : emit[C + (q - np)];
-        const K k = skey[i];
-        const AT ai = samp[i];
-        if ((k & cmask) != cval) {
-          keep0 = true;  // controls not met: the branch is unchanged
-          k0 = k;
-          o0 = ai;
-        } else {
-          const bool kt = (k & bmask) != (K)0;
-          const int j = partner[i];
-          k0 = k & ~bmask;
-          k1 = k | bmask;
-          const uint64_t av = angle_value(g, k0);
-          if (!kt)
-            children<AT>(g, av, true, ai, j >= 0, j >= 0 ? samp[j] : ai, o0, o1);
-          else
-            children<AT>(g, av, false, ai, true, ai, o0, o1);
-          keep0 = keep_amp(o0, g.eps, g.epsf, g.eps2);
-          keep1 = keep_amp(o1, g.eps, g.epsf, g.eps2);
-        }
-      }
-      const unsigned int b0 = __ballot_sync(0xffffffffu, keep0);
-      const unsigned int b1 = __ballot_sync(0xffffffffu, keep1);
-      const unsigned int tot = __popc(b0) + __popc(b1);
-      unsigned int wbase = 0;
-      if (lane == 0 && tot) wbase = atomicAdd(&fill, tot);
-      wbase = __shfl_sync(0xffffffffu, wbase, 0);
-      if (keep0) {
-        const uint64_t pos = obase + wbase + __popc(b0 & lt);
-        st_key<KW>(out, pos, k0);
-        ((AT*)out.amp)[pos] = o0;
-      }
-      if (keep1) {
-        const uint64_t pos = obase + wbase + __popc(b0) + __popc(b1 & lt);
-        st_key<KW>(out, pos, k1);
-        ((AT*)out.amp)[pos] = o1;
-      }
-    }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-      out.seg_cnt[b] = fill;
-      if (fill) atomicAdd(&ctl->cnt[out_slot], (unsigned long long)fill);
-      next_b = drawn;
-    }
-    __syncthreads();  // fill, next_b and the tables are reused by the next bucket
+    pair_bucket<KW, AT>(ctl, g, n, C, skey, samp, slot, partner, sh, out, b, out_slot, seq);
+    if (threadIdx.x == 0) next_b = drawn;
+    __syncthreads();  // next_b is reused by the next bucket
   }
 }
 
@@ -428,17 +455,19 @@ constexpr uint32_t kExpandChunkLog2 = 12;
 // shared-memory latencies of the fused run.
 constexpr int kExpandILP = 2;
 
-template <int KW, class AT>
+template <int KW, class AT, class LT>
 __global__ void __launch_bounds__(kStreamThreads, 4)
     k_expand(Ctl* ctl, Arr in, int in_slot, uint64_t n_chunks, Arr out, int out_slot,
-             const __grid_constant__ OpList ops, Gate1 g, uint32_t seq) {
+             const __grid_constant__ LT ops, Gate1 g, uint32_t seq) {
   typedef typename KT<KW>::T K;
-  __shared__ AT tab[kTabEntries];
-  __shared__ DevOp sops[kMaxOps];
+  __shared__ AT tab[LT::kTab];
+  __shared__ DevOp sops[LT::kOps];
   __shared__ unsigned int wtot[kStreamThreads / 32];
   __shared__ unsigned long long round_base;
-  if (ctl->err) return;
+  pdl_next();
   load_ops(ops, sops, tab);
+  pdl_wait();
+  if (ctl->err) return;
   if (blockIdx.x == 0 && threadIdx.x == 0) {
     ctl->cnt[(out_slot + 1) & 3] = 0;
     atomicMax(&ctl->peak, ctl->cnt[in_slot]);
@@ -604,21 +633,23 @@ constexpr size_t fold_smem_bytes() {
   return (size_t)kFoldSub * (sizeof(typename KT<KW>::T) + sizeof(AT));
 }
 
-template <int KW, class AT>
+template <int KW, class AT, class LT>
 __global__ void __launch_bounds__(kStreamThreads, 3)
     k_fold(Ctl* ctl, Arr in, int in_slot, uint64_t n_chunks, Arr out, int out_slot,
-           const __grid_constant__ OpList ops, Gate1 g, uint32_t seq) {
+           const __grid_constant__ LT ops, Gate1 g, uint32_t seq) {
   typedef typename KT<KW>::T K;
-  __shared__ AT tab[kTabEntries];
-  __shared__ DevOp sops[kMaxOps];
+  __shared__ AT tab[LT::kTab];
+  __shared__ DevOp sops[LT::kOps];
   __shared__ unsigned int wtot[kStreamThreads / 32];
   __shared__ unsigned long long round_base;
   __shared__ unsigned int n_act;
   extern __shared__ __align__(16) unsigned char fold_smem[];
   K* skey = (K*)fold_smem;
   AT* samp = (AT*)(fold_smem + (size_t)kFoldSub * sizeof(K));
-  if (ctl->err) return;
+  pdl_next();
   load_ops(ops, sops, tab);
+  pdl_wait();
+  if (ctl->err) return;
   if (blockIdx.x == 0 && threadIdx.x == 0) {
     ctl->cnt[(out_slot + 1) & 3] = 0;
     atomicMax(&ctl->peak, ctl->cnt[in_slot]);
@@ -993,6 +1024,8 @@ __global__ void __launch_bounds__(kStreamThreads, 4)
   __shared__ unsigned long long round_base;
   __shared__ unsigned int abort_flag;
   extern __shared__ __align__(128) unsigned char exp_smem[];
+  pdl_next();
+  pdl_wait();
   if (ctl->err) return;
   if (blockIdx.x == 0 && threadIdx.x == 0) {
     ctl->cnt[(out_slot + 1) & 3] = 0;
@@ -1150,6 +1183,8 @@ __global__ void __launch_bounds__(kStreamThreads, 4)
   __shared__ unsigned int n_act, abort_flag;
   extern __shared__ __align__(128) unsigned char fold_smem[];
   uint16_t* list = (uint16_t*)(fold_smem + stream_smem_bytes<KW, AT>());
+  pdl_next();
+  pdl_wait();
   if (ctl->err) return;
   if (blockIdx.x == 0 && threadIdx.x == 0) {
     ctl->cnt[(out_slot + 1) & 3] = 0;
@@ -1533,6 +1568,111 @@ __device__ __forceinline__ T* map_rank(T* p, uint32_t rank) {
   return (T*)out;
 }
 
+// ---------------------------------------------------------------------------
+// Bucket merge of a small state in one launch.  A cluster of CTAs, one bucket
+// each, takes the place of k_partition and k_pair: every CTA loads its share of
+// the branches, applies the queued operations and hands each branch to the CTA
+// of its pair class through distributed shared memory; after one cluster
+// barrier each CTA pairs its bucket as k_pair does.  Below about 16000 branches
+// a merge is latency (launch, counter, atomics, bucket round trip): 8 us here
+// against 15 us for the two launches at 4096 branches.
+constexpr uint32_t kMergeCap = 2048;  // branches per CTA (mean at most half)
+
+template <int KW, class AT>
+constexpr size_t merge_smem_bytes() {
+  return (size_t)kMergeCap * (sizeof(typename KT<KW>::T) + sizeof(AT) + 4 + 8);
+}
+
+template <int KW, class AT, class LT>
+__global__ void __launch_bounds__(kPairThreads)
+    k_merge_small(Ctl* ctl, Arr in, int in_slot, const __grid_constant__ LT ops, Gate1 g, Arr out,
+                  int out_slot, uint32_t seq) {
+  typedef typename KT<KW>::T K;
+  extern __shared__ __align__(16) unsigned char smem_ms[];
+  __shared__ AT tab[LT::kTab];
+  __shared__ DevOp sops[LT::kOps];
+  __shared__ unsigned int count, dead;
+  __shared__ PairShared sh;
+  AT* const samp = (AT*)smem_ms;
+  K* const skey = (K*)(samp + kMergeCap);
+  unsigned int* const slot = (unsigned int*)(skey + kMergeCap);
+  int* const partner = (int*)(slot + 2 * kMergeCap);
+  pdl_next();
+  // The first cluster barrier (every CTA's counter is zero) is waited for only
+  // before the first branch is handed over.
+  if (threadIdx.x == 0) count = 0u;
+  asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+  load_ops(ops, sops, tab);
+  for (uint32_t i = threadIdx.x; i < 2 * kMergeCap; i += blockDim.x) slot[i] = 0u;
+  for (uint32_t i = threadIdx.x; i < kMergeCap; i += blockDim.x) partner[i] = -1;
+  pdl_wait();
+  if (threadIdx.x == 0) dead = ctl->err;  // one answer for the CTA
+  const uint64_t n_dense = ctl->cnt[in_slot];
+  if (blockIdx.x == 0 && threadIdx.x == 0) {
+    atomicMax(&ctl->peak, n_dense);
+    ctl->cnt[(out_slot + 1) & 3] = 0;
+  }
+  bool may_push = false;
+  auto all_zero = [&] {
+    if (!may_push) asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+    may_push = true;
+  };
+  __syncthreads();
+  const K bmask = bit_mask<KW>(g.t);
+  constexpr int kILP = 2;
+  // One tile of the input.
+  auto take = [&](uint64_t base, uint32_t lim) {
+    K k[kILP];
+    AT v[kILP];
+    bool live[kILP];
+#pragma unroll
+    for (int q = 0; q < kILP; ++q) {
+      const uint32_t j = q * kPairThreads + threadIdx.x;
+      live[q] = j < lim;
+      k[q] = 0;
+      v[q].x = v[q].y = 0;
+      if (live[q]) {
+        k[q] = ld_key<KW>(in, base + j);
+        v[q] = ((const AT*)in.amp)[base + j];
+      }
+    }
+    apply_ops_n<KW, AT, kILP>(ops.n, sops, tab, k, v, live);
+    all_zero();
+#pragma unroll
+    for (int q = 0; q < kILP; ++q) {
+      if (!live[q]) continue;
+      const uint32_t r = (uint32_t)(((khash(k[q] & ~bmask) >> 32) * (uint64_t)gridDim.x) >> 32);
+      const unsigned int at = atomicAdd(map_rank(&count, r), 1u);
+      if (at < kMergeCap) {
+        *map_rank(skey + at, r) = k[q];
+        *map_rank(samp + at, r) = v[q];
+      } else {
+        raise_err(ctl, kErrBucket, seq, (unsigned long long)at + 1);
+      }
+    }
+  };
+  constexpr uint32_t kTile = kILP * kPairThreads;
+  if (dead) {
+  } else if (in.seg_cnt) {
+    for (uint32_t sg = blockIdx.x; sg < in.n_seg; sg += gridDim.x) {
+      const uint32_t cnt = in.seg_cnt[sg];
+      const uint64_t first = (uint64_t)sg << in.seg_log2;
+      for (uint32_t j = 0; j < cnt; j += kTile) take(first + j, cnt - j < kTile ? cnt - j : kTile);
+    }
+  } else {
+    // An even share of the dense input per CTA.
+    const uint64_t share = (n_dense + gridDim.x - 1) / gridDim.x;
+    const uint64_t lo = share * blockIdx.x, hi = lo + share < n_dense ? lo + share : n_dense;
+    for (uint64_t j = lo; j < hi; j += kTile) take(j, (uint32_t)(hi - j < kTile ? hi - j : kTile));
+  }
+  all_zero();
+  cluster_sync_all();  // every branch has arrived
+  if (dead) return;
+  const uint32_t n = count > kMergeCap ? 0u : count;  // an overflow is flagged
+  pair_bucket<KW, AT>(ctl, g, n, kMergeCap, skey, samp, slot, partner, sh, out, blockIdx.x,
+                      out_slot, seq);
+}
+
 // Slot tag: (CTA rank << 12 | index) + 1; 0 marks an empty slot.
 __device__ __forceinline__ uint32_t ctag(uint32_t r, uint32_t i) { return ((r << kSliceLog2) | i) + 1u; }
 
@@ -1764,11 +1904,7 @@ static int stream_grid(const Launch& L, int threads) {
 }
 
 cudaError_t launch_init(const Launch& L, Ctl* ctl, Arr a, int slot, bool amp32) {
-  if (amp32)
-    k_init<float2><<<1, 32, 0, L.stream>>>(ctl, a, slot);
-  else
-    k_init<double2><<<1, 32, 0, L.stream>>>(ctl, a, slot);
-  return cudaGetLastError();
+  return launch_next(amp32 ? k_init<float2> : k_init<double2>, 1, 32, 0, L.stream, ctl, a, slot);
 }
 
 #define SQS_DISPATCH(kw, amp32, MACRO) \
@@ -1782,26 +1918,47 @@ cudaError_t launch_init(const Launch& L, Ctl* ctl, Arr a, int slot, bool amp32) 
     }                                  \
   } while (0)
 
-template <int KW, class AT>
-static void apply_inplace_t(const Launch& L, Ctl* ctl, Arr a, int slot, const OpList& ops) {
-  const int g = stream_grid(L, kStreamThreads);
-  if (ops.touches_keys && ops.touches_amps)
-    k_apply_inplace<KW, AT, true, true>
-        <<<g, kStreamThreads, 0, L.stream>>>(ctl, a, slot, ops, L.seq);
-  else if (ops.touches_keys)
-    k_apply_inplace<KW, AT, true, false>
-        <<<g, kStreamThreads, 0, L.stream>>>(ctl, a, slot, ops, L.seq);
-  else
-    k_apply_inplace<KW, AT, false, true>
-        <<<g, kStreamThreads, 0, L.stream>>>(ctl, a, slot, ops, L.seq);
+// Calls f with the list itself or, when it fits, its small form.
+template <class F>
+static cudaError_t with_list(const OpList& ops, F f) {
+  if (!fits_small(ops)) return f(ops);
+  OpListSmall s;
+  copy_small(ops, s);
+  return f(s);
 }
+
+template <int KW, class AT, class LT, int NI>
+static cudaError_t apply_inplace_ni(const Launch& L, Ctl* ctl, Arr a, int slot, const LT& ops) {
+  const auto kern = ops.touches_keys
+                        ? (ops.touches_amps ? k_apply_inplace<KW, AT, true, true, LT, NI>
+                                            : k_apply_inplace<KW, AT, true, false, LT, NI>)
+                        : k_apply_inplace<KW, AT, false, true, LT, NI>;
+  return launch_next(kern, stream_grid(L, NI * kStreamThreads), kStreamThreads, 0, L.stream, ctl, a,
+                     slot, ops, L.seq);
+}
+template <int KW, class AT, class LT>
+static cudaError_t apply_inplace_t(const Launch& L, Ctl* ctl, Arr a, int slot, const LT& ops) {
+  // Slots that do not fill the SMs once: one branch a thread, so that an
+  // operation's instructions spread over four times the warps.
+  return L.n_hint <= (uint64_t)L.sm_count * kStreamThreads
+             ? apply_inplace_ni<KW, AT, LT, 1>(L, ctl, a, slot, ops)
+             : apply_inplace_ni<KW, AT, LT, kApplyILP>(L, ctl, a, slot, ops);
+}
+
+// The variant of `f` for the key words and amplitude type.
+#define SQS_PICK(kw, amp32, f) \
+  ((kw) == 1 ? ((amp32) ? f<1, float2> : f<1, double2>) : ((amp32) ? f<2, float2> : f<2, double2>))
+// ... and the type of an operation list.
+#define SQS_PICK_L(kw, amp32, f, LT)                         \
+  ((kw) == 1 ? ((amp32) ? f<1, float2, LT> : f<1, double2, LT>) \
+             : ((amp32) ? f<2, float2, LT> : f<2, double2, LT>))
 
 cudaError_t launch_apply_inplace(const Launch& L, int kw, bool amp32, Ctl* ctl, Arr a, int slot,
                                  const OpList& ops) {
-#define SQS_AI(KW_, AT_) apply_inplace_t<KW_, AT_>(L, ctl, a, slot, ops)
-  SQS_DISPATCH(kw, amp32, SQS_AI);
-#undef SQS_AI
-  return cudaGetLastError();
+  return with_list(ops, [&](const auto& list) {
+    typedef std::decay_t<decltype(list)> LT;
+    return SQS_PICK_L(kw, amp32, apply_inplace_t, LT)(L, ctl, a, slot, list);
+  });
 }
 
 cudaError_t launch_apply_compact(const Launch& L, int kw, bool amp32, Ctl* ctl, Arr in,
@@ -1809,13 +1966,8 @@ cudaError_t launch_apply_compact(const Launch& L, int kw, bool amp32, Ctl* ctl, 
   const uint64_t chunks = (L.n_hint + (1ull << out.seg_log2) - 1) >> out.seg_log2;
   uint64_t g = chunks < 1 ? 1 : chunks;
   if (g > (uint64_t)L.sm_count * 8) g = (uint64_t)L.sm_count * 8;
-#define SQS_AC(KW_, AT_)                                                              \
-  k_apply_compact<KW_, AT_>                                                           \
-      <<<(int)g, kStreamThreads, 0, L.stream>>>(ctl, in, in_slot, out, out_slot, ops, \
-                                                L.seq)
-  SQS_DISPATCH(kw, amp32, SQS_AC);
-#undef SQS_AC
-  return cudaGetLastError();
+  return launch_next(SQS_PICK(kw, amp32, k_apply_compact), g, kStreamThreads, 0, L.stream, ctl, in,
+                     in_slot, out, out_slot, ops, L.seq);
 }
 
 __global__ void k_angle_table(double2* tab, uint32_t digits, double scale, double offset) {
@@ -1882,9 +2034,8 @@ static cudaError_t expand_staged_t(const Launch& L, Ctl* ctl, Arr in, int in_slo
   uint64_t grid = (uint64_t)L.sm_count * (uint64_t)occ;
   if (grid > units) grid = units;
   if (grid < 1) grid = 1;
-  k_expand_staged<KW, AT><<<(int)grid, kStreamThreads, smem, L.stream>>>(
-      ctl, in, in_slot, n_chunks, out, out_slot, g, L.seq);
-  return cudaGetLastError();
+  return launch_next(k_expand_staged<KW, AT>, grid, kStreamThreads, smem, L.stream, ctl, in,
+                     in_slot, n_chunks, out, out_slot, g, L.seq);
 }
 
 template <int KW, class AT>
@@ -1903,9 +2054,8 @@ static cudaError_t fold_staged_t(const Launch& L, Ctl* ctl, Arr in, int in_slot,
   uint64_t grid = (uint64_t)L.sm_count * (uint64_t)occ;
   if (grid > units) grid = units;
   if (grid < 1) grid = 1;
-  k_fold_staged<KW, AT><<<(int)grid, kStreamThreads, smem, L.stream>>>(
-      ctl, in, in_slot, n_chunks, out, out_slot, g, L.seq);
-  return cudaGetLastError();
+  return launch_next(k_fold_staged<KW, AT>, grid, kStreamThreads, smem, L.stream, ctl, in, in_slot,
+                     n_chunks, out, out_slot, g, L.seq);
 }
 
 cudaError_t launch_expand(const Launch& L, int kw, bool amp32, Ctl* ctl, Arr in, int in_slot,
@@ -1920,26 +2070,24 @@ cudaError_t launch_expand(const Launch& L, int kw, bool amp32, Ctl* ctl, Arr in,
   }
   uint64_t grid = n_chunks < 1 ? 1 : n_chunks;
   if (grid > (uint64_t)L.sm_count * 8) grid = (uint64_t)L.sm_count * 8;
-#define SQS_EX(KW_, AT_)                                                                  \
-  k_expand<KW_, AT_><<<(int)grid, kStreamThreads, 0, L.stream>>>(ctl, in, in_slot, n_chunks, \
-                                                                 out, out_slot, ops, g, L.seq)
-  SQS_DISPATCH(kw, amp32, SQS_EX);
-#undef SQS_EX
-  return cudaGetLastError();
+  return with_list(ops, [&](const auto& list) {
+    typedef std::decay_t<decltype(list)> LT;
+    return launch_next(SQS_PICK_L(kw, amp32, k_expand, LT), grid, kStreamThreads, 0, L.stream, ctl,
+                       in, in_slot, n_chunks, out, out_slot, list, g, L.seq);
+  });
 }
 
-template <int KW, class AT>
+template <int KW, class AT, class LT>
 static cudaError_t fold_t(const Launch& L, Ctl* ctl, Arr in, int in_slot, uint64_t n_chunks,
-                          const OpList& ops, const Gate1& g, Arr out, int out_slot) {
+                          const LT& ops, const Gate1& g, Arr out, int out_slot) {
   const size_t smem = fold_smem_bytes<KW, AT>();
   static std::atomic<unsigned long long> configured{0};
-  cudaError_t e = ensure_smem_optin((const void*)k_fold<KW, AT>, smem, configured);
+  cudaError_t e = ensure_smem_optin((const void*)k_fold<KW, AT, LT>, smem, configured);
   if (e != cudaSuccess) return e;
   uint64_t grid = n_chunks < 1 ? 1 : n_chunks;
   if (grid > (uint64_t)L.sm_count * 12) grid = (uint64_t)L.sm_count * 12;
-  k_fold<KW, AT><<<(int)grid, kStreamThreads, smem, L.stream>>>(ctl, in, in_slot, n_chunks, out,
-                                                                out_slot, ops, g, L.seq);
-  return cudaGetLastError();
+  return launch_next(k_fold<KW, AT, LT>, grid, kStreamThreads, smem, L.stream, ctl, in, in_slot,
+                     n_chunks, out, out_slot, ops, g, L.seq);
 }
 
 cudaError_t launch_fold(const Launch& L, int kw, bool amp32, Ctl* ctl, Arr in, int in_slot,
@@ -1953,23 +2101,68 @@ cudaError_t launch_fold(const Launch& L, int kw, bool amp32, Ctl* ctl, Arr in, i
     return amp32 ? fold_staged_t<2, float2>(L, ctl, in, in_slot, n_chunks, g, out, out_slot)
                  : fold_staged_t<2, double2>(L, ctl, in, in_slot, n_chunks, g, out, out_slot);
   }
-  if (kw == 1)
-    return amp32 ? fold_t<1, float2>(L, ctl, in, in_slot, n_chunks, ops, g, out, out_slot)
-                 : fold_t<1, double2>(L, ctl, in, in_slot, n_chunks, ops, g, out, out_slot);
-  return amp32 ? fold_t<2, float2>(L, ctl, in, in_slot, n_chunks, ops, g, out, out_slot)
-               : fold_t<2, double2>(L, ctl, in, in_slot, n_chunks, ops, g, out, out_slot);
+  return with_list(ops, [&](const auto& list) {
+    typedef std::decay_t<decltype(list)> LT;
+    return SQS_PICK_L(kw, amp32, fold_t, LT)(L, ctl, in, in_slot, n_chunks, list, g, out, out_slot);
+  });
 }
 
 cudaError_t launch_partition(const Launch& L, int kw, bool amp32, Ctl* ctl, Arr in, int in_slot,
                              const OpList& ops, const uint64_t clear[2], Arr bk,
                              uint32_t fill_target) {
-  const int grid = stream_grid(L, kStreamThreads);
-#define SQS_PT(KW_, AT_)                                                                \
-  k_partition<KW_, AT_><<<grid, kStreamThreads, 0, L.stream>>>(             \
-      ctl, in, in_slot, ops, clear[0], clear[1], bk, L.seq, fill_target)
-  SQS_DISPATCH(kw, amp32, SQS_PT);
-#undef SQS_PT
-  return cudaGetLastError();
+  const int grid = stream_grid(L, kPartILP * kStreamThreads);
+  return with_list(ops, [&](const auto& list) {
+    typedef std::decay_t<decltype(list)> LT;
+    return launch_next(SQS_PICK_L(kw, amp32, k_partition, LT), grid, kStreamThreads, 0, L.stream,
+                       ctl, in, in_slot, list, clear[0], clear[1], bk, L.seq, fill_target);
+  });
+}
+
+uint64_t merge_small_max() { return (uint64_t)16 * (kMergeCap / 2); }
+
+template <int KW, class AT, class LT>
+static cudaError_t merge_small_t(const Launch& L, Ctl* ctl, Arr in, int in_slot, const LT& ops,
+                                 const Gate1& g, Arr out, int out_slot) {
+  const auto kern = k_merge_small<KW, AT, LT>;
+  const size_t smem = merge_smem_bytes<KW, AT>();
+  static std::atomic<unsigned long long> configured{0}, wide{0};
+  cudaError_t e = ensure_smem_optin((const void*)kern, smem, configured);
+  if (e != cudaSuccess) return e;
+  int dev = 0;
+  e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  if (out.n_seg > 8 && !(dev < 64 && (wide.load(std::memory_order_acquire) >> dev & 1ull))) {
+    e = cudaFuncSetAttribute((const void*)kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    if (e != cudaSuccess) return e;
+    if (dev < 64) wide.fetch_or(1ull << dev, std::memory_order_acq_rel);
+  }
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(out.n_seg);
+  cfg.blockDim = dim3(kPairThreads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = L.stream;
+  cudaLaunchAttribute attr[2];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = out.n_seg;
+  attr[0].val.clusterDim.y = 1;
+  attr[0].val.clusterDim.z = 1;
+  attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[1].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 2;
+  uint32_t seq = L.seq;
+  void* ptr[] = {&ctl, &in, &in_slot, (void*)&ops, (void*)&g, &out, &out_slot, &seq};
+  return cudaLaunchKernelExC(&cfg, (const void*)kern, ptr);
+}
+
+cudaError_t launch_merge_small(const Launch& L, int kw, bool amp32, Ctl* ctl, Arr in, int in_slot,
+                               const OpList& ops, const Gate1& g, Arr out, int out_slot) {
+  if (out.n_seg < 1 || out.n_seg > 16 || (out.n_seg & (out.n_seg - 1)))
+    return cudaErrorInvalidValue;
+  return with_list(ops, [&](const auto& list) {
+    typedef std::decay_t<decltype(list)> LT;
+    return SQS_PICK_L(kw, amp32, merge_small_t, LT)(L, ctl, in, in_slot, list, g, out, out_slot);
+  });
 }
 
 int pair_log2_capacity(int kw, bool amp32) {
@@ -2006,8 +2199,8 @@ static cudaError_t pair_t(const Launch& L, Ctl* ctl, const Gate1& g, Arr bk, Arr
   uint64_t grid = (uint64_t)L.sm_count * (uint64_t)occ;
   if (grid > bk.n_seg) grid = bk.n_seg;
   if (grid < 1) grid = 1;
-  k_pair<KW, AT><<<(int)grid, kPairThreads, smem, L.stream>>>(ctl, g, bk, out, out_slot, L.seq);
-  return cudaGetLastError();
+  return launch_next(k_pair<KW, AT>, grid, kPairThreads, smem, L.stream, ctl, g, bk, out, out_slot,
+                     L.seq);
 }
 
 cudaError_t launch_pair(const Launch& L, int kw, bool amp32, Ctl* ctl, const Gate1& g, Arr bk,

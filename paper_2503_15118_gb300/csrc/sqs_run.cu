@@ -74,17 +74,19 @@ __device__ __forceinline__ typename KT<KW>::T key_of(const SlotMap& m, uint32_t 
 
 constexpr int kScatterILP = 4;
 
-template <int KW, class AT, bool OPS>
+template <int KW, class AT, class LT>
 __global__ void __launch_bounds__(kStreamThreads)
-    k_slot_scatter(Ctl* ctl, Arr in, int in_slot, const __grid_constant__ OpList ops,
+    k_slot_scatter(Ctl* ctl, Arr in, int in_slot, const __grid_constant__ LT ops,
                    const __grid_constant__ SlotMap map, AT* amp, uint8_t* pres) {
   typedef typename KT<KW>::T K;
-  __shared__ AT tab[OPS ? kTabEntries : 1];
-  __shared__ DevOp sops[OPS ? kMaxOps : 1];
+  __shared__ AT tab[LT::kTab];
+  __shared__ DevOp sops[LT::kOps];
   __shared__ uint16_t ulist[kStreamThreads];
   __shared__ unsigned int n_ulist;
+  pdl_next();
+  load_ops(ops, sops, tab);
+  pdl_wait();
   if (ctl->err) return;
-  if (OPS) load_ops(ops, sops, tab);
   const uint64_t n_dense = ctl->cnt[in_slot];
   if (blockIdx.x == 0 && threadIdx.x == 0) atomicMax(&ctl->peak, n_dense);
   for_units(in, n_dense, kScatterILP * blockDim.x, ulist, &n_ulist,
@@ -103,7 +105,7 @@ __global__ void __launch_bounds__(kStreamThreads)
         v[q] = ((const AT*)in.amp)[base + j];
       }
     }
-    if (OPS) apply_ops_n<KW, AT, kScatterILP>(ops.n, sops, tab, k, v, live);
+    if (ops.n) apply_ops_n<KW, AT, kScatterILP>(ops.n, sops, tab, k, v, live);
 #pragma unroll
     for (int q = 0; q < kScatterILP; ++q) {
       if (live[q]) {
@@ -301,6 +303,8 @@ __device__ __forceinline__ void finish_run(Ctl* ctl, const RunProg& prog, RunSha
 }
 
 __device__ __forceinline__ void begin_run(Ctl* ctl, RunShared& sh, int out_slot) {
+  pdl_next();
+  pdl_wait();
   if (blockIdx.x == 0 && threadIdx.x == 0) ctl->cnt[(out_slot + 1) & 3] = 0;
   for (uint32_t i = threadIdx.x; i < kMaxItems; i += blockDim.x) sh.stage[i] = 0u;
   if (threadIdx.x < 4) sh.lc[threadIdx.x >> 1][threadIdx.x & 1u] = 0u;
@@ -518,13 +522,13 @@ cudaError_t scatter_t(const Launch& L, Ctl* ctl, Arr in, int in_slot, const OpLi
   uint64_t grid = (L.n_hint + per - 1) / per;
   const uint64_t cap = (uint64_t)L.sm_count * 8;
   grid = grid < 1 ? 1 : (grid > cap ? cap : grid);
-  if (ops.n)
-    k_slot_scatter<KW, AT, true><<<(int)grid, kStreamThreads, 0, L.stream>>>(
-        ctl, in, in_slot, ops, map, (AT*)amp, pres);
-  else
-    k_slot_scatter<KW, AT, false><<<(int)grid, kStreamThreads, 0, L.stream>>>(
-        ctl, in, in_slot, ops, map, (AT*)amp, pres);
-  return cudaGetLastError();
+  if (!fits_small(ops))
+    return launch_next(k_slot_scatter<KW, AT, OpList>, grid, kStreamThreads, 0, L.stream, ctl, in,
+                       in_slot, ops, map, (AT*)amp, pres);
+  OpListSmall s;
+  copy_small(ops, s);
+  return launch_next(k_slot_scatter<KW, AT, OpListSmall>, grid, kStreamThreads, 0, L.stream, ctl,
+                     in, in_slot, s, map, (AT*)amp, pres);
 }
 
 template <int KW, class AT>
@@ -536,9 +540,8 @@ cudaError_t run_t(const Launch& L, Ctl* ctl, void* amp, uint8_t* pres, const Slo
   if (e != cudaSuccess) return e;
   const uint32_t wave = (uint32_t)L.sm_count * 2u;
   const uint32_t grid = prog.n_areas < wave ? prog.n_areas : wave;
-  k_slot_run<KW, AT><<<grid, kRunThreads, run_smem_bytes<AT>(prog.area_log2), L.stream>>>(
-      ctl, (AT*)amp, pres, map, prog, out, out_slot, L.seq);
-  return cudaGetLastError();
+  return launch_next(k_slot_run<KW, AT>, grid, kRunThreads, run_smem_bytes<AT>(prog.area_log2),
+                     L.stream, ctl, (AT*)amp, pres, map, prog, out, out_slot, L.seq);
 }
 
 template <int KW, class AT>
@@ -550,9 +553,8 @@ cudaError_t bucket_t(const Launch& L, Ctl* ctl, Arr bk, const SlotMap& map, cons
   if (e != cudaSuccess) return e;
   const uint32_t wave = (uint32_t)L.sm_count * 2u;
   const uint32_t grid = bk.n_seg < wave ? bk.n_seg : wave;
-  k_bucket_run<KW, AT><<<grid ? grid : 1u, kRunThreads, smem, L.stream>>>(
-      ctl, bk, map, prog, k, tmask[0], tmask[1], out, out_slot, L.seq);
-  return cudaGetLastError();
+  return launch_next(k_bucket_run<KW, AT>, grid ? grid : 1u, kRunThreads, smem, L.stream, ctl, bk,
+                     map, prog, k, tmask[0], tmask[1], out, out_slot, L.seq);
 }
 
 }  // namespace
