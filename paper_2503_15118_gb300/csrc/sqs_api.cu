@@ -153,6 +153,7 @@ struct sqs_state {
 
   std::vector<HostOp> pending;
   OpList ops_buf;   // staging for one launch's fused operations
+  sqs::PlaneList planes;  // the same on bit planes
   sqs::RunProg run_prog;  // staging for one addressed run
   uint64_t ub = 1;  // upper bound of the current branch count
   uint32_t seq = 0;
@@ -518,20 +519,31 @@ sqs_status no_capture(sqs_state* st, const char* what) {
 struct Group {
   std::vector<const HostOp*> ops;
   std::vector<uint32_t> shift, nbits;
+  std::vector<bool> swapped;  // the selector bit is a flipped one: c0 and c1 change places
   uint32_t bits = 0;
 };
 
 void fold_group(Group& g, OpList& L) {
   if (g.ops.empty()) return;
   const uint32_t size = 1u << g.bits;
-  for (uint32_t idx = 0; idx < size; ++idx) {
-    std::complex<double> f(1.0, 0.0);
-    for (size_t j = 0; j < g.ops.size(); ++j) {
-      const uint32_t oc = (idx >> g.shift[j]) & ((1u << g.nbits[j]) - 1u);
-      if (oc == 1) f *= g.ops[j]->c0;
-      else if (oc == 2) f *= g.ops[j]->c1;
+  // Built operation by operation: the entries so far (outcome 0 of operation j),
+  // times its factors for the other outcomes.
+  double2* const tab = L.tab + L.n_tab;
+  tab[0] = make_double2(1.0, 0.0);
+  for (size_t j = 0; j < g.ops.size(); ++j) {
+    const uint32_t n = 1u << g.shift[j];
+    const std::complex<double> c[2] = {g.swapped[j] ? g.ops[j]->c1 : g.ops[j]->c0,
+                                       g.swapped[j] ? g.ops[j]->c0 : g.ops[j]->c1};
+    for (uint32_t oc = 1; oc < (1u << g.nbits[j]); ++oc) {
+      double2* const to = tab + (size_t)oc * n;
+      if (oc == 3) {  // never selected
+        std::memcpy(to, tab, n * sizeof(double2));
+        continue;
+      }
+      const double re = c[oc - 1].real(), im = c[oc - 1].imag();
+      for (uint32_t i = 0; i < n; ++i)
+        to[i] = make_double2(tab[i].x * re - tab[i].y * im, tab[i].x * im + tab[i].y * re);
     }
-    L.tab[L.n_tab + idx] = make_double2(f.real(), f.imag());
   }
   DevOp t;
   std::memset(&t, 0, sizeof(t));
@@ -552,6 +564,24 @@ size_t pack_ops(const std::vector<HostOp>& ops, size_t from, OpList& L) {
   Group g;
   size_t i = from;
   constexpr uint32_t kGroupBits = 10;
+  // Uncontrolled X are not issued one by one: the bits flipped so far are
+  // carried along (a later predicate or selector on such a bit is the opposite
+  // one) and flipped in one operation before a field is read or written, or at
+  // the end.
+  uint64_t flip[2] = {0, 0};
+  auto flipped = [&](uint32_t q) { return (flip[q >> 6] >> (q & 63)) & 1ull; };
+  auto emit_flips = [&] {
+    if (!(flip[0] | flip[1])) return;
+    DevOp x;
+    std::memset(&x, 0, sizeof(x));
+    x.kind = sqs::OP_XOR;
+    x.sel_bit = 128;
+    x.xmask[0] = flip[0];
+    x.xmask[1] = flip[1];
+    L.op[L.n++] = x;
+    L.touches_keys = 1;
+    flip[0] = flip[1] = 0;
+  };
   for (; i < ops.size(); ++i) {
     const HostOp& h = ops[i];
     const uint32_t kind = h.d.kind;
@@ -563,14 +593,26 @@ size_t pack_ops(const std::vector<HostOp>& ops, size_t from, OpList& L) {
     uint32_t need_tab = L.n_tab + pend_tab;
     if (mul) need_tab = closes ? need_tab + (1u << nb) : L.n_tab + (1u << (g.bits + nb));
     const uint32_t groups_after = (closes || g.ops.empty() ? 0u : 1u) + (mul ? 1u : 0u) +
-                                  (closes && !g.ops.empty() ? 1u : 0u);
+                                  (closes && !g.ops.empty() ? 1u : 0u) + 1u;  // the flips
     if (L.n + 1 + groups_after > (uint32_t)sqs::kMaxOps || need_tab > (uint32_t)sqs::kTabEntries)
       break;
+    if (kind == sqs::OP_XOR && !(h.d.pmask[0] | h.d.pmask[1])) {
+      flip[0] ^= h.d.xmask[0];
+      flip[1] ^= h.d.xmask[1];
+      continue;
+    }
     if (closes) fold_group(g, L);
     DevOp d = h.d;
+    if (kind != sqs::OP_XOR && !mul && kind != sqs::OP_PRUNE) {
+      emit_flips();  // the operation reads or writes a field
+    } else {
+      d.pval[0] ^= flip[0] & d.pmask[0];
+      d.pval[1] ^= flip[1] & d.pmask[1];
+    }
     if (mul) {
       d.shift = g.bits;
       g.ops.push_back(&h);
+      g.swapped.push_back(d.sel_bit < 128 && flipped(d.sel_bit));
       g.shift.push_back(g.bits);
       g.nbits.push_back(nb);
       g.bits += nb;
@@ -584,8 +626,16 @@ size_t pack_ops(const std::vector<HostOp>& ops, size_t from, OpList& L) {
     L.op[L.n++] = d;
   }
   fold_group(g, L);
+  emit_flips();
   return i - from;
 }
+
+// In-place passes of this many operations work on bit planes, over at least a
+// tile of 4096 branches per SM or so: with fewer, whole SMs would idle, and the
+// latency of the operations one after another is the same (4096 branches, 20
+// qubits: 316 us a circuit on planes, 290 branch by branch).
+constexpr uint32_t kPlaneMin = 12;
+constexpr uint64_t kPlaneSlots = 1ull << 19;
 
 // Standalone pass over the current state with the packed list.
 sqs_status run_list(sqs_state* st, const OpList& L) {
@@ -614,8 +664,13 @@ sqs_status run_list(sqs_state* st, const OpList& L) {
     st->cur_slot = out_slot;
   } else if (L.touches_keys || L.touches_amps) {
     Traced tr(st, SQS_K_APPLY);
-    e = sqs::launch_apply_inplace(launch_of(st, in_slots), st->kw, st->amp32, st->ctl,
-                                  st->cur.view(), st->cur_slot, L);
+    if (L.n >= kPlaneMin && in_slots >= kPlaneSlots &&
+        sqs::plane_list(L, st->total_bits, st->planes))
+      e = sqs::launch_apply_planes(launch_of(st, in_slots), st->kw, st->amp32, st->ctl,
+                                   st->cur.view(), st->cur_slot, st->planes);
+    else
+      e = sqs::launch_apply_inplace(launch_of(st, in_slots), st->kw, st->amp32, st->ctl,
+                                    st->cur.view(), st->cur_slot, L);
   }
   if (e != cudaSuccess) return cuda_fail(st, e, "launch");
   return SQS_OK;
