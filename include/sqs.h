@@ -361,6 +361,11 @@ sqs_status sqs_state_set_wait_test(sqs_state* st, uint32_t wait_limit, int32_t s
  * Waits. */
 sqs_status sqs_export(sqs_state* st, uint64_t* keys, double* amps, uint64_t cap, uint64_t* n);
 
+/* The same with the key words in two arrays: keys_lo receives the low words,
+ * keys_hi the high words of two-word keys (ignored, may be NULL, otherwise). */
+sqs_status sqs_export_split(sqs_state* st, uint64_t* keys_lo, uint64_t* keys_hi, double* amps,
+                            uint64_t cap, uint64_t* n);
+
 /* Replaces the state with n branches from host memory (same layout as
  * sqs_export; keys must be distinct and fit the register widths).  Work
  * issued before and not yet executed (queued operations, a held run of

@@ -11,12 +11,15 @@ import glob
 import os
 import shutil
 import subprocess
+import sysconfig
 
 HERE = os.path.dirname(os.path.abspath(__file__))
 ROOT = os.path.dirname(HERE)
 CSRC = os.path.join(HERE, "csrc")
 OUT_DIR = os.path.join(HERE, "_build")
 LIB = os.path.join(OUT_DIR, "libsqs.so")
+WALK_SRC = os.path.join(CSRC, "sqs_walk.cpp")
+WALK = os.path.join(OUT_DIR, "sqs_walk.so")
 
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 NVCC_FLAGS = ["-O3", "-std=c++17", "-lineinfo", "-fmad=false", "-Xcompiler", "-fPIC,-O2",
@@ -38,7 +41,8 @@ def sources():
 
 
 def _newest_input():
-    files = sources() + glob.glob(os.path.join(CSRC, "*.h")) + glob.glob(os.path.join(CSRC, "*.cuh")) + \
+    files = sources() + [WALK_SRC] + glob.glob(os.path.join(CSRC, "*.h")) + \
+        glob.glob(os.path.join(CSRC, "*.cuh")) + \
         [os.path.join(ROOT, "include", "sqs.h"), os.path.abspath(__file__)]
     return max(os.path.getmtime(f) for f in files)
 
@@ -73,12 +77,31 @@ def build(force: bool = False, verbose: bool = False, ptxas_info: bool = False) 
         f.write("{ global: sqs_*; local: *; };\n")
     tmp = LIB + ".tmp"
     cmd = [nvcc, *ARCH, "-shared", "-o", tmp, *objs, "-lcudart_static",
-           "-Xlinker", f"--version-script={vscript}"]
+           "-Xlinker", f"--version-script={vscript}", "-Xlinker", "-soname=libsqs.so"]
     r = subprocess.run(cmd, capture_output=True, text=True)
     if r.returncode != 0:
         raise RuntimeError(f"link failed:\n{r.stderr}")
-    os.replace(tmp, LIB)
+    build_walk(tmp)
+    os.replace(tmp, LIB)  # last: its time tells whether everything is built
     return LIB
+
+
+def build_walk(lib: str) -> None:
+    """The gate-list walker (csrc/sqs_walk.cpp), a CPython module linked to the
+    library beside it; without Python's headers the binding walks gate lists in
+    Python."""
+    inc = sysconfig.get_paths()["include"]
+    if not os.path.exists(os.path.join(inc, "Python.h")):
+        if os.path.exists(WALK):
+            os.remove(WALK)
+        return
+    cmd = [shutil.which("g++") or "g++", "-O2", "-std=c++17", "-fPIC", "-shared", "-I", inc,
+           "-I", os.path.join(ROOT, "include"), WALK_SRC, lib, "-Wl,-rpath,$ORIGIN",
+           "-o", WALK + ".tmp"]
+    r = subprocess.run(cmd, capture_output=True, text=True)
+    if r.returncode != 0:
+        raise RuntimeError(f"g++ failed on {WALK_SRC}:\n{r.stderr}")
+    os.replace(WALK + ".tmp", WALK)
 
 
 if __name__ == "__main__":

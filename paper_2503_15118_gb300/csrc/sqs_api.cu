@@ -3388,7 +3388,10 @@ sqs_status sqs_probabilities_sparse(sqs_state* st, uint32_t reg, uint64_t* value
   return SQS_OK;
 }
 
-sqs_status sqs_export(sqs_state* st, uint64_t* keys, double* amps, uint64_t cap, uint64_t* n) {
+// Branches to host memory, ascending keys: low words at keys[stride * i], high
+// words of two-word keys at keys_hi[stride * i].
+static sqs_status export_to(sqs_state* st, uint64_t* keys, uint64_t* keys_hi, uint64_t stride,
+                            double* amps, uint64_t cap, uint64_t* n) {
   {
     sqs_status g = no_capture(st, "sqs_export");
     if (g != SQS_OK) return g;
@@ -3402,7 +3405,7 @@ sqs_status sqs_export(sqs_state* st, uint64_t* keys, double* amps, uint64_t cap,
   *n = cnt;
   if (cnt > cap) return fail(st, SQS_ERR_ARG, "export needs %llu branches", (unsigned long long)cnt);
   if (cnt == 0) return SQS_OK;
-  if (!keys || !amps) return fail(st, SQS_ERR_ARG, "null buffers");
+  if (!keys || !amps || (st->kw == 2 && !keys_hi)) return fail(st, SQS_ERR_ARG, "null buffers");
   // Ascending keys: a sorted copy (the state keeps its own order).  States
   // of 2^32 or more branches are copied in storage order.
   Store* src = nullptr;
@@ -3417,12 +3420,15 @@ sqs_status sqs_export(sqs_state* st, uint64_t* keys, double* amps, uint64_t cap,
     src = &st->cur;
   }
   cudaError_t e;
-  if (st->kw == 1) {
+  if (stride == 1) {
     e = cudaMemcpyAsync(keys, src->k0, cnt * 8, cudaMemcpyDeviceToHost, st->stream);
+    if (e == cudaSuccess && st->kw == 2)
+      e = cudaMemcpyAsync(keys_hi, src->k1, cnt * 8, cudaMemcpyDeviceToHost, st->stream);
   } else {
-    e = cudaMemcpy2DAsync(keys, 16, src->k0, 8, 8, cnt, cudaMemcpyDeviceToHost, st->stream);
-    if (e == cudaSuccess)
-      e = cudaMemcpy2DAsync(keys + 1, 16, src->k1, 8, 8, cnt, cudaMemcpyDeviceToHost,
+    e = cudaMemcpy2DAsync(keys, 8 * stride, src->k0, 8, 8, cnt, cudaMemcpyDeviceToHost,
+                          st->stream);
+    if (e == cudaSuccess && st->kw == 2)
+      e = cudaMemcpy2DAsync(keys_hi, 8 * stride, src->k1, 8, 8, cnt, cudaMemcpyDeviceToHost,
                             st->stream);
   }
   if (e == cudaSuccess) {
@@ -3439,6 +3445,16 @@ sqs_status sqs_export(sqs_state* st, uint64_t* keys, double* amps, uint64_t cap,
   }
   if (e != cudaSuccess) return cuda_fail(st, e, "export");
   return sync_ctl(st);  // waits; a sort that gave up is an error, not an export
+}
+
+sqs_status sqs_export(sqs_state* st, uint64_t* keys, double* amps, uint64_t cap, uint64_t* n) {
+  const uint64_t stride = st && st->kw == 2 ? 2 : 1;
+  return export_to(st, keys, keys ? keys + 1 : nullptr, stride, amps, cap, n);
+}
+
+sqs_status sqs_export_split(sqs_state* st, uint64_t* keys_lo, uint64_t* keys_hi, double* amps,
+                            uint64_t cap, uint64_t* n) {
+  return export_to(st, keys_lo, keys_hi, 1, amps, cap, n);
 }
 
 sqs_status sqs_import(sqs_state* st, const uint64_t* keys, const double* amps, uint64_t n) {

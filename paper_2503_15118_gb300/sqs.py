@@ -9,6 +9,7 @@ built, importing the binding raises: there is no CPU fallback.
 from __future__ import annotations
 
 import ctypes
+import importlib.util
 import os
 
 import numpy as np
@@ -115,6 +116,7 @@ SIGNATURES = {
     "sqs_nnz": (_S, [_P, _UP]),
     "sqs_peak_nnz": (_S, [_P, _UP]),
     "sqs_export": (_S, [_P, _UP, _DP, _u64, _UP]),
+    "sqs_export_split": (_S, [_P, _UP, _UP, _DP, _u64, _UP]),
     "sqs_import": (_S, [_P, _UP, _DP, _u64]),
     "sqs_sync": (_S, [_P]),
     "sqs_flush": (_S, [_P]),
@@ -142,6 +144,7 @@ SIGNATURES = {
 }
 
 _lib = None
+_walk = None  # the native gate-list walker, when it was built
 
 
 def library_path():
@@ -161,6 +164,11 @@ def load(build_if_missing=True):
         f = getattr(lib, name)
         f.restype = res
         f.argtypes = args
+    global _walk
+    if os.path.exists(_build.WALK):
+        spec = importlib.util.spec_from_file_location("sqs_walk", _build.WALK)
+        _walk = importlib.util.module_from_spec(spec)
+        spec.loader.exec_module(_walk)
     _lib = lib
     return lib
 
@@ -397,7 +405,7 @@ class State:
 
     def probabilities(self, reg, with_probs=True):
         w = self.widths[reg]
-        probs = np.zeros(2 ** w if with_probs else 1, np.float64)
+        probs = np.empty(2 ** w if with_probs else 1, np.float64)
         n2 = ctypes.c_double()
         self._chk(self.lib.sqs_probabilities(self.h, reg,
                                              probs.ctypes.data_as(_DP) if with_probs else None,
@@ -411,19 +419,27 @@ class State:
     def probabilities_sparse(self, reg):
         """(values, probs, norm2): the distinct values of register ``reg``
         ascending and the summed |a|^2 of each (sqs_probabilities_sparse)."""
+        # At most one value per branch and per setting of the register: room for
+        # that many (pages nothing is written to cost nothing), unless it is far
+        # more than is likely needed; then the count is asked for first.
+        w = self.widths[reg] if 0 <= reg < len(self.widths) else 64
+        cap = min(self.nnz(), 1 << min(w, 62))
         cnt = ctypes.c_uint64()
         n2 = ctypes.c_double()
-        st = self.lib.sqs_probabilities_sparse(self.h, reg, None, None, 0, ctypes.byref(cnt),
-                                               ctypes.byref(n2))
-        if st not in (OK, ERR_ARG):
-            self._chk(st)
-        c = int(cnt.value)
-        vals = np.zeros(max(c, 1), np.uint64)
-        probs = np.zeros(max(c, 1), np.float64)
+        if cap > 1 << 26:
+            st = self.lib.sqs_probabilities_sparse(self.h, reg, None, None, 0, ctypes.byref(cnt),
+                                                   ctypes.byref(n2))
+            if st not in (OK, ERR_ARG):
+                self._chk(st)
+            cap = int(cnt.value)
+        vals = np.empty(max(cap, 1), np.uint64)
+        probs = np.empty(max(cap, 1), np.float64)
         self._chk(self.lib.sqs_probabilities_sparse(self.h, reg, vals.ctypes.data_as(_UP),
-                                                    probs.ctypes.data_as(_DP), c,
+                                                    probs.ctypes.data_as(_DP), cap,
                                                     ctypes.byref(cnt), ctypes.byref(n2)))
         c = int(cnt.value)
+        if c < cap // 2:
+            return vals[:c].copy(), probs[:c].copy(), float(n2.value)
         return vals[:c], probs[:c], float(n2.value)
 
     def export(self):
@@ -433,15 +449,14 @@ class State:
         if st not in (OK, ERR_ARG):
             self._chk(st)
         cnt = int(n.value)
-        keys = np.zeros(max(cnt, 1) * self.kw, np.uint64)
-        amps = np.zeros(2 * max(cnt, 1), np.float64)
-        self._chk(self.lib.sqs_export(self.h, keys.ctypes.data_as(_UP), amps.ctypes.data_as(_DP),
-                                      cnt, ctypes.byref(n)))
+        lo = np.empty(max(cnt, 1), np.uint64)
+        hi = np.empty(max(cnt, 1), np.uint64) if self.kw == 2 else np.zeros(cnt, np.uint64)
+        amps = np.empty(2 * max(cnt, 1), np.float64)
+        self._chk(self.lib.sqs_export_split(self.h, lo.ctypes.data_as(_UP),
+                                            hi.ctypes.data_as(_UP) if self.kw == 2 else None,
+                                            amps.ctypes.data_as(_DP), cnt, ctypes.byref(n)))
         cnt = int(n.value)
-        keys = keys[: cnt * self.kw].reshape(cnt, self.kw)
-        lo = keys[:, 0].copy()
-        hi = keys[:, 1].copy() if self.kw == 2 else np.zeros(cnt, np.uint64)
-        return lo, hi, amps[: 2 * cnt].view(np.complex128)
+        return lo[:cnt], hi[:cnt], amps[: 2 * cnt].view(np.complex128)
 
     def to_dict(self):
         lo, hi, a = self.export()
@@ -523,9 +538,29 @@ class State:
 
     def run(self, circ, upto=None):
         tables = circ.get("tables", ())
-        for g in circ["gates"] if upto is None else circ["gates"][:upto]:
-            self.apply(g, tables)
+        gates = circ["gates"] if upto is None else circ["gates"][:upto]
+        if _walk is None or type(self) is not State or type(gates) not in (list, tuple):
+            for g in gates:
+                self.apply(g, tables)
+            return self
+        # The native walker issues what it takes; a gate that it leaves (a
+        # matrix, a table not on the device yet, anything unusual) goes through
+        # apply(), and the walk continues after it.
+        i = 0
+        while i < len(gates):
+            i, status = _walk.run(self.h.value or 0, gates, i, self._handles(tables))
+            self._chk(status)
+            if i < len(gates):
+                self.apply(gates[i], tables)
+                i += 1
         return self
+
+    def _handles(self, tables):
+        """Device handles of the tables uploaded so far (None for the others)."""
+        if not isinstance(tables, (list, tuple)):
+            return ()
+        known = (self._tables.get(id(t)) for t in tables)
+        return tuple(k and k[0].value for k in known)
 
 
 class Graph:
