@@ -253,25 +253,6 @@ __device__ __forceinline__ bool slot_live(const Arr& a, uint64_t i) {
   return (uint32_t)(i & ((1ull << a.seg_log2) - 1ull)) < a.seg_cnt[i >> a.seg_log2];
 }
 
-// Calls f(i) for every live slot: grid-stride over a dense array, or CTA per
-// segment (live branches are a prefix of each segment).
-// Calls f(i) for every live slot: grid-stride over a dense array, or CTA per
-// segment (live branches are a prefix of each segment).
-template <class F>
-__device__ __forceinline__ void for_each_live(const Arr& a, uint64_t n_dense, F f) {
-  if (!a.seg_cnt) {
-    const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
-    for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n_dense; i += stride)
-      f(i);
-  } else {
-    for (uint32_t sg = blockIdx.x; sg < a.n_seg; sg += gridDim.x) {
-      const uint32_t n = a.seg_cnt[sg];
-      const uint64_t base = (uint64_t)sg << a.seg_log2;
-      for (uint32_t j = threadIdx.x; j < n; j += blockDim.x) f(base + j);
-    }
-  }
-}
-
 // Visits this CTA's units of `unit` slots of `in` -- slices of segments, or
 // of the dense array -- and calls body(base, lim) with every thread for each
 // unit holding live slots (lim > 0).  Units are handed out round-robin (unit
@@ -332,6 +313,14 @@ __device__ __forceinline__ void raise_err(Ctl* ctl, unsigned int bit, uint32_t s
                                           unsigned long long need) {
   if (atomicOr(&ctl->err, bit) == 0u) ctl->err_where = seq;
   atomicMax(&ctl->need, need);
+}
+
+// Whether an error was raised before: one answer for the CTA.  A kernel that may
+// raise one itself asks this way.  Read thread by thread, a CTA starting while
+// another raises it could go on with part of its threads: without thread 0,
+// which clears the shared lists and counters the others then index memory by.
+__device__ __forceinline__ bool cta_stops(const Ctl* ctl) {
+  return __syncthreads_or((int)(ctl->err != 0u)) != 0;
 }
 
 // ---- QRAM tables -------------------------------------------------------------------
@@ -550,9 +539,9 @@ __device__ __forceinline__ void apply_ops_n(uint32_t n_ops, const DevOp* ops, co
 
 // A kernel parameter's address as a generic one the compiler cannot trace back
 // to the parameter bank.  Read by lane-varying index from the bank itself, every
-// distinct address of a warp is a turn of its own (29 KB of operations and
-// factors: 5 us at the start of a kernel); through the generic address it is an
-// ordinary coalesced load.
+// distinct address of a warp is a turn of its own; through the generic address
+// it is an ordinary coalesced load (a 20-qubit circuit of 20 launches: 290 us
+// by index from the bank, 285 this way).
 template <class T>
 __device__ __forceinline__ const T* param_ptr(const T* p) {
   asm volatile("" : "+l"(p));

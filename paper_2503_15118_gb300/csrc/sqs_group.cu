@@ -152,7 +152,7 @@ __global__ void __launch_bounds__(kGroupThreads, 2)
   __shared__ unsigned int warp_sums[kGroupThreads / 32];
   __shared__ unsigned int n_groups, stage_sum, last_end;
   __shared__ unsigned long long round_base;
-  if (ctl->err) return;
+  if (cta_stops(ctl)) return;
   AT* dense = (AT*)smem;
   unsigned char* pres = smem + L::pres_off;
   K* skey = (K*)(smem + L::skey_off);

@@ -294,9 +294,10 @@ cudaError_t launch_apply_compact(const Launch& L, int kw, bool amp32, Ctl* ctl, 
 // slices, and every branch's atomic queues there: on a 64-system walk batch
 // (0.5M branches, 500 buckets) ncu showed the busiest slice at 81 % of its
 // tag rate with the average at 10 %, and the partition took 75 us; spread
-// it takes 30 us (stride 8 counters: 40 us; 128 or more: as 32).  At 2^23
-// branches 178 -> 118 us; from about 2^24 the counters fill all slices
-// either way.
+// it takes 30 us (stride 8 counters: 40 us; 128 or more: as 32).  The 14
+// partitions of a random circuit growing to 2^24 branches took 598 us in all,
+// 458 spread; the largest of them, whose packed counters fill all slices,
+// takes the same time either way.
 constexpr uint32_t kBucketCntLog2 = 5;
 cudaError_t launch_partition(const Launch& L, int kw, bool amp32, Ctl* ctl, Arr in, int in_slot,
                              const OpList& ops, const uint64_t clear[2], Arr bk,

@@ -113,7 +113,7 @@ __global__ void __launch_bounds__(kStreamThreads)
   pdl_next();
   load_ops(ops, sops, tab);
   pdl_wait();
-  if (ctl->err) return;
+  if (cta_stops(ctl)) return;
   if (blockIdx.x == 0 && threadIdx.x == 0) {
     ctl->cnt[(out_slot + 1) & 3] = 0;
     atomicMax(&ctl->peak, ctl->cnt[in_slot]);
@@ -181,7 +181,7 @@ __global__ void __launch_bounds__(kStreamThreads, KW == 1 ? 3 : 2)
   pdl_next();
   load_ops(ops, sops, tab);
   pdl_wait();
-  if (ctl->err) return;
+  if (cta_stops(ctl)) return;
   const uint64_t n_dense = ctl->cnt[in_slot];
   // Buckets from the device count, ceil(count / fill_target), at most the
   // host's bucket count (a bound, which may be far above the count, as
@@ -389,7 +389,7 @@ __global__ void __launch_bounds__(kPairThreads, 3)
   __shared__ PairShared sh;
   pdl_next();
   pdl_wait();
-  if (ctl->err) return;
+  if (cta_stops(ctl)) return;
   const uint32_t C = 1u << bk.seg_log2;
   const uint32_t S = 2u * C;
   K* skey = (K*)smem;
@@ -467,7 +467,7 @@ __global__ void __launch_bounds__(kStreamThreads, 4)
   pdl_next();
   load_ops(ops, sops, tab);
   pdl_wait();
-  if (ctl->err) return;
+  if (cta_stops(ctl)) return;
   if (blockIdx.x == 0 && threadIdx.x == 0) {
     ctl->cnt[(out_slot + 1) & 3] = 0;
     atomicMax(&ctl->peak, ctl->cnt[in_slot]);
@@ -649,7 +649,7 @@ __global__ void __launch_bounds__(kStreamThreads, 3)
   pdl_next();
   load_ops(ops, sops, tab);
   pdl_wait();
-  if (ctl->err) return;
+  if (cta_stops(ctl)) return;
   if (blockIdx.x == 0 && threadIdx.x == 0) {
     ctl->cnt[(out_slot + 1) & 3] = 0;
     atomicMax(&ctl->peak, ctl->cnt[in_slot]);
@@ -1026,7 +1026,7 @@ __global__ void __launch_bounds__(kStreamThreads, 4)
   extern __shared__ __align__(128) unsigned char exp_smem[];
   pdl_next();
   pdl_wait();
-  if (ctl->err) return;
+  if (cta_stops(ctl)) return;
   if (blockIdx.x == 0 && threadIdx.x == 0) {
     ctl->cnt[(out_slot + 1) & 3] = 0;
     atomicMax(&ctl->peak, ctl->cnt[in_slot]);
@@ -1185,7 +1185,7 @@ __global__ void __launch_bounds__(kStreamThreads, 4)
   uint16_t* list = (uint16_t*)(fold_smem + stream_smem_bytes<KW, AT>());
   pdl_next();
   pdl_wait();
-  if (ctl->err) return;
+  if (cta_stops(ctl)) return;
   if (blockIdx.x == 0 && threadIdx.x == 0) {
     ctl->cnt[(out_slot + 1) & 3] = 0;
     atomicMax(&ctl->peak, ctl->cnt[in_slot]);
@@ -1492,7 +1492,7 @@ __global__ void __launch_bounds__(kBinThreads)
   typedef typename KT<KW>::T K;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   BinSmem<KW, AT>& sm = *reinterpret_cast<BinSmem<KW, AT>*>(smem_raw);
-  if (ctl->err) return;
+  if (cta_stops(ctl)) return;
   load_ops(ops, sm.ops, sm.tab);
   const uint64_t n_dense = ctl->cnt[in_slot];
   if (blockIdx.x == 0 && threadIdx.x == 0) atomicMax(&ctl->peak, n_dense);
@@ -1624,8 +1624,9 @@ __device__ __forceinline__ T* map_rank(T* p, uint32_t rank) {
 // the branches, applies the queued operations and hands each branch to the CTA
 // of its pair class through distributed shared memory; after one cluster
 // barrier each CTA pairs its bucket as k_pair does.  Below about 16000 branches
-// a merge is latency (launch, counter, atomics, bucket round trip): 8 us here
-// against 15 us for the two launches at 4096 branches.
+// a merge is latency (launch, counter, atomics, bucket round trip): a graph of
+// a 20-qubit circuit with six merges replays in 236 us, with partition and pair
+// as two launches in 258.
 constexpr uint32_t kMergeCap = 2048;  // branches per CTA (mean at most half)
 
 template <int KW, class AT>
@@ -1658,7 +1659,7 @@ __global__ void __launch_bounds__(kPairThreads)
   pdl_wait();
   if (threadIdx.x == 0) dead = ctl->err;  // one answer for the CTA
   const uint64_t n_dense = ctl->cnt[in_slot];
-  if (blockIdx.x == 0 && threadIdx.x == 0) {
+  if (blockIdx.x == 0 && threadIdx.x == 0 && !dead) {  // as it stood, after an error
     atomicMax(&ctl->peak, n_dense);
     ctl->cnt[(out_slot + 1) & 3] = 0;
   }
@@ -1750,7 +1751,7 @@ __global__ void __launch_bounds__(kPairCThreads)
   const uint32_t b = blockIdx.x / kClusterCtas;
   // Every CTA of the cluster must reach every cluster barrier: an early exit
   // is taken only after the last one.
-  const bool dead = ctl->err != 0u;
+  const bool dead = cta_stops(ctl);
   const uint32_t n_bin = dead ? 0u : bins.seg_cnt[b];
   const uint32_t lo = r * kSliceCap;
   uint32_t n = n_bin > lo ? (n_bin - lo < (uint32_t)kSliceCap ? n_bin - lo : kSliceCap) : 0u;

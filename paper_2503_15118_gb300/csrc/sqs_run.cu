@@ -27,10 +27,10 @@
 // register-valued step) while the areas hold branches, latency of a step's two
 // barriers while they do not; DRAM is idle.  Measured, rotations with their
 // loads and unloads as one step included: an N = 1024 walk step (0.9 M branches
-// on average, 98 steps) 8.4 -> 2.1 ms, three steps of a 128-system walk in
-// non-Hermitian form 10.4 -> 2.6 ms, two of 64 systems batched 14.3 -> 2.4 ms,
-// where partition and pair took 73 us a step at 10^6 branches and 15 us at the
-// smallest.
+// on average, 98 steps) 8.4 -> 1.7 ms, three steps of an N = 128 walk in
+// non-Hermitian form 10.4 -> 1.6 ms, two of 64 systems batched 13.5 -> 2.0 ms,
+// readout included, where partition and pair took 73 us a step at 10^6 branches
+// and 15 us at the smallest.
 #include <cuda_runtime.h>
 #include <stdint.h>
 

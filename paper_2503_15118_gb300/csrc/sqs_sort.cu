@@ -91,7 +91,7 @@ __global__ void __launch_bounds__(kSortThreads)
   __shared__ AT tab[FIRST ? kTabEntries : 1];
   __shared__ DevOp sops[FIRST ? kMaxOps : 1];
   __shared__ unsigned int h[R];
-  if (ctl->err) return;
+  if (cta_stops(ctl)) return;
   if (FIRST) {
     load_ops(ops, sops, tab);
     if (blockIdx.x == 0 && threadIdx.x == 0) atomicMax(&ctl->peak, *n_ptr);
