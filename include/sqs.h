@@ -92,26 +92,31 @@ typedef enum {
 #define SQS_FUSE_OFF 128u         /* run every interference step alone.  By
                                      default (exact sizing, SQS_MERGE_AUTO or
                                      SQS_MERGE_TUNED) interference steps issued
-                                     back to back on distinct target qubits,
-                                     with no other operation queued between
-                                     them and no step's controls or angle
-                                     register on another step's target, are
-                                     held and executed together when the run
-                                     ends (Sec. II.D.2: each coherent group --
-                                     the branches equal on every other qubit --
-                                     is transformed as one vector of up to
-                                     2^k entries, k <= 12).  The result is
-                                     bit-identical to the steps run one by
-                                     one, peak count included.  Runs end at
-                                     the next operation of another kind that
-                                     must execute, any read, sqs_flush, or
-                                     when they reach 12 steps.  A held run
-                                     executes fused when that is estimated to
-                                     move less memory (sort passes plus the
-                                     group pass against a scatter and a merge
-                                     pass per step, one pass per constant-bit
-                                     expansion) on at least 2^14 branches;
-                                     otherwise its steps run one by one.     */
+                                     back to back are held and executed
+                                     together when the run ends (Sec. II.D.2:
+                                     each coherent group -- the branches equal
+                                     on every other qubit -- is transformed as
+                                     one vector of up to 2^k entries, k <= 12).
+                                     The result is bit-identical to the steps
+                                     run one by one, peak count included.
+                                     A run executes in one of three forms:
+                                     - addressed, while at most 24 key bits
+                                       vary: every branch has a slot of its
+                                       own; targets may repeat, steps may read
+                                       other steps' targets, and one diagonal
+                                       phase may lie between two steps;
+                                     - bucketed, on a state with more varying
+                                       bits: the same, up to 5 targets;
+                                     - sorted: distinct targets, none read by
+                                       another step, nothing between them.
+                                     Runs end at the next operation of another
+                                     kind that must execute, any read,
+                                     sqs_flush, or when they are full.  A run
+                                     executes in the form that is estimated to
+                                     take the fewest launches and passes over
+                                     the state; where none beats its steps, or
+                                     memory for it is refused, they run one by
+                                     one.                                    */
 #define SQS_FUSE_ALWAYS 256u      /* execute every held run of two or more
                                      steps fused, whatever its size and
                                      estimated cost (exercises the fused path
@@ -489,6 +494,9 @@ sqs_status sqs_state_read_records(sqs_state* st, float* X, float* y, uint32_t ca
  * QRAM tables and rotation tables exist).  Learned sizing and the sort,
  * cluster and measured merges cannot be captured, nor can a state created on
  * the legacy default stream (SQS_ERR_ARG).
+ * Of the fused runs (SQS_FUSE_OFF) only the addressed form is captured, where
+ * its slots fit what sqs_capture_begin reserved (2^20 slots, or eight per
+ * branch of the bound); other runs take their steps one by one.
  * sqs_capture_end closes the capture, instantiates the graph into *out and
  * leaves the state at |0...0> (nothing was run).  On failure nothing is
  * returned and the state is usable.

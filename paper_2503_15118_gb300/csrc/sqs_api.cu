@@ -1600,12 +1600,28 @@ void build_run(sqs_state* st, const std::vector<sqs_state::Held>& run, const uin
   }
 }
 
+// No memory for a run's buffers: gives back what it got and runs the operations
+// packed for its first kernel, so that the steps, which need less, can follow
+// one by one.
+sqs_status no_room(sqs_state* st) {
+  if (st->capturing || st->captured)  // a graph holds the buffers
+    return st->sticky = fail(st, SQS_ERR_OOM, "cannot allocate the buffers of a fused run");
+  free_store(st, st->alt);
+  free_store(st, st->bk);
+  dfree(st, st->slot_amp);
+  dfree(st, st->slot_pres);
+  st->slot_amp = st->slot_pres = nullptr;
+  st->slot_cap = 0;
+  return st->ops_buf.n ? run_list(st, st->ops_buf) : SQS_OK;
+}
+
 // The held run (k targets) by direct addressing: the queued operations and
 // the scatter of every branch to its slot, then every group transformed in
 // shared memory.  No host wait: the output holds at most one branch per slot,
-// or 2^k per input branch.
+// or 2^k per input branch.  *taken stays false, with only the queued operations
+// run, when there is no memory for the slots or that output.
 sqs_status run_slots(sqs_state* st, const std::vector<sqs_state::Held>& run,
-                     const uint64_t tmask[2]) {
+                     const uint64_t tmask[2], bool& taken) {
   TraceCall attribution(st, run[0].g.issue_call);
   sqs_status s = run_pending(st, true);  // leaves the fused operations in ops_buf
   if (s != SQS_OK) return st->sticky = s;
@@ -1621,13 +1637,10 @@ sqs_status run_slots(sqs_state* st, const std::vector<sqs_state::Held>& run,
   prog.area_log2 = sqs::run_area_log2(k);
   prog.n_areas = bits > prog.area_log2 ? 1u << (bits - prog.area_log2) : 1u;
   const uint64_t want = (uint64_t)prog.n_areas << prog.area_log2;
-  if (!ensure_slots(st, want))
-    return st->sticky = fail(st, SQS_ERR_OOM, "cannot allocate %llu slots",
-                             (unsigned long long)want);
   const uint64_t grown = st->ub > (slots >> k) ? slots : st->ub << k;
-  if (st->alt.cap < grown && !ensure_store(st, st->alt, grown))
-    return st->sticky = fail(st, SQS_ERR_OOM, "cannot allocate %llu branches",
-                             (unsigned long long)grown);
+  taken = ensure_slots(st, want) &&
+          (st->alt.cap >= grown || ensure_store(st, st->alt, grown));
+  if (!taken) return no_room(st);
   st->alt.set_dense();
   const uint64_t in_slots = st->cur.slots(st->ub);
   const int out_slot = (st->cur_slot + 1) & 3;
@@ -1657,9 +1670,10 @@ sqs_status run_slots(sqs_state* st, const std::vector<sqs_state::Held>& run,
 
 // Steps on few targets over hash buckets (k_partition with the targets cleared,
 // k_bucket_run): any state, whatever its keys.  *taken stays false, with
-// nothing done, when the output -- up to 2^k branches per input branch -- would
-// need more memory than it should: a quarter of what is free, or, after a graph
-// capture, any move of the buffers.
+// nothing but the queued operations done, when the output -- up to 2^k branches
+// per input branch -- would need more memory than it should: a quarter of what
+// is free, more than the allocator gives, or, after a graph capture, any move
+// of the buffers.
 sqs_status run_bucketed(sqs_state* st, const std::vector<sqs_state::Held>& run,
                         const uint64_t tmask[2], bool& taken) {
   taken = false;
@@ -1701,9 +1715,10 @@ sqs_status run_bucketed(sqs_state* st, const std::vector<sqs_state::Held>& run,
   if (s != SQS_OK) return st->sticky = s;
   const uint64_t out_need = grown(), B = buckets();
   if ((st->bk.cap < (B << kBucketLog2) && !ensure_store(st, st->bk, B << kBucketLog2)) ||
-      (st->alt.cap < out_need && !ensure_store(st, st->alt, out_need)))
-    return st->sticky = fail(st, SQS_ERR_OOM, "cannot allocate %llu branches",
-                             (unsigned long long)out_need);
+      (st->alt.cap < out_need && !ensure_store(st, st->alt, out_need))) {
+    taken = false;
+    return no_room(st);
+  }
   sqs::SlotMap map;
   build_run(st, run, tmask, nullptr, map);
   st->bk.set_segments(kBucketLog2, (uint32_t)B);
@@ -1851,12 +1866,9 @@ sqs_status flush_run(sqs_state* st) {
     if (!fits() && !st->capturing) s = sync_bound(st);
     addressed = s == SQS_OK && fits();
   }
-  if (s != SQS_OK) {
-  } else if (addressed) {
-    s = run_slots(st, run, tmask);
-  } else {
-    s = run_pieces(st, run, slot_bits > (int)sqs::kMaxSlotBits);
-  }
+  bool taken = false;
+  if (s == SQS_OK && addressed) s = run_slots(st, run, tmask, taken);
+  if (s == SQS_OK && !taken) s = run_pieces(st, run, slot_bits > (int)sqs::kMaxSlotBits);
   if (st->pending.empty()) st->pending.swap(after);
   else st->pending.insert(st->pending.end(), after.begin(), after.end());
   return s;
