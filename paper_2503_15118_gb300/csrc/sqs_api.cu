@@ -2235,8 +2235,9 @@ void set_load_field(sqs_state* st, const HostOp& h, bool before) {
 // Issues an interference step.  A register-valued rotation right after a QRAM
 // load into its angle register commutes with the load when no entry of the
 // table depends on the target qubit (a rotation angle looked up at an address
-// that the rotated qubit is no part of, or at a prefix): the step then reads
-// the entry itself (Gate1::atab), and the load stays queued past it, where
+// that the rotated qubit is no part of, or at a prefix) and no control sits in
+// the loaded register (it asks for the bit that the load leaves): the step then
+// reads the entry itself (Gate1::atab), and the load stays queued past it, where
 // the unload that usually follows cancels it (qram()).  A load, a rotation
 // and an unload are then one step that writes the target bit only: nothing
 // is queued before it, and the angle register stays known constant.
@@ -2246,8 +2247,11 @@ sqs_status issue_branching(sqs_state* st, const Gate1& g_in, uint32_t n_ctrl) {
   const HostOp load = st->pending.back();
   const DevOp& d = load.d;
   const uint32_t q = g_in.t - d.src_off;  // address bit of the target (wraps when below)
+  bool reads_data = false;  // some control bit is one that the load writes
+  for (uint32_t b = 0; b < g_in.ang_w; ++b) reads_data |= ctrl_touches(g_in.cmask, g_in.ang_off + b);
   if (d.kind != sqs::OP_QRAM || d.pmask[0] || d.pmask[1] || d.dst_off != g_in.ang_off ||
-      d.dst_w != g_in.ang_w || (g_in.t >= d.src_off && q < d.src_w && ((load.varies >> q) & 1ull)))
+      d.dst_w != g_in.ang_w || reads_data ||
+      (g_in.t >= d.src_off && q < d.src_w && ((load.varies >> q) & 1ull)))
     return issue_step(st, g_in, n_ctrl);
   Gate1 g = g_in;
   g.atab = d.table;

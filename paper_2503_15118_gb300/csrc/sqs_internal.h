@@ -199,8 +199,8 @@ struct Gate1 {            // the interference operation of one merge step
   // Mode 1, rotation between a QRAM load into the angle register and its
   // unload: the angle value is the register XOR the word the load would have
   // put there, entry `address field` of atab (0 past its end).  The host sets
-  // it only when no entry depends on the target bit, so that the load commutes
-  // with the step.  null: the register alone.
+  // it only when no entry depends on the target bit and no control reads the
+  // register, so that the load commutes with the step.  null: the register alone.
   const void* atab;
   uint64_t atab_n;
   uint32_t atab_off, atab_w, atab_bytes;
