@@ -2167,24 +2167,23 @@ void note_branch(sqs_state* st, const Gate1& g) {
 // of its target (every branch's partner present with +-1 times its
 // amplitude, tracked the same way whatever merge path runs), which also
 // guarantees that no queued operation reads or writes the target.  The
-// queued operations must not write a control bit or an angle bit of the
-// step, and none may prune.  The step is linear on the amplitudes of each
-// pair and the operations permute keys and multiply amplitudes without
-// touching the pair's bit, so the two orders give the same state; applied
-// after the step, the operations stream half as many branches or fewer.
+// queued operations must not write a bit that the step reads (a control, an
+// angle bit, an address bit of a table it looks up itself), and none may
+// prune.  The step is linear on the amplitudes of each pair and the operations
+// permute keys and multiply amplitudes without touching the pair's bit, so the
+// two orders give the same state; applied after the step, the operations
+// stream half as many branches or fewer.
 // Off in learned-sizing mode, whose queued steps carry their own operations.
 bool defer_ops_ok(const sqs_state* st, const Gate1& g) {
   // The operations queued now are those between this step and anything held
   // before it (a held run keeps its own preceding operations), whatever the
-  // merge path, so the decision is the same in every mode.
+  // merge path, so the decision is the same in every mode -- but for a step
+  // that reads its table itself: under SQS_MERGE_PLAIN the load stays queued
+  // before it and, writing its angle register, keeps it from being passed.
   if (st->pair_sign[g.t] == 0 || st->pending.empty()) return false;
   if (st->flags & SQS_SIZING_LEARNED) return false;
-  uint64_t guard[2] = {g.cmask[0], g.cmask[1]};
-  if (g.mode == 1)
-    for (uint32_t b = 0; b < g.ang_w; ++b) {
-      const uint32_t q = g.ang_off + b;
-      if (q < 128) guard[q >> 6] |= 1ull << (q & 63);
-    }
+  uint64_t guard[2];
+  step_reads(g, guard);
   auto field = [](uint64_t m[2], uint32_t off, uint32_t w) {
     for (uint32_t b = 0; b < w; ++b) {
       const uint32_t q = off + b;

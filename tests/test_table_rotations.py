@@ -64,3 +64,33 @@ def test_controls_on_the_loaded_register(sqs, amp32, value, loaded, before):
                                    ((2, 4, value),)),
               ("ry_reg", 1, 2, 2, 0.05, 0.0, ((2, 0, 1), (0, 1, value))), ("qunload", 0, 2, 0)]
     _check(sqs, widths, gates, [table], amp32)
+
+
+WRITES = {
+    "x": [("x", 0, 1, ())],
+    "cx": [("x", 0, 0, ((3, 1, 1),))],
+    "add": [("add", 0, -1, 3, ())],
+    "sub": [("sub", 0, 3, 0, ())],
+    "swap": [("swap", 0, 4, ())],
+    "load": [("qload", 3, 0, 1)],
+    "x_other": [("x", 4, 0, ()), ("x", 4, 3, ((3, 0, 1),))],
+    "x_ignored": [("x", 0, 3, ())],
+}
+
+
+@pytest.mark.parametrize("amp32", [False, True])
+@pytest.mark.parametrize("write", sorted(WRITES))
+@pytest.mark.parametrize("ctrl", [(), ((4, 2, 1),)])
+def test_folds_after_a_write_to_the_address(sqs, amp32, write, ctrl):
+    """The target is copy-paired (a Hadamard on a constant bit), so that queued
+    operations may wait until after the rotation; those that write its table's
+    address may not.  (Address bit 3 is one that no entry depends on.)"""
+    rng = np.random.default_rng(11)
+    widths = [4, 3, 9, 3, 4]  # address, target, angle, other, other
+    t = rng.integers(0, 512, size=8).astype(np.uint16)
+    tables = [np.concatenate([t, t]), rng.integers(0, 16, size=8).astype(np.uint8)]
+    gates = [("h", 0, b, ()) for b in range(2)] + [("h", 3, b, ()) for b in range(3)]
+    gates += [("h", 4, 2, ()), ("ry", 4, 1, 0.4, ()), ("h", 1, 0, ())]
+    gates += WRITES[write]
+    gates += [("qload", 0, 2, 0), ("ry_reg", 1, 0, 2, 0.013, 0.2, ctrl), ("qunload", 0, 2, 0)]
+    _check(sqs, widths, gates, tables, amp32)
