@@ -275,9 +275,9 @@ struct sqs_state {
   sqs_status capture_err = SQS_OK;
   HostSnap entry_snap;
   uint64_t launches_at_capture = 0;
-  // A graph was captured: it holds the buffers, which eager issue then leaves
-  // where they are as long as the count allows.
-  bool captured = false;
+  // The captured graphs not yet destroyed: they hold the buffers, which eager
+  // issue then leaves where they are as long as the count allows.
+  std::vector<sqs_graph*> graphs;
 
   sqs_stats stats{};
   std::unordered_map<void*, size_t> sizes;
@@ -391,11 +391,11 @@ uint64_t max_branches(const sqs_state* st) {
 }
 
 // Bounds up to this many branches are allocated for without reading the exact
-// count first: a few MB against a host wait per step.  None after a graph
-// capture, whose buffers eager issue leaves in place while the count allows,
+// count first: a few MB against a host wait per step.  None while a captured
+// graph holds the buffers, which eager issue leaves in place as the count allows,
 // nor under the measured merge choice, whose timings complete as it waits.
 uint64_t small_bound(const sqs_state* st) {
-  return st->captured || (st->flags & SQS_MERGE_TUNED) ? 1ull : 1ull << 16;
+  return !st->graphs.empty() || (st->flags & SQS_MERGE_TUNED) ? 1ull : 1ull << 16;
 }
 
 // Branches a state can hold once step g has run: one per setting of the key
@@ -871,7 +871,7 @@ sqs_status run_hashed(sqs_state* st, const Gate1& g, double est_in, int64_t rec_
     uint32_t ctas = 1;
     while (ctas < 16 && (uint64_t)ctas * (kBucketFill / 2) < want) ctas *= 2;
     const uint64_t slots = (uint64_t)ctas << kSegLog2;
-    const bool fixed = st->captured || st->capturing;  // buffers stay where they are
+    const bool fixed = !st->graphs.empty() || st->capturing;  // buffers stay where they are
     if (st->alt.cap >= slots || (!fixed && ensure_store(st, st->alt, slots))) {
       st->alt.set_segments(kSegLog2, ctas);
       const int out_slot = (st->cur_slot + 1) & 3;
@@ -1604,7 +1604,7 @@ void build_run(sqs_state* st, const std::vector<sqs_state::Held>& run, const uin
 // packed for its first kernel, so that the steps, which need less, can follow
 // one by one.
 sqs_status no_room(sqs_state* st) {
-  if (st->capturing || st->captured)  // a graph holds the buffers
+  if (st->capturing || !st->graphs.empty())  // a graph holds the buffers
     return st->sticky = fail(st, SQS_ERR_OOM, "cannot allocate the buffers of a fused run");
   free_store(st, st->alt);
   free_store(st, st->bk);
@@ -1672,8 +1672,8 @@ sqs_status run_slots(sqs_state* st, const std::vector<sqs_state::Held>& run,
 // k_bucket_run): any state, whatever its keys.  *taken stays false, with
 // nothing but the queued operations done, when the output -- up to 2^k branches
 // per input branch -- would need more memory than it should: a quarter of what
-// is free, more than the allocator gives, or, after a graph capture, any move
-// of the buffers.
+// is free, more than the allocator gives, or, while a captured graph holds the
+// buffers, any move of them.
 sqs_status run_bucketed(sqs_state* st, const std::vector<sqs_state::Held>& run,
                         const uint64_t tmask[2], bool& taken) {
   taken = false;
@@ -1699,7 +1699,7 @@ sqs_status run_bucketed(sqs_state* st, const std::vector<sqs_state::Held>& run,
   }
   if (buckets() > 0x7fffffffull) return SQS_OK;
   if (!fits()) {
-    if (st->captured) return SQS_OK;
+    if (!st->graphs.empty()) return SQS_OK;
     size_t free_b = 0, total_b = 0;
     if (cudaMemGetInfo(&free_b, &total_b) != cudaSuccess) {
       cudaGetLastError();
@@ -1854,7 +1854,7 @@ sqs_status flush_run(sqs_state* st) {
   const int slot_bits = bits_set(vary);
   bool addressed = run.size() >= 2 && slot_bits <= (int)sqs::kMaxSlotBits &&
                    slots_pay(st, run, slot_bits);
-  if (addressed && (st->captured || st->capturing)) {
+  if (addressed && (!st->graphs.empty() || st->capturing)) {
     // Output and slots must fit where the graph has them (run_slots would move
     // them).
     const int k = bits_set(tmask);
@@ -2685,7 +2685,7 @@ void put_snap(sqs_state* st, const HostSnap& h) {
 // A captured sequence of calls: the CUDA graph, and the host bookkeeping
 // (buffer roles, count slot and bound, per-qubit history) before and after.
 struct sqs_graph {
-  sqs_state* st = nullptr;
+  sqs_state* st = nullptr;  // null once the state is destroyed
   cudaGraph_t graph = nullptr;
   cudaGraphExec_t exec = nullptr;
   HostSnap entry, exit;
@@ -2858,6 +2858,7 @@ sqs_status sqs_state_create(const uint32_t* reg_widths, uint32_t n_regs, uint32_
 void sqs_state_destroy(sqs_state* st) {
   if (!st) return;
   cudaStreamSynchronize(st->stream);
+  for (sqs_graph* g : st->graphs) g->st = nullptr;
   // Autotuner choices to the cache file: merged with entries other states
   // wrote (this state's measured keys win), written through a temporary file.
   if (const char* path = std::getenv("SQS_TUNE_CACHE")) {
@@ -3660,7 +3661,7 @@ sqs_status sqs_capture_begin(sqs_state* st, uint64_t static_bound) {
     return st->sticky = fail(st, SQS_ERR_OOM, "cannot size buffers for the capture");
   // Slots for addressed runs: up to 2^20 (a circuit of 20 qubits), or eight per
   // branch of the bound; a run over more of them takes its steps one by one.
-  if (fusing(st) && !st->captured) {
+  if (fusing(st) && st->graphs.empty()) {
     uint64_t slots = 1ull << 12;
     while (slots < (1ull << std::min(st->total_bits, sqs::kMaxSlotBits)) &&
            slots < std::max<uint64_t>(1ull << 20, 8 * static_bound))
@@ -3711,7 +3712,7 @@ sqs_status sqs_capture_end(sqs_state* st, sqs_graph** out) {
   g->exit = std::move(exit_snap);
   g->launches = launches;
   *out = g;
-  st->captured = true;
+  st->graphs.push_back(g);
   return SQS_OK;
 }
 
@@ -3739,6 +3740,10 @@ sqs_status sqs_graph_launch(sqs_state* st, sqs_graph* g) {
 
 void sqs_graph_destroy(sqs_graph* g) {
   if (!g) return;
+  if (g->st) {
+    std::vector<sqs_graph*>& live = g->st->graphs;
+    live.erase(std::remove(live.begin(), live.end(), g), live.end());
+  }
   if (g->exec) cudaGraphExecDestroy(g->exec);
   if (g->graph) cudaGraphDestroy(g->graph);
   delete g;
