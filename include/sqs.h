@@ -496,7 +496,8 @@ sqs_status sqs_state_read_records(sqs_state* st, float* X, float* y, uint32_t ca
  * the legacy default stream (SQS_ERR_ARG).
  * Of the fused runs (SQS_FUSE_OFF) only the addressed form is captured, where
  * its slots fit what sqs_capture_begin reserved (2^20 slots, or eight per
- * branch of the bound); other runs take their steps one by one.
+ * branch of the bound, when the allocator has room for them and no live graph
+ * of the state holds slots of its own); other runs take their steps one by one.
  * sqs_capture_end closes the capture, instantiates the graph into *out and
  * leaves the state at |0...0> (nothing was run).  On failure nothing is
  * returned and the state is usable.

@@ -3660,14 +3660,14 @@ sqs_status sqs_capture_begin(sqs_state* st, uint64_t static_bound) {
       !ensure_store(st, st->bk, B << kBucketLog2))
     return st->sticky = fail(st, SQS_ERR_OOM, "cannot size buffers for the capture");
   // Slots for addressed runs: up to 2^20 (a circuit of 20 qubits), or eight per
-  // branch of the bound; a run over more of them takes its steps one by one.
-  if (fusing(st) && st->graphs.empty()) {
+  // branch of the bound; a run over more of them takes its steps one by one, and
+  // so does every run where the allocator has no room for them.
+  if (fusing(st) && (st->graphs.empty() || !st->slot_cap)) {
     uint64_t slots = 1ull << 12;
     while (slots < (1ull << std::min(st->total_bits, sqs::kMaxSlotBits)) &&
            slots < std::max<uint64_t>(1ull << 20, 8 * static_bound))
       slots <<= 1;
-    if (!ensure_slots(st, slots))
-      return st->sticky = fail(st, SQS_ERR_OOM, "cannot size buffers for the capture");
+    ensure_slots(st, slots);
   }
   s = sqs_state_reset(st);  // the state the graph starts from, now
   if (s != SQS_OK) return s;

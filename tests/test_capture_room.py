@@ -84,3 +84,28 @@ def test_graphs_and_states_closed_in_either_order(sqs):
     gb.close()
     b.close()
     gc.close()
+
+
+@pytest.mark.parametrize("amp32", [False, True])
+def test_capture_without_room_for_slots(sqs, monkeypatch, amp32):
+    """The slots of addressed runs are larger than all other buffers of a small
+    bound; where the allocator has none, the captured steps run one by one."""
+    widths = [8, 8, 8]
+    circ = W.random_circuit(widths, 60, seed=5, kinds=("x", "cx", "ry", "phase", "add"))
+    # Rotations back to back, undone again: what an addressed run takes.
+    run = [("ry", 1, b, 0.2 + b, ()) for b in range(4)]
+    circ["gates"] = [("h", 0, b, ()) for b in range(4)] + circ["gates"][:20] + run + \
+        [W.inverse_gate(g) for g in reversed(run)]
+    bound = 1 << 13
+    eager = _state(sqs, widths, amp32=amp32).run(circ)
+    want = eager.to_dict()
+    assert eager.peak_nnz() <= bound
+    given = sqs._TorchAllocator.alloc
+    monkeypatch.setattr(sqs._TorchAllocator, "alloc",
+                        lambda self, ctx, n, s: None if n > 4 << 20 else given(self, ctx, n, s))
+    st = _state(sqs, widths, amp32=amp32)
+    graph = st.capture(circ, bound)
+    for _ in range(2):
+        graph.launch()
+        assert st.to_dict() == want
+    graph.close()
