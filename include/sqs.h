@@ -352,6 +352,10 @@ sqs_status sqs_tune_import(sqs_state* st, const char* json);
  * finish without its slice.  skip_copy_rank >= 0 makes the CTAs of that rank
  * in every cluster issue no copy, so that their wait runs out (a fault
  * injected on the host side of the copy, not on the GPU); -1 turns it off.
+ * The one-launch sort of small states (exports, sparse marginals) takes both
+ * in the same way: its grid barriers poll at most wait_limit times (default
+ * 2^21), and the CTA of that number leaves its arrivals out (no effect on a
+ * sort of fewer CTAs; 2048 branches each).
  * The next waiting call returns SQS_ERR_TIMEOUT; sqs_state_reset makes the
  * state usable again.  For tests only. */
 sqs_status sqs_state_set_wait_test(sqs_state* st, uint32_t wait_limit, int32_t skip_copy_rank);

@@ -253,9 +253,10 @@ struct Launch {
   int sm_count;
   uint32_t seq;        // launch sequence number (error attribution)
   uint64_t n_hint;     // host-side upper bound of the branches streamed (grid size)
-  // Bounded device waits (cluster merge): polls before giving up (0: the
-  // default), and a testing hook -- a cluster rank whose CTAs issue no bulk
-  // copy, so that their wait runs out (-1: none).
+  // Bounded device waits (cluster merge, one-launch sort): polls before giving
+  // up (0: the default), and a testing hook -- a cluster rank whose CTAs issue
+  // no bulk copy, or the CTA of a sort that leaves out its barrier arrivals, so
+  // that the wait runs out (-1: none).
   uint32_t wait_limit = 0;
   int32_t skip_copy_rank = -1;
 };

@@ -318,8 +318,9 @@ __global__ void __launch_bounds__(kSortThreads)
 // A whole LSD sort in one cooperative launch, for states that fit one tile per
 // SM.  Every pass of the kernels above is four launches, each a few microseconds
 // of latency at these sizes.  Here CTA t keeps tile t's branches in registers from its
-// histogram to its scatter, and a grid barrier -- bounded: after kGridWait polls
-// it records an error and the grid returns -- separates the phases.  An export
+// histogram to its scatter, and a grid barrier -- bounded: after wait_limit polls
+// (kGridWait by default) it records an error and the grid returns -- separates the
+// phases.  An export
 // of 65536 one-word branches (8 passes) takes 140 us in place of 276, of 4000
 // branches 130 in place of 252; past one tile per SM the passes above are
 // bound by their traffic.  Same order as the passes above
@@ -331,20 +332,25 @@ struct SmallSort {
   uint32_t shift[kSmallPasses];
 };
 
-// All CTAs of the grid; false (for every thread) when the wait ran out.
+// All CTAs of the grid; false (for every thread) when the wait ran out.  absent:
+// this CTA leaves out its arrivals, so that every CTA's wait runs out (testing).
+struct GridWait {
+  uint32_t limit;
+  bool absent;
+};
 __device__ __forceinline__ bool grid_barrier(unsigned int* bar, unsigned int& phase,
-                                             unsigned int* ok) {
+                                             unsigned int* ok, const GridWait& wait) {
   __syncthreads();
   if (threadIdx.x == 0) {
     ++phase;
     const unsigned int target = phase * gridDim.x;
     __threadfence();
-    atomicAdd(bar, 1u);
+    if (!wait.absent) atomicAdd(bar, 1u);
     uint32_t it = 0;
     unsigned int seen;
     do {
       asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(seen) : "l"(bar) : "memory");
-    } while (seen < target && ++it < kGridWait);
+    } while (seen < target && ++it < wait.limit);
     __threadfence();
     *ok = seen >= target;
   }
@@ -356,9 +362,10 @@ template <int KW, class AT>
 __global__ void __launch_bounds__(kSortThreads)
     k_rsort_small(Ctl* ctl, Arr in, uint64_t n, Arr buf0, Arr buf1, const SmallSort passes,
                   unsigned int* hist, unsigned int* bar, unsigned long long* n_dev, uint32_t seq,
-                  uint64_t cm0, uint64_t cm1, uint32_t t) {
+                  uint64_t cm0, uint64_t cm1, uint32_t t, uint32_t wait_limit, int absent_cta) {
   typedef typename KT<KW>::T K;
   constexpr uint32_t R = 256;
+  const GridWait wait = {wait_limit, (int)blockIdx.x == absent_cta};
   const K cm = mk<KW>(cm0, cm1);
   extern __shared__ __align__(16) unsigned char smem[];
   K* skey = (K*)smem;
@@ -410,7 +417,7 @@ __global__ void __launch_bounds__(kSortThreads)
       }
       __syncthreads();
     }
-    if (!grid_barrier(bar, phase, &ok)) return give_up();
+    if (!grid_barrier(bar, phase, &ok, wait)) return give_up();
     src = &buf1;
   }
   const uint64_t base = (uint64_t)blockIdx.x * kSortTile;
@@ -455,7 +462,7 @@ __global__ void __launch_bounds__(kSortThreads)
       mine += c;
     }
     h[(size_t)blockIdx.x * R + threadIdx.x] = mine;
-    if (!grid_barrier(bar, phase, &ok)) return give_up();
+    if (!grid_barrier(bar, phase, &ok, wait)) return give_up();
     unsigned int before = 0u, total = 0u;
 #pragma unroll 8
     for (uint32_t u = 0; u < T; ++u) {
@@ -502,7 +509,7 @@ __global__ void __launch_bounds__(kSortThreads)
       st_key<KW>(dst, pos, skey[i]);
       ((AT*)dst.amp)[pos] = samp[i];
     }
-    if (p + 1 < passes.n_pass && !grid_barrier(bar, phase, &ok)) return give_up();
+    if (p + 1 < passes.n_pass && !grid_barrier(bar, phase, &ok, wait)) return give_up();
     src = &dst;
   }
 }
@@ -708,8 +715,10 @@ static cudaError_t small_t(const Launch& L, Ctl* ctl, Arr in, uint64_t n, Arr bu
   ps.n_pass = n_pass;
   for (uint32_t p = 0; p < n_pass; ++p) ps.shift[p] = shifts[p];
   uint64_t cm0 = clear_mask ? clear_mask[0] : 0ull, cm1 = clear_mask ? clear_mask[1] : 0ull;
-  uint32_t seq = L.seq;
-  void* args[] = {&ctl, &in, &n, &buf0, &buf1, &ps, &hist, &bar, &n_dev, &seq, &cm0, &cm1, &t};
+  uint32_t seq = L.seq, limit = L.wait_limit ? L.wait_limit : kGridWait;
+  int absent = L.skip_copy_rank;
+  void* args[] = {&ctl, &in,  &n,   &buf0, &buf1, &ps,    &hist,  &bar,
+                  &n_dev, &seq, &cm0, &cm1,  &t,    &limit, &absent};
   const uint64_t grid = (n + kSortTile - 1) / kSortTile;
   return cudaLaunchCooperativeKernel((const void*)k_rsort_small<KW, AT>,
                                      dim3((unsigned)(grid ? grid : 1)), dim3(kSortThreads), args,
