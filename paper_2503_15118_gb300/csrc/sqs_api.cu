@@ -2726,9 +2726,13 @@ sqs_status sort_copy(sqs_state* st, uint64_t n, const uint64_t keep[2], Store** 
     tiles0 = std::max<uint64_t>(1, (n + tile - 1) / tile);
   }
   const uint64_t tilesN = std::max<uint64_t>(1, (n + tile - 1) / tile);
+  const uint32_t npass = (uint32_t)shifts.size();
+  const bool small = rb == 8 && npass <= 16 && n <= sqs::small_sort_max(st->sm_count);
   unsigned int *hist, *part;
   unsigned long long* n_dev;
-  sqs_status s = sort_scratch(st, std::max(tiles0, 2 * tilesN), hist, part, n_dev, rb);
+  // (The one-launch sort keeps the counters of two passes.)
+  sqs_status s = sort_scratch(st, small ? 2 * tilesN : std::max(tiles0, tilesN), hist, part,
+                              n_dev, rb);
   if (s != SQS_OK) return s;
   if ((st->bk.cap < n && !ensure_store(st, st->bk, n)) ||
       (st->alt.cap < n && !ensure_store(st, st->alt, n)))
@@ -2743,10 +2747,8 @@ sqs_status sort_copy(sqs_state* st, uint64_t n, const uint64_t keep[2], Store** 
   Store* buf[2] = {&st->alt, &st->bk};
   const unsigned long long* n_ptr = &st->ctl->cnt[st->cur_slot];
   Arr src = st->cur.view();
-  const uint32_t npass = (uint32_t)shifts.size();
   cudaError_t e = cudaSuccess;
   if (timed) tune_begin(st, tkey);
-  const bool small = rb == 8 && npass <= 16 && n <= sqs::small_sort_max(st->sm_count);
   if (small) {
     // One launch for all passes: latency, not bandwidth, bounds a small sort.
     for (Store* b : buf) b->set_dense();

@@ -1,5 +1,5 @@
 """The one-launch sort of small states at its limits: a grid barrier that runs out is an
-error of the call, not a wrong order."""
+error of the call, not a wrong order, and larger sorts ask for no scratch of its."""
 import time
 
 import numpy as np
@@ -55,3 +55,22 @@ def test_grid_barrier_runs_out_then_recovers(sqs, segmented, read):
     if read == "export" and not segmented:
         assert all(np.array_equal(x, y) for x, y in zip(got, want))
     assert np.array_equal(got[0], want[0])
+
+
+def test_scratch_of_larger_sorts(sqs, monkeypatch):
+    """A sort in passes needs 256 four-byte counters per tile of 2048 branches,
+    and what does not grow with the state (under 128 KB with the bucket counters)."""
+    n = (1 << 19) + 5
+    asked = []
+    given = sqs._TorchAllocator.alloc
+    monkeypatch.setattr(sqs._TorchAllocator, "alloc",
+                        lambda self, ctx, b, s: asked.append(b) or given(self, ctx, b, s))
+    st = sqs.State([30, 30])
+    lo, hi, a = W.random_state([30, 30], n, seed=9)
+    st.import_(lo, hi, a)
+    del asked[:]
+    got = st.export()
+    order = np.argsort(lo)
+    assert np.array_equal(got[0], lo[order]) and np.array_equal(got[2], a[order])
+    scratch = [b for b in asked if b < 8 * n]
+    assert scratch and max(scratch) <= 1024 * ((n + 2047) // 2048) + (128 << 10)
