@@ -539,7 +539,9 @@ class State:
     def run(self, circ, upto=None):
         tables = circ.get("tables", ())
         gates = circ["gates"] if upto is None else circ["gates"][:upto]
-        if _walk is None or type(self) is not State or type(gates) not in (list, tuple):
+        # (A closed state has no handle to walk with: the library refuses its gates.)
+        if (_walk is None or not self.h or type(self) is not State
+                or type(gates) not in (list, tuple)):
             for g in gates:
                 self.apply(g, tables)
             return self
@@ -548,7 +550,7 @@ class State:
         # apply(), and the walk continues after it.
         i = 0
         while i < len(gates):
-            i, status = _walk.run(self.h.value or 0, gates, i, self._handles(tables))
+            i, status = _walk.run(self.h.value, gates, i, self._handles(tables))
             self._chk(status)
             if i < len(gates):
                 self.apply(gates[i], tables)
