@@ -184,8 +184,8 @@ bool issue(sqs_state* st, PyObject* g, PyObject* tables, sqs_status& s) {
     } else if (!a.integer(addr, first)) {
       return false;
     }
-    if (ti < 0 || ti >= PyTuple_GET_SIZE(tables)) return false;
-    PyObject* h = PyTuple_GET_ITEM(tables, (Py_ssize_t)ti);
+    if (ti < 0 || ti >= PyList_GET_SIZE(tables)) return false;
+    PyObject* h = PyList_GET_ITEM(tables, (Py_ssize_t)ti);
     if (!PyLong_CheckExact(h)) return false;  // not on the device yet
     const sqs_table* t = (const sqs_table*)PyLong_AsVoidPtr(h);
     s = call([&] {
@@ -212,12 +212,12 @@ bool issue(sqs_state* st, PyObject* g, PyObject* tables, sqs_status& s) {
 // run(handle, gates, first, tables) -> (index, status): issues gates[first:]
 // until one is not taken here or fails; index is that gate's (len(gates) when
 // all were issued), status the failing call's (0 otherwise).  gates: a list or
-// tuple; tables: a tuple of device table handles, None where there is none yet.
+// tuple; tables: a list of device table handles, None where there is none yet.
 PyObject* run(PyObject*, PyObject* args) {
   unsigned long long handle;
   PyObject *gates, *tables;
   Py_ssize_t first;
-  if (!PyArg_ParseTuple(args, "KOnO!", &handle, &gates, &first, &PyTuple_Type, &tables))
+  if (!PyArg_ParseTuple(args, "KOnO!", &handle, &gates, &first, &PyList_Type, &tables))
     return nullptr;
   if (!PyList_CheckExact(gates) && !PyTuple_CheckExact(gates)) {
     PyErr_SetString(PyExc_TypeError, "gates: a list or a tuple");

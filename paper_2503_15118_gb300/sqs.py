@@ -548,21 +548,25 @@ class State:
         # The native walker issues what it takes; a gate that it leaves (a
         # matrix, a table not on the device yet, anything unusual) goes through
         # apply(), and the walk continues after it.
+        handles = self._handles(tables)
         i = 0
         while i < len(gates):
-            i, status = _walk.run(self.h.value, gates, i, self._handles(tables))
+            i, status = _walk.run(self.h.value, gates, i, handles)
             self._chk(status)
             if i < len(gates):
-                self.apply(gates[i], tables)
+                g = gates[i]
+                self.apply(g, tables)
+                if handles and g[0] in ("qload", "qunload"):  # its table is on the device now
+                    handles[g[3]] = self._tables[id(tables[g[3]])][0].value
                 i += 1
         return self
 
     def _handles(self, tables):
         """Device handles of the tables uploaded so far (None for the others)."""
         if not isinstance(tables, (list, tuple)):
-            return ()
+            return []
         known = (self._tables.get(id(t)) for t in tables)
-        return tuple(k and k[0].value for k in known)
+        return [k and k[0].value for k in known]
 
 
 class Graph:
