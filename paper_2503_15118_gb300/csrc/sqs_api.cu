@@ -3238,7 +3238,7 @@ sqs_status sqs_prune(sqs_state* st, double eps, uint64_t* nnz_out) {
   if (s != SQS_OK) return s;
   if (!(eps >= 0.0) || std::isinf(eps)) return fail(st, SQS_ERR_ARG, "bad eps");
   push_prune(st, eps);
-  s = run_pending(st, false);
+  s = flush_all(st);
   if (s != SQS_OK) return s;
   if (nnz_out) {
     s = sync_ctl(st);
