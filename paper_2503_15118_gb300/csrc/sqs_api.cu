@@ -192,6 +192,17 @@ struct sqs_state {
   // Learned sizing: queued interference steps (with the operations before
   // each), sized at the next flush from one batched inference.
   sqs_predictor* predictor = nullptr;
+  // The state as a queued step's own launches find it.  Operations ahead of the
+  // step that do not fit its launch ran before, in place (`ran` of them): a step
+  // that is run again from here must not apply them again.  run_pending() writes
+  // it to snap_at while run_lazy() runs a step.
+  struct Snap {
+    Store cur, alt, bk;
+    int cur_slot = 0;
+    uint32_t seq = 0;
+    size_t ran = 0;
+  };
+  Snap* snap_at = nullptr;
   struct Lazy {
     Gate1 g;
     std::vector<HostOp> ops;
@@ -700,7 +711,11 @@ sqs_status run_pending(sqs_state* st, bool keep_tail) {
   for (;;) {
     const size_t used = pack_ops(st->pending, from, L);
     const bool last = from + used >= st->pending.size();
-    if (last && keep_tail) break;
+    if (last && keep_tail) {
+      if (st->snap_at)
+        *st->snap_at = {st->cur, st->alt, st->bk, st->cur_slot, st->seq, from};
+      break;
+    }
     sqs_status s = run_list(st, L);
     if (s != SQS_OK) return s;
     from += used;
@@ -2393,12 +2408,7 @@ sqs_status run_lazy(sqs_state* st) {
   std::vector<HostOp> tail;
   tail.swap(st->pending);  // operations queued after the last step
 
-  struct Snap {
-    Store cur, alt, bk;
-    int cur_slot;
-    uint32_t seq;
-  };
-  std::vector<Snap> snaps(n);
+  std::vector<sqs_state::Snap> snaps(n);
   st->defer_frees = true;
   // Estimated count entering each step.  Chained step by step with the
   // quarter-bit margin of grow_factor, and capped one bit plus a margin that
@@ -2437,9 +2447,11 @@ sqs_status run_lazy(sqs_state* st) {
     st->grow_hint_b = (uint64_t)std::min(peak * 1.2 / fill, 0x1p40) + 1;
   }
   for (size_t i = 0; i < n && s == SQS_OK; ++i) {
-    snaps[i] = Snap{st->cur, st->alt, st->bk, st->cur_slot, st->seq};
+    snaps[i] = {st->cur, st->alt, st->bk, st->cur_slot, st->seq, 0};
+    st->snap_at = &snaps[i];
     st->pending = st->lazy[i].ops;
     s = run_branching(st, st->lazy[i].g, est[i]);
+    st->snap_at = nullptr;
   }
   st->stats.learned_steps += n;
   if (s == SQS_OK) s = sync_ctl(st, true);
@@ -2462,7 +2474,8 @@ sqs_status run_lazy(sqs_state* st) {
       cudaMemsetAsync(st->bk.segs, 0, st->bk.seg_entries() * sizeof(unsigned int), st->stream);
     s = sync_ctl(st);  // exact input count of the failed step
     for (size_t i = f; i < n && s == SQS_OK; ++i) {
-      st->pending = st->lazy[i].ops;
+      const std::vector<HostOp>& ops = st->lazy[i].ops;
+      st->pending.assign(ops.begin() + (ptrdiff_t)(i == f ? snaps[f].ran : 0), ops.end());
       s = run_branching(st, st->lazy[i].g);
       st->stats.overflow_reruns++;
     }
