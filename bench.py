@@ -429,8 +429,10 @@ def fp32_error(ref, got):
 
 def time_workload(sqs, circ, hint, amp32, fuse_off, stream, flush, args, hbm, keep=False):
     """Updates/s of one workload in one form (storage type, fused runs on or
-    off), with the HBM-roofline fraction of its interference steps.  With
-    keep, also returns the final state (exported)."""
+    off), with the algorithmic byte rate of its interference steps against HBM
+    (a bandwidth only when no run was fused: the steps of a fused run pass
+    through shared memory, `is_bandwidth`).  With keep, also returns the final
+    state (exported)."""
     st = sqs.State(circ["widths"], capacity_hint=hint, stream=stream.cuda_stream,
                    eps=circ["eps"], amp32=amp32, merge=fuse_off)
     try:
@@ -472,7 +474,9 @@ def time_workload(sqs, circ, hint, amp32, fuse_off, stream, flush, args, hbm, ke
         if tms > 0:
             gbs = byts / (tms / 1e3) / 1e9
             entry["interference_roofline"] = {"achieved": gbs, "peak": hbm, "unit": "GB/s",
-                                              "frac": gbs / hbm, "kernel_ms_per_step": tms}
+                                              "frac": gbs / hbm, "kernel_ms_per_step": tms,
+                                              "is_bandwidth": not any(r[0] == "k_group"
+                                                                      for r in recs)}
         if keep:
             return entry, st.export()
         return entry
