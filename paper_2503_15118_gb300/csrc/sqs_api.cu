@@ -259,8 +259,9 @@ struct sqs_state {
   };
   std::vector<AngTab> ang_tabs;
 
-  // Fused run (exact sizing): interference steps on distinct targets issued
-  // back to back with nothing queued between them, held until the run ends.
+  // Fused run (exact sizing): interference steps issued back to back, held until
+  // the run ends.  Targets may repeat and a step may read other steps' targets;
+  // at most one phase lies between two steps (hold_step has the rules).
   struct Held {
     Gate1 g;
     bool after_phase;  // `phase` (one queued phase) comes between the last step and this one
@@ -1694,8 +1695,9 @@ sqs_status run_bucketed(sqs_state* st, const std::vector<sqs_state::Held>& run,
   taken = false;
   const uint32_t k = (uint32_t)bits_set(tmask);
   // Groups come whole, up to 2^k branches: lower fills than the pair merge's
-  // keep an overflow of the 2048 slots (64 groups where 16 are the mean) as
-  // far away, e^-80 a bucket for k = 4, e^-55 for k = 5.
+  // keep an overflow of the 2048 slots as far away.  Whole groups of 16 (k = 4):
+  // 32 are the mean, 128 fit, more come with e^-80 a bucket; of 32 (k = 5): 12
+  // are the mean, 64 fit, e^-55.
   const uint64_t fill = k <= 4 ? 512 : 384;
   auto grown = [&] {
     uint64_t vary[2];

@@ -1335,8 +1335,8 @@ __global__ void __launch_bounds__(kStreamThreads, 4)
 // a register's value often stays the same over thousands of branches: a thread
 // keeps the sum of its current value and adds it to the bin when the value
 // changes; and below 2^12 bins each has several copies, taken by lane.  The norm
-// is the sum of the bins.  Measured (N = 1024 walk, 4.2e6 branches, marginals of
-// X
+// is the sum of the bins.  Measured: the two marginals at the end of an N = 1024
+// walk step 492 -> 160 us, three marginals of 1.6e7 branches 848 -> 576 us.
 constexpr int kProbThreads = 256;
 constexpr uint32_t kSmemBinsLog2 = 12;
 constexpr uint32_t kBinCopiesLog2 = 3;  // at most 8 copies
