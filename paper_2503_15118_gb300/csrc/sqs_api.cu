@@ -642,12 +642,31 @@ size_t pack_ops(const std::vector<HostOp>& ops, size_t from, OpList& L) {
   return i - from;
 }
 
-// In-place passes of this many operations work on bit planes, over at least a
-// tile of 4096 branches per SM or so: with fewer, whole SMs would idle, and the
-// latency of the operations one after another is the same (4096 branches, 20
-// qubits: 316 us a circuit on planes, 290 branch by branch).
-constexpr uint32_t kPlaneMin = 12;
-constexpr uint64_t kPlaneSlots = 1ull << 19;
+// Whether an in-place pass pays on bit planes.  A branch's way into planes and
+// back costs about what twelve X cost branch by branch, and a factor table some
+// more: its index goes through a transposition of its own, with the same FP64
+// products on either side.  And the tiles of 4096 branches have to fill the SMs
+// often enough that their long chains overlap, with a table more so, most of all
+// where a key word's planes leave room for six CTAs an SM only.  Measured (us a
+// pass, branch by branch / planes; 64-bit, 32-bit, 84-bit keys; a list with a
+// table is one operation a gate less the uncontrolled X, and the table):
+//   12 X, CNOT, Toffoli      2^19: 13 / 14   13 / 13   12 / 14   2^24: 104 / 104
+//   24 of them               2^20: 26 / 22   25 / 18   30 / 25   2^24: 211 / 112
+//   24 additions and swaps   2^19: 32 / 24   30 / 20   42 / 32   2^24: 514 / 173
+//   12 with four phases      2^21: 36 / 50   36 / 37   53 / 50   2^24: 210 / 237
+//   24 with eight phases     2^20: 33 / 34   32 / 31   45 / 37
+//                            2^21: 51 / 56   51 / 41   75 / 60
+//                            2^22: 90 / 85   90 / 68  139 / 97   2^24: 305 / 265
+// (4096 branches, 20 qubits: 316 us a circuit on planes, 290 branch by branch.)
+bool planes_pay(const OpList& L, uint64_t slots, uint32_t key_bits) {
+  constexpr uint32_t kFew = 12, kTable = 4;
+  if (L.n < kFew || slots < (1ull << 19)) return false;
+  uint32_t tables = 0;
+  for (uint32_t i = 0; i < L.n; ++i) tables += L.op[i].kind == sqs::OP_TABLE;
+  if (!tables) return true;
+  const bool wide_word = key_bits > 32 && key_bits <= 64;
+  return L.n >= kFew + kTable * tables && slots >= (1ull << (wide_word ? 22 : 20));
+}
 
 // Standalone pass over the current state with the packed list.
 sqs_status run_list(sqs_state* st, const OpList& L) {
@@ -676,7 +695,7 @@ sqs_status run_list(sqs_state* st, const OpList& L) {
     st->cur_slot = out_slot;
   } else if (L.touches_keys || L.touches_amps) {
     Traced tr(st, SQS_K_APPLY);
-    if (L.n >= kPlaneMin && in_slots >= kPlaneSlots &&
+    if (planes_pay(L, in_slots, st->total_bits) &&
         sqs::plane_list(L, st->total_bits, st->planes))
       e = sqs::launch_apply_planes(launch_of(st, in_slots), st->kw, st->amp32, st->ctl,
                                    st->cur.view(), st->cur_slot, st->planes);

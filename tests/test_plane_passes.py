@@ -1,17 +1,18 @@
-"""Long queued runs on states large enough for the pass on bit planes (2^19 slots),
-dense and after a merge (segments part full), against the same gates flushed three at a
-time, which takes the pass branch by branch: keys bit for bit, amplitudes to the
-roundings of the folded factors.  The kernels that ran are read from the profiler."""
+"""Long queued runs on states large enough for the pass on bit planes (2^19 slots; with
+factors 2^20, or 2^22 for a key word of more than 32 bits), dense and after a merge
+(segments part full), against the same gates flushed three at a time, which takes the
+pass branch by branch: keys bit for bit, amplitudes to the roundings of the folded
+factors.  The kernels that ran are read from the profiler."""
 import numpy as np
 import pytest
 
 import oracle
 from paper_2503_15118_gb300 import workloads as W
-from tests.helpers import compare_states
 
 pytestmark = pytest.mark.gpu
 
-KINDS = ("x", "cx", "ccx", "phase", "cphase", "add", "sub", "swap")
+KINDS = ("x", "cx", "ccx", "add", "sub", "swap")
+FACTORS = KINDS + ("phase", "cphase")
 
 
 @pytest.fixture(scope="module")
@@ -24,11 +25,11 @@ def sqs():
     return S
 
 
-def _gates(rng, widths, n):
+def _gates(rng, widths, n, factors):
     qs = [(r, b) for r, w in enumerate(widths) for b in range(w)]
     out = []
     for _ in range(n):
-        g = W._draw_gate(rng, KINDS, qs, widths, 0)
+        g = W._draw_gate(rng, FACTORS if factors else KINDS, qs, widths, 0)
         if rng.random() < 0.3 and g[0] in ("add", "sub", "swap"):
             used = {g[1], g[2]}
             free = [q for q in qs if q[0] not in used]
@@ -36,7 +37,7 @@ def _gates(rng, widths, n):
                 c = tuple(free[i] + (int(rng.integers(2)),)
                           for i in rng.choice(len(free), size=min(3, len(free)), replace=False))
                 g = g[:-1] + (c,)
-        if rng.random() < 0.1:  # a predicate over most of the key
+        if factors and rng.random() < 0.1:  # a predicate over most of the key
             some = [q + (int(rng.integers(2)),) for q in qs[:: int(rng.integers(2, 5))]]
             g = ("phase", tuple(some), 0.31)
         out.append(g)
@@ -54,7 +55,7 @@ def _kernels(f):
     return names or None
 
 
-def _pass(sqs, widths, amp32, state, gates, every, segmented):
+def _pass(sqs, widths, amp32, state, gates, every, segmented, on_planes=True):
     st = sqs.State(widths, amp32=amp32, merge=sqs.MERGE_HASH | sqs.FUSE_OFF)
     st.import_(*state)
     if segmented:
@@ -72,7 +73,7 @@ def _pass(sqs, widths, amp32, state, gates, every, segmented):
     if names is not None:
         planes = any("k_apply_planes" in n for n in names)
         singly = any("k_apply_inplace" in n for n in names)
-        assert (singly and not planes) if every else planes, names
+        assert planes if on_planes and not every else singly and not planes, names
     return st
 
 
@@ -87,29 +88,65 @@ def _compare(one, three, amp32, n_factors):
     return l1, h1, a1
 
 
+def _fp32(state, amp32):
+    return state[:2] + (state[2].astype(np.complex64).astype(np.complex128),) if amp32 else state
+
+
 @pytest.mark.parametrize("amp32", [False, True])
 @pytest.mark.parametrize("widths", [[9, 14, 9], [16, 16, 16, 16], [31, 33, 31, 33],
                                     [64, 13, 13, 20]])
-@pytest.mark.parametrize("extra,length", [(0, 12), (1, 90), (4095, 40), (4097 + 31, 90)])
+@pytest.mark.parametrize("extra,length", [(0, 12), (1, 90), (4095, 40), (4097 + 31, 150)])
 def test_dense_states(sqs, widths, amp32, extra, length):
     """Whole tiles of 4096, one branch over, one short of a tile; a run of the
-    fewest operations that goes to planes, and runs with more predicate bits or
-    factors than the smaller list takes."""
+    fewest operations that goes to planes, and runs of more than a launch."""
     rng = np.random.default_rng(sum(widths) + extra)
-    if length == 12:  # exactly so many operations after packing: controlled X and one phase
+    if length == 12:  # exactly so many operations after packing: controlled X
         qs = [(r, b) for r, w in enumerate(widths) for b in range(w)]
-        gates = []
-        for i in range(13):
-            (r, b), c = qs[int(rng.integers(1, len(qs)))], qs[0] + (i & 1,)
-            gates.append(("x", r, b, (c,)))
+        gates = [("x",) + qs[int(rng.integers(1, len(qs)))] + ((qs[0] + (i & 1,),),)
+                 for i in range(12)]
     else:
-        gates = _gates(rng, widths, length)
-    state = W.random_state(widths, (1 << 19) + extra, seed=extra)
-    if amp32:
-        state = state[:2] + (state[2].astype(np.complex64).astype(np.complex128),)
+        gates = _gates(rng, widths, length, False)
+    state = _fp32(W.random_state(widths, (1 << 19) + extra, seed=extra), amp32)
     one = _pass(sqs, widths, amp32, state, gates, 0, False)
     three = _pass(sqs, widths, amp32, state, gates, 3, False)
-    _compare(one, three, amp32, length)
+    _compare(one, three, amp32, 0)
+
+
+@pytest.mark.parametrize("amp32", [False, True])
+@pytest.mark.parametrize("widths,size", [([9, 14, 9], 20), ([31, 33, 31, 33], 20),
+                                         ([64, 13, 13, 20], 20), ([16, 16, 16, 16], 22)])
+@pytest.mark.parametrize("length", [40, 90])
+def test_factors(sqs, widths, size, amp32, length):
+    """Phases among the operations: more predicate bits or factors than the smaller
+    list takes, indices of a few bits and of all ten."""
+    gates = _gates(np.random.default_rng(sum(widths)), widths, length, True)
+    n = (1 << size) + 33
+    i = np.arange(n, dtype=np.uint64)
+    lo = i * np.uint64(0x9E3779B97F4A7C15)  # odd: distinct below 2^22 in the low 32 bits too
+    hi = i >> np.uint64(2) if sum(widths) > 64 else np.zeros(n, np.uint64)
+    if sum(widths) < 64:
+        lo &= np.uint64((1 << sum(widths)) - 1)
+    elif sum(widths) < 128:
+        hi &= np.uint64((1 << (sum(widths) - 64)) - 1)
+    rng = np.random.default_rng(length)
+    a = rng.standard_normal(n) + 1j * rng.standard_normal(n)
+    state = _fp32((lo, hi, a), amp32)
+    one = _pass(sqs, widths, amp32, state, gates, 0, False)
+    three = _pass(sqs, widths, amp32, state, gates, 3, False)
+    _compare(one, three, amp32, len(gates))
+
+
+@pytest.mark.parametrize("n,length,phases", [(1 << 19, 30, 2), (1 << 20, 14, 2), ((1 << 19) - 1, 30, 0),
+                                             (1 << 20, 11, 0)])
+def test_lists_that_stay_branch_by_branch(sqs, n, length, phases):
+    """Too few slots or operations for planes: with a factor table the line is higher."""
+    widths = [20, 16]
+    gates = [("x", 1, i % 16, ((0, i % 20, i & 1),)) for i in range(length - phases)]
+    gates += [("phase", ((1, i, 1),), 0.3) for i in range(phases)]
+    state = W.random_state(widths, n, seed=1)
+    one = _pass(sqs, widths, False, state, gates, 0, False, on_planes=False)
+    three = _pass(sqs, widths, False, state, gates, 3, False)
+    _compare(one, three, False, phases)
 
 
 @pytest.mark.parametrize("amp32", [False, True])
@@ -117,12 +154,10 @@ def test_dense_states(sqs, widths, amp32, extra, length):
 def test_segmented_states(sqs, widths, amp32):
     """After a merge every segment holds a number of branches of its own.  (The
     storage order after a merge is not fixed; the sorted exports are compared.)"""
-    rng = np.random.default_rng(4)
-    gates = _gates(rng, widths, 70)
-    state = W.random_state(widths, (1 << 18) + 77, seed=6, pair_fraction=0.4,
-                           target=(len(widths) - 1, 1))
-    if amp32:
-        state = state[:2] + (state[2].astype(np.complex64).astype(np.complex128),)
+    factors = sum(widths) > 64
+    gates = _gates(np.random.default_rng(4), widths, 70, factors)
+    state = _fp32(W.random_state(widths, (1 << 18) + 77, seed=6, pair_fraction=0.4,
+                                 target=(len(widths) - 1, 1)), amp32)
     one = _pass(sqs, widths, amp32, state, gates, 0, True)
     three = _pass(sqs, widths, amp32, state, gates, 3, True)
     _compare(one, three, amp32, len(gates))
@@ -130,8 +165,8 @@ def test_segmented_states(sqs, widths, amp32):
 
 def test_against_the_oracle(sqs):
     widths = [20, 32, 32]
-    gates = _gates(np.random.default_rng(2), widths, 40)
-    state = W.random_state(widths, (1 << 19) + 1003, seed=8)
+    gates = _gates(np.random.default_rng(2), widths, 30, True)
+    state = W.random_state(widths, (1 << 20) + 1003, seed=8)
     got = _pass(sqs, widths, False, state, gates, 0, False).export()
     o = oracle.OracleState(widths, 1e-14)
     o.import_(*state)
