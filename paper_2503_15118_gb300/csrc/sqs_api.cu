@@ -902,12 +902,16 @@ sqs_status run_hashed(sqs_state* st, const Gate1& g, double est_in, int64_t rec_
   }
   st->stats.steps_hash++;
   if (est_in < 0 && want <= sqs::merge_small_max()) {
-    // About 512 branches a CTA while the cluster can grow (16 CTAs at most).
+    // About 512 branches a CTA while the cluster can grow (16 CTAs at most), at
+    // most 1024.  Where the buffers stay as they are, no more segments than the
+    // other buffer takes as well: what follows may write as many into it.
+    const bool fixed = !st->graphs.empty() || st->capturing;
+    const uint64_t room = std::min(st->alt.cap, st->cur.cap) >> kSegLog2;
     uint32_t ctas = 1;
     while (ctas < 16 && (uint64_t)ctas * (kBucketFill / 2) < want) ctas *= 2;
+    while (fixed && ctas > room && (uint64_t)(ctas / 2) * kBucketFill >= want) ctas /= 2;
     const uint64_t slots = (uint64_t)ctas << kSegLog2;
-    const bool fixed = !st->graphs.empty() || st->capturing;  // buffers stay where they are
-    if (st->alt.cap >= slots || (!fixed && ensure_store(st, st->alt, slots))) {
+    if (fixed ? ctas <= room : st->alt.cap >= slots || ensure_store(st, st->alt, slots)) {
       st->alt.set_segments(kSegLog2, ctas);
       const int out_slot = (st->cur_slot + 1) & 3;
       cudaError_t e;

@@ -1,5 +1,6 @@
 """What a graph capture reserves, and for how long: the buffers a live graph holds stay
 where they are, and once every graph is destroyed the state is as free as before."""
+import numpy as np
 import pytest
 
 from paper_2503_15118_gb300 import workloads as W
@@ -108,4 +109,31 @@ def test_capture_without_room_for_slots(sqs, monkeypatch, amp32):
     for _ in range(2):
         graph.launch()
         assert st.to_dict() == want
+    graph.close()
+
+
+@pytest.mark.parametrize("before", [0, 1, 2])
+@pytest.mark.parametrize("after", ["prune", "diag"])
+def test_a_small_merge_leaves_room_for_what_follows(sqs, before, after):
+    """A state whose two buffers differ in size (an import grows the one it fills): what
+    follows the merge of a captured circuit writes as many segments as the merge into
+    the other buffer."""
+    widths = [13, 3]
+    gates = [("h", 0, b, ()) for b in range(13)] + [("phase", ((0, 5, 1),), 0.4)]
+    gates += [("prune", 1e-14)] * before + [("ry", 0, 5, 0.3, ()), ("x", 1, 0, ((0, 2, 1),))]
+    gates += [("prune", 1e-14)] if after == "prune" else \
+        [("u1q", 0, 1, [[0.6 + 0.8j, 0], [0, 1j]], ())]
+    circ = {"widths": widths, "eps": 1e-14, "tables": [], "gates": gates}
+    want = _state(sqs, widths).run(circ).to_dict()
+    st = _state(sqs, widths)
+    st.import_(np.arange(50000, dtype=np.uint64), None, np.full(50000, 50000.0 ** -0.5, complex))
+    graph = st.capture(circ, 1 << 13)
+    for _ in range(2):
+        graph.launch()
+        assert st.to_dict() == want
+    st.reset()
+    st.run(circ)             # eager again: the graph's buffers stay where they are
+    assert st.to_dict() == want
+    graph.launch()
+    assert st.to_dict() == want
     graph.close()
